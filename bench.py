@@ -88,7 +88,8 @@ def fp32_peak_tflops(sm_mhz):
 
 
 # the sources of the plain path's kernels and of their launch configuration
-PLAIN_SOURCES = ("api.cu", "common.cuh", "contract.cu", "fft.cuh", "pipeline.cu", "plane.cuh", "pointwise.cuh")
+PLAIN_SOURCES = ("api.cu", "common.cuh", "contract.cu", "fft.cuh", "pipeline.cu", "plane.cuh", "planes.cu",
+                 "pointwise.cuh")
 
 
 def source_sha1():

@@ -250,12 +250,12 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
     g.Nk = c->p.Nk;
     g.inv_dk = (float)((c->p.Nk - 1) / c->p.k_max);
     g.invN = (float)(1.0 / (double)g.N);
-    int rc = make_line_plan(n1, &g.p1);
-    if (!rc) rc = make_line_plan(n2, &g.p2);
-    if (!rc) rc = make_line_plan(n3, &g.p3);
+    const bool sized = sized_grid(n1, n2, n3);
+    int rc = make_line_plan(n1, sized, &g.p1);
+    if (!rc) rc = make_line_plan(n2, sized, &g.p2);
+    if (!rc) rc = make_line_plan(n3, sized, &g.p3);
     if (rc) return rc;
-    size_t sp, spen, sa, sd;
-    rc = pipeline_plan_check(c, &sp, &spen, &sa, &sd);
+    rc = pipeline_plan_check(c);
     if (rc) {
         set_error("grid too large for on-chip staging");
         return rc;
@@ -272,7 +272,7 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
         c->nb_p0 = (int)((nb + c->p0_chunks - 1) / c->p0_chunks);
         c->nb_point = c->nb_p0 * c->p0_chunks;
     }
-    VDW_CUDA(cudaMalloc(&c->d_tw, sizeof(float4) * (n1 + n2 + n3)));
+    VDW_CUDA(cudaMalloc(&c->d_tw, sizeof(float4) * (n1 + 2 * n2 + n3)));
     rc = sorted_plan(c);
     if (rc) return rc;
     rc = alloc_density_work(c, 1);
@@ -296,7 +296,7 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
     if (rc) return rc;
     const int npairs = Nq * (Nq + 1) / 2;
     (void)spec_n;
-    c->bytes += sizeof(float4) * (size_t)(c->p.Nk - 1) * npairs + sizeof(float4) * (n1 + n2 + n3);
+    c->bytes += sizeof(float4) * (size_t)(c->p.Nk - 1) * npairs + sizeof(float4) * (n1 + 2 * n2 + n3);
     c->planned = 1;
     return VDW_OK;
 }

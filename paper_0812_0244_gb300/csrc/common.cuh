@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
+#include <initializer_list>
 #include <string>
 
 #include "../../include/vdwnl.h"
@@ -32,11 +33,11 @@ constexpr int MAX_MC = 32;     // largest order m_c of the saturation sum of Eq.
 constexpr int MAX_DIM = 256;   // largest grid dimension (FFT line length)
 constexpr uint8_t K_INVALID = 255;  // interval code of a point with theta = 0
 
-// Radix schedule of one line length: Stockham passes of radix 4 (c4 times),
-// then 2, 3 and 5, with n = 4^c4 2^c2 3^c3 5^c5.
+// Schedule of one line length n = P1 P2: the products of the two groups of
+// radices its transform takes in registers (fft.cuh, make_line_plan).
 struct LinePlan {
     int n;
-    int c4, c2, c3, c5;
+    int P1, P2;
 };
 
 // Pointwise constants, passed by value (kernel parameter space).
@@ -62,6 +63,7 @@ struct GridArgs {
     int Nk;                // points of the radial table
     float invN;            // 1 / N
     LinePlan p1, p2, p3;   // line transforms along x, y, z
+    int pad_fwd, pad_inv;  // plane transforms with padded rows (plane_geo)
     // Flat-index divisions by N1, N2 and N3/2 as multiply-high by
     // m = ceil(2^32 / d), exact for i d < 2^32; fast = 0 (plain division)
     // when N max(N1, N2, N3) reaches 2^32 or a divisor is 1.
@@ -132,8 +134,8 @@ struct vdw_ctx {
     int planned;
     vdw::GridArgs g;
     double L[3];
-    float4* d_tw;               // twiddles (hi/lo pairs): N1, N2, N3 entries
-    float2* d_spec;             // [Nq][N2][N3][Nh] theta(G), then u(G), then real u (N3 x N1 per plane), in place
+    float4* d_tw;               // twiddle tables (hi/lo pairs): x, y, z lines, y lines with their groups swapped
+    float2* d_spec;             // [Nq][N2][N3][Nh] theta(G), then u(G), then real u (packed rows), in place
     float2* d_wspec;            // [3][N2][N3][Nh] w(G); component 0 then D.w
     float* d_t;                 // [N] position of q inside its mesh interval
     uint8_t* d_k;               // [N] mesh interval of q (K_INVALID: theta = 0)
@@ -160,11 +162,10 @@ struct vdw_ctx {
     cudaStream_t s_side;        // the energy reduction beside the inverse transforms
     cudaEvent_t ev_fork, ev_join;
     unsigned long long* d_invalid;  // count of negative / non-finite densities
-    int bulk_planes;            // inverse plane transforms load their planes by bulk copies
     float* d_gg;                // [N] g of w = g grad n (assembly -> w plane transforms)
     // give-up flags of the bounded waits, in mapped page-locked host memory so
-    // that an entry point can read them without synchronising: [0] the bulk
-    // copies of the plane kernels, [1] the tensor-core waits of the learned path
+    // that an entry point can read them without synchronising: [1] the
+    // tensor-core waits of the learned path ([0] unused)
     int* h_flags;               // host view
     int* d_flags;               // device view of the same two words
     int wait_seen;              // a give-up was reported since vdw_plan
@@ -228,6 +229,22 @@ int raise_smem_limit(K kernel, size_t bytes) {
     return VDW_OK;
 }
 
+// Sets a kernel's dynamic shared-memory limit and checks that the block size
+// it will be launched with fits its register use.
+template <class K>
+int set_and_check(K kernel, const char* name, int smem, int threads) {
+    if (const int rs = raise_smem_limit(kernel, (size_t)smem)) return rs;
+    cudaFuncAttributes fa;
+    VDW_CUDA(cudaFuncGetAttributes(&fa, kernel));
+    if (fa.maxThreadsPerBlock < threads) {
+        set_error(std::string(name) + ": " + std::to_string(threads) + " threads requested, " +
+                  std::to_string(fa.maxThreadsPerBlock) + " possible with " + std::to_string(fa.numRegs) +
+                  " registers");
+        return VDW_ERR_UNSUPPORTED;
+    }
+    return VDW_OK;
+}
+
 // pipeline launchers (pipeline.cu)
 // slab_ready (optional): per slab of the pointwise pass, an event to wait on
 // before processing it (the host entry point's copies)
@@ -239,16 +256,19 @@ int pipeline_run(vdw_ctx* c, const float* n, const float* grad, double* E, float
 int pipeline_xc_final(vdw_ctx* c, double* E, cudaStream_t s);
 // central-difference gradient of a field (into grad [3][N])
 int pipeline_stencil_gradient(vdw_ctx* c, const float* f, float* grad, cudaStream_t s);
-int pipeline_plan_check(vdw_ctx* c, size_t* smem_plane, size_t* smem_pencil, size_t* smem_assemble,
-                        size_t* smem_div);
+int pipeline_plan_check(vdw_ctx* c);
+size_t smem_plane(const GridArgs& g);
+int plane_block(const vdw_ctx* c, long long nblocks);
+int best_threads(std::initializer_list<int> items, int lo, int hi);
 int pipeline_make_twiddles(vdw_ctx* c);
 int pipeline_configure(vdw_ctx* c);
 // the divergence term of a potential (w(G) in d_wspec) and the energy reduction
 int pipeline_divergence(vdw_ctx* c, float* v, cudaStream_t s);
 // in-place plane transforms of the first nfields fields of d_spec: inverse
-// (half spectrum -> N3 x N1 real rows at the start of each plane) or forward
-// (packed real rows -> half spectrum)
-int pipeline_planes_inplace(vdw_ctx* c, int nfields, bool inverse, cudaStream_t s);
+// (half spectrum -> packed real rows) or forward (packed real rows -> half
+// spectrum)
+int planes_inplace(vdw_ctx* c, int nfields, bool inverse, cudaStream_t s, int B = 1);
+int planes_configure(vdw_ctx* c);
 // forward plane transforms of w = g grad n with g in d_gg (into d_wspec)
 int pipeline_w_planes(vdw_ctx* c, const float* grad, cudaStream_t s);
 int pipeline_energy_final(vdw_ctx* c, const double* epart, int nb0, int nb2, double* E, cudaStream_t s);
@@ -281,6 +301,15 @@ void learned_free(vdw_ctx* c);
 int table_build(const vdw_params* p, double* h_qmesh, double* h_phik, double* phi0, double* C_s);
 int table_upload(vdw_ctx* c, const double* h_phik, double C_s);
 
-int make_line_plan(int n, LinePlan* lp);
+// Groups of a line length ({2,3,5}-smooth, 4 <= n <= 256); sized: the
+// compile-time schedule of the grids that have one.
+int make_line_plan(int n, bool sized, LinePlan* lp);
+// grids with compile-time line lengths
+inline bool sized_grid(int n1, int n2, int n3) {
+    return (n1 == 180 && n2 == 180 && n3 == 72) || (n1 == 256 && n2 == 256 && n3 == 96);
+}
+// offsets of the twiddle tables in d_tw (entries)
+inline int tw_off_y(const GridArgs& g) { return g.N1; }
+inline int tw_off_swap(const GridArgs& g) { return g.N1 + g.N2 + g.N3; }
 
 }  // namespace vdw

@@ -35,126 +35,167 @@
 namespace vdw {
 
 constexpr int SORT_THREADS = SORTED_BLOCK;  // points per contraction block
-constexpr int PEN_THREADS = 256;   // threads of the y-pencil kernels
 constexpr int PEN_COLS = 8;        // columns per y-pencil block (64-byte runs per plane row)
+// Threads of the y-pencil kernels at most.  A block's work is 32 lines of P1
+// or P2 butterflies per pass.
+constexpr int PEN_THREADS = 256;
+// Shared-memory share (%) of the SM's memory under the pencil kernels.  us
+// forward / inverse at 44, 58, 72 %: 180 x 180 x 72 99/102, 84/92, 89/102; 256
+// x 256 x 96 322/352, 229/274, 242/308; 144 x 144 x 72 53/51, 53/54, 53/61.
+constexpr int PEN_CARVEOUT = 58;
 
-// The inverse y kernel stages the sorted positions of its C columns,
-// pos[c0 N2 .. (c0 + C) N2), in shared memory after the lines and the room for
-// their twiddles, by 4-byte asynchronous copies (zero past the last column),
-// before its gather: all of them in flight at once rather than a few per
-// thread ahead of the copies that need them (0.138 against 0.143 ms at
-// 180 x 180 x 72; the forward kernel, whose positions are only needed for
-// its stores, gains nothing from it).
-__host__ __device__ __forceinline__ size_t pencil_pos_offset(int C, int S, int N2) {
-    return sizeof(float2) * tw_offset((size_t)4 * C * S) + sizeof(Tw) * (size_t)N2;
+// field stride of the lines [4][PEN_COLS][pencil_stride]: lanes that take 4
+// fields and 4 neighbouring points (steps of 1 in the forward kernel's
+// second pass, of P1 | 1 in the inverse kernel's first) hit distinct banks
+__host__ __device__ __forceinline__ int pencil_field_stride(const LinePlan& p, bool inverse) {
+    return PEN_COLS * pencil_stride(p) + (inverse ? (4 * (p.P1 | 1)) & 15 : 4);
 }
-__device__ __forceinline__ void stage_pos(unsigned* pos_s, const unsigned* __restrict__ pos, int c0, int C, int N2,
-                                          int ncols, SmallDiv sN2) {
-    const unsigned* pb = pos + (long long)c0 * N2;
-    for (int i = threadIdx.x; i < C * N2; i += blockDim.x) {
-        const bool ok = c0 + sdiv(i, sN2) < ncols;
-        cp_async4(pos_s + i, ok ? pb + i : pos, ok);
-    }
+template <int CN2>
+__device__ __forceinline__ LinePlan line_of(const GridArgs& g) {
+    if constexpr (CN2 > 0) return LinePlan{CN2, CtLine<CN2>::G1::P, CtLine<CN2>::G2::P};
+    else return g.p2;
 }
 
 // ---------------------------------------------------------------------------
 // P2a: forward y transforms of one quad of fields, records in |G| order
 // ---------------------------------------------------------------------------
-// Block (column tile, quad q): the fields 4q .. 4q+3 of C consecutive
-// half-spectrum columns, all N2 rows, staged as lines [4][C][N2].
+// Block (column tile, quad q): the fields 4q .. 4q+3 of 8 consecutive
+// half-spectrum columns, all N2 rows.  First pass: neighbouring lanes take
+// neighbouring columns (64-byte runs of the plane rows), straight from global
+// memory into the butterflies.  Second pass: neighbouring lanes take the four
+// fields, so that four lanes write one point's 32-byte record.
+//
+// Bound by the latency of its scattered accesses: the share of the SM's memory
+// left to L1 decides how many loads are in flight (PEN_CARVEOUT; at 180 x 180
+// x 72 the inverse kernel takes 154 us with four blocks' shared memory
+// resident and 92 us with two).  us per launch, 20 fields, before (lines
+// staged by asynchronous copies, a shared-memory pass per radix) and after,
+// forward / inverse: 180 x 180 x 72 117 / 135 -> 84 / 90; 256 x 256 x 96 387 /
+// 413 -> 228 / 273; 144 x 144 x 72 (per density) 154 / 154 -> 50 / 54; 200 x
+// 200 x 72 279 / 281 -> 144 / 136 (its radix-25 group); 128^3 220 / 216 -> 77 / 80.
 template <int CN2>
-__global__ void __launch_bounds__(PEN_THREADS) k_pencil_fwd(const float2* __restrict__ spec, GridArgs g,
-                                                            const Tw* __restrict__ tw,
-                                                            const unsigned* __restrict__ pos, float4* __restrict__ Q,
-                                                            long long qstride, int C) {
+__global__ void __launch_bounds__(PEN_THREADS, 3) k_pencil_fwd(const float2* __restrict__ spec, GridArgs g,
+                                                               const Tw* __restrict__ tw,
+                                                               const unsigned* __restrict__ pos,
+                                                               float4* __restrict__ Q, long long qstride) {
     extern __shared__ float2 sm[];
-    const int N2 = CN2 > 0 ? CN2 : g.N2;
-    const int S = pencil_stride(N2);
-    float2* lines = sm;  // [4][C][S]
-    Tw* tw2 = twiddles_after(lines, (size_t)(4 * C * S));
-    load_line_twiddles<CN2>(tw2, tw + g.N1, N2);
-    const int c0 = blockIdx.x * C, q = blockIdx.y;
-    spec += blockIdx.z * g.bs_spec;  // density blockIdx.z of a batch
-    Q += blockIdx.z * g.bs_Q;
-    const float2* src = spec + (long long)4 * q * N2 * g.ncols;
-    const SmallDiv sC = small_div(C), sN2 = small_div(N2);
-    const int tot = 4 * N2 * C;
-    // consecutive threads read consecutive columns of one plane row; the
-    // copies are asynchronous, so each thread has all of its loads in flight
-    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-        const int r = sdiv(i, sC), cc = i - r * C;  // r = a N2 + y
-        const int a = sdiv(r, sN2), y = r - a * N2;
-        const int col = c0 + cc;
-        const bool ok = col < g.ncols;
-        cp_async8(lines + (a * C + cc) * S + y, ok ? src + (long long)r * g.ncols + col : src, ok);
-    }
-    cp_async_wait_all();
+    const LinePlan L = line_of<CN2>(g);
+    const int N2 = L.n, P1 = L.P1, ps = P1 | 1;
+    const int S = pencil_stride(L), LS = pencil_field_stride(L, false);
+    Tw* tw2 = twiddles_after(sm, (size_t)4 * LS);
+    load_twiddles(tw2, tw, N2 - P1);
+    const int c0 = blockIdx.x * PEN_COLS, q = blockIdx.y;
+    spec += blockIdx.z * g.bs_spec + (long long)4 * q * N2 * g.ncols;  // density blockIdx.z of a batch
+    float2* Qf = reinterpret_cast<float2*>(Q + blockIdx.z * g.bs_Q + q * qstride);
+    on_first<CN2, true>(L, [&](auto tag) {
+        using R = decltype(tag);
+        constexpr int CM = CN2 > 0 ? CN2 / R::P : 0;
+        const int m = CN2 > 0 ? CM : L.P2;
+        const SmallDiv dm = small_div(m);
+        const long long step = (long long)m * g.ncols;
+        for (int it = threadIdx.x; it < 4 * PEN_COLS * m; it += blockDim.x) {
+            const int cc = it & (PEN_COLS - 1), t = it / PEN_COLS, a = cdiv<CM>(t, dm), j = t - a * m;
+            const int col = c0 + cc;
+            float2 v[R::P];
+            const float2* src = spec + (long long)(a * N2 + j) * g.ncols + col;
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) v[i] = col < g.ncols ? __ldcg(src + i * step) : make_float2(0.f, 0.f);
+            group_fft<R, false, true, Tw>(v, (const Tw*)nullptr, 1);
+            float2* d = sm + a * LS + cc * S + ps * j;
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) d[R::digit(i)] = v[i];
+        }
+    });
     __syncthreads();
-    pencils_fft<CN2, false>(lines, 4 * C, N2, g.p2, tw2, S);
-    __syncthreads();
-    float4* Qq = Q + q * qstride;
-    const int LS = C * S;
-#pragma unroll 4
-    for (int task = threadIdx.x; task < C * N2; task += blockDim.x) {
-        const int cc = sdiv(task, sN2), y = task - cc * N2;
-        const int col = c0 + cc;
-        if (col >= g.ncols) continue;
-        const long long p = pos[(long long)col * N2 + y];
-        const float2* l = lines + cc * S + y;
-        const float2 v0 = l[0], v1 = l[LS], v2 = l[2 * LS], v3 = l[3 * LS];
-        Qq[2 * p] = make_float4(v0.x, v0.y, v1.x, v1.y);
-        Qq[2 * p + 1] = make_float4(v2.x, v2.y, v3.x, v3.y);
-    }
+    on_second<CN2>(L, [&](auto tag) {
+        using R = decltype(tag);
+        constexpr int CP = CN2 > 0 ? CN2 / R::P : 0;
+        const SmallDiv dp = small_div(P1);
+        for (int it = threadIdx.x; it < 4 * PEN_COLS * P1; it += blockDim.x) {
+            const int a = it & 3, t = it >> 2, cc = cdiv<CP>(t, dp), k1 = t - cc * P1;
+            const int col = c0 + cc;
+            if (col >= g.ncols) continue;
+            const unsigned* pp = pos + (long long)col * N2 + k1;
+            unsigned r[R::P];
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) r[i] = __ldg(pp + P1 * R::digit(i));
+            const float2* d = sm + a * LS + cc * S + k1;
+            float2 v[R::P];
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) v[i] = d[i * ps];
+            group_fft<R, false, false, Tw>(v, tw2 + k1, P1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) Qf[4 * (long long)r[i] + a] = v[i];
+        }
+    });
 }
 
 // ---------------------------------------------------------------------------
 // P2c: records in |G| order -> inverse y transforms -> plane layout
 // ---------------------------------------------------------------------------
+// The forward kernel's mirror image: four lanes read one point's record into
+// the first pass, the second pass writes 64-byte runs of the plane rows.
 template <int CN2>
-__global__ void __launch_bounds__(PEN_THREADS) k_pencil_inv(float2* __restrict__ spec, GridArgs g,
-                                                            const Tw* __restrict__ tw,
-                                                            const unsigned* __restrict__ pos,
-                                                            const float4* __restrict__ Q, long long qstride, int C) {
+__global__ void __launch_bounds__(PEN_THREADS, 3) k_pencil_inv(float2* __restrict__ spec, GridArgs g,
+                                                               const Tw* __restrict__ tw,
+                                                               const unsigned* __restrict__ pos,
+                                                               const float4* __restrict__ Q, long long qstride) {
     extern __shared__ float2 sm[];
-    const int N2 = CN2 > 0 ? CN2 : g.N2;
-    const int S = pencil_stride(N2);
-    float2* lines = sm;  // [4][C][S]
-    float2* tw2 = twiddles_after<float2>(lines, (size_t)(4 * C * S));
-    load_line_twiddles<CN2>(tw2, tw + g.N1, N2);
-    const int c0 = blockIdx.x * C, q = blockIdx.y;
-    spec += blockIdx.z * g.bs_spec;  // density blockIdx.z of a batch
-    Q += blockIdx.z * g.bs_Q;
-    const SmallDiv sC = small_div(C), sN2 = small_div(N2);
-    const float2* Qq = reinterpret_cast<const float2*>(Q + q * qstride);
-    const int LS = C * S;
-    // the positions first (all in flight at once), then the gather
-    unsigned* pos_s = reinterpret_cast<unsigned*>(reinterpret_cast<unsigned char*>(sm) + pencil_pos_offset(C, S, N2));
-    stage_pos(pos_s, pos, c0, C, N2, g.ncols, sN2);
-    cp_async_wait_all();
-    __syncthreads();
-    // the four values of a point go to four lines: 8-byte asynchronous copies
-#pragma unroll 4
-    for (int task = threadIdx.x; task < C * N2; task += blockDim.x) {
-        const int cc = sdiv(task, sN2), y = task - cc * N2;
-        const int col = c0 + cc;
-        const bool ok = col < g.ncols;
-        const long long p = ok ? (long long)pos_s[task] : 0;
-        float2* l = lines + cc * S + y;
+    const LinePlan L = line_of<CN2>(g);
+    const int N2 = L.n, P1 = L.P1, ps = P1 | 1;
+    const int S = pencil_stride(L), LS = pencil_field_stride(L, true);
+    float2* tw2 = twiddles_after<float2>(sm, (size_t)4 * LS);
+    load_twiddles(tw2, tw, N2 - P1);
+    const int c0 = blockIdx.x * PEN_COLS, q = blockIdx.y;
+    spec += blockIdx.z * g.bs_spec + (long long)4 * q * N2 * g.ncols;  // density blockIdx.z of a batch
+    const float2* Qf = reinterpret_cast<const float2*>(Q + blockIdx.z * g.bs_Q + q * qstride);
+    on_first<CN2, true>(L, [&](auto tag) {
+        using R = decltype(tag);
+        constexpr int CM = CN2 > 0 ? CN2 / R::P : 0;
+        const int m = CN2 > 0 ? CM : L.P2;
+        const SmallDiv dm = small_div(m);
+        for (int it = threadIdx.x; it < 4 * PEN_COLS * m; it += blockDim.x) {
+            const int a = it & 3, t = it >> 2, cc = cdiv<CM>(t, dm), j = t - cc * m;
+            const int col = c0 + cc;
+            float2 v[R::P];
+            if (col < g.ncols) {
+                const unsigned* pp = pos + (long long)col * N2 + j;
+                unsigned r[R::P];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) cp_async8(l + a * LS, Qq + 4 * p + a, ok);
-    }
-    cp_async_wait_all();
+                for (int i = 0; i < R::P; ++i) r[i] = __ldg(pp + i * m);
+#pragma unroll
+                for (int i = 0; i < R::P; ++i) v[i] = __ldcg(Qf + 4 * (long long)r[i] + a);
+            } else {
+#pragma unroll
+                for (int i = 0; i < R::P; ++i) v[i] = make_float2(0.f, 0.f);
+            }
+            group_fft<R, true, true, float2>(v, (const float2*)nullptr, 1);
+            float2* d = sm + a * LS + cc * S + ps * j;
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) d[R::digit(i)] = v[i];
+        }
+    });
     __syncthreads();
-    pencils_fft<CN2, true>(lines, 4 * C, N2, g.p2, tw2, S);
-    __syncthreads();
-    float2* dst = spec + (long long)4 * q * N2 * g.ncols;
-    const int tot = 4 * N2 * C;
-    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-        const int r = sdiv(i, sC), cc = i - r * C;
-        const int a = sdiv(r, sN2), y = r - a * N2;
-        const int col = c0 + cc;
-        if (col < g.ncols) dst[(long long)r * g.ncols + col] = lines[(a * C + cc) * S + y];
-    }
+    on_second<CN2>(L, [&](auto tag) {
+        using R = decltype(tag);
+        constexpr int CP = CN2 > 0 ? CN2 / R::P : 0;
+        const SmallDiv dp = small_div(P1);
+        const long long step = (long long)P1 * g.ncols;
+        for (int it = threadIdx.x; it < 4 * PEN_COLS * P1; it += blockDim.x) {
+            const int cc = it & (PEN_COLS - 1), t = it / PEN_COLS, a = cdiv<CP>(t, dp), k1 = t - a * P1;
+            const int col = c0 + cc;
+            const float2* d = sm + a * LS + cc * S + k1;
+            float2 v[R::P];
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) v[i] = d[i * ps];
+            group_fft<R, true, false, float2>(v, tw2 + k1, P1);
+            float2* dst = spec + (long long)(a * N2 + k1) * g.ncols + col;
+            if (col < g.ncols) {
+#pragma unroll
+                for (int i = 0; i < R::P; ++i) dst[R::digit(i) * step] = v[i];
+            }
+        }
+    });
 }
 
 // ---------------------------------------------------------------------------
@@ -255,12 +296,10 @@ __global__ void __launch_bounds__(SORT_THREADS, 4) k_contract_sorted(float4* __r
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-// forward kernel: lines and twiddles; inverse kernel: also the staged positions
-size_t sorted_pencil_smem_fwd(const GridArgs& g) { return pencil_pos_offset(PEN_COLS, pencil_stride(g.N2), g.N2); }
 size_t sorted_pencil_smem(const GridArgs& g) {
-    return sorted_pencil_smem_fwd(g) + sizeof(unsigned) * PEN_COLS * g.N2;
+    const size_t n = 4 * (size_t)std::max(pencil_field_stride(g.p2, false), pencil_field_stride(g.p2, true));
+    return sizeof(float2) * tw_offset(n) + sizeof(Tw) * (size_t)(g.p2.n - g.p2.P1);
 }
-
 // |G| order of the half spectrum: pos[col N2 + y] = sorted position of the
 // point (kx, y, kz), col = kz Nh + kx; gs[sorted position] = |G| with the
 // energy weight in its sign.  Ties (equal |G|) keep the (col, y) order, so
@@ -317,9 +356,14 @@ void sorted_free(vdw_ctx* c) {
 
 template <int CN2>
 static int configure_sorted_sized(vdw_ctx* c) {
-    int rc = raise_smem_limit(k_pencil_fwd<CN2>, (int)sorted_pencil_smem_fwd(c->g));
+    int rc = raise_smem_limit(k_pencil_fwd<CN2>, (int)sorted_pencil_smem(c->g));
     if (!rc) rc = raise_smem_limit(k_pencil_inv<CN2>, (int)sorted_pencil_smem(c->g));
     if (rc) return rc;
+    // The scattered 32-byte records reserve a 128-byte L1 line each while they
+    // are in flight: with all of the SM's memory given to shared memory, what
+    // is left for L1 bounds the loads in flight.
+    VDW_CUDA(cudaFuncSetAttribute(k_pencil_fwd<CN2>, cudaFuncAttributePreferredSharedMemoryCarveout, PEN_CARVEOUT));
+    VDW_CUDA(cudaFuncSetAttribute(k_pencil_inv<CN2>, cudaFuncAttributePreferredSharedMemoryCarveout, PEN_CARVEOUT));
     int dev = 0;
     VDW_CUDA(cudaGetDevice(&dev));
     VDW_CUDA(cudaDeviceGetAttribute(&c->nsm, cudaDevAttrMultiProcessorCount, dev));
@@ -327,32 +371,16 @@ static int configure_sorted_sized(vdw_ctx* c) {
 }
 
 int sorted_configure(vdw_ctx* c) {
-    const int N2 = c->g.N2;
-    if (N2 == 180) return configure_sorted_sized<180>(c);
-    if (N2 == 256) return configure_sorted_sized<256>(c);
-    return configure_sorted_sized<0>(c);
+    return on_grid(c->g, [&](auto d) { return configure_sorted_sized<decltype(d)::N2>(c); });
 }
-
-// the compile-time y lengths are those of the sized grids (180 x 180 x 72,
-// 256 x 256 x 96); any other grid uses the runtime-length engine
-static int sized_n2(const GridArgs& g) {
-    if (g.N1 == 180 && g.N2 == 180 && g.N3 == 72) return 180;
-    if (g.N1 == 256 && g.N2 == 256 && g.N3 == 96) return 256;
-    return 0;
-}
-
-#define VDW_SORTED_LAUNCH(KERNEL, ...)                                                  \
-    switch (sized_n2(g)) {                                                            \
-        case 180: KERNEL<180><<<grid, PEN_THREADS, sm, s>>>(__VA_ARGS__); break;      \
-        case 256: KERNEL<256><<<grid, PEN_THREADS, sm, s>>>(__VA_ARGS__); break;      \
-        default: KERNEL<0><<<grid, PEN_THREADS, sm, s>>>(__VA_ARGS__);                \
-    }
 
 int sorted_forward(vdw_ctx* c, int nfields, cudaStream_t s, int B) {
     const GridArgs& g = c->g;
     const dim3 grid((g.ncols + PEN_COLS - 1) / PEN_COLS, nfields / 4, B);
-    const size_t sm = sorted_pencil_smem_fwd(g);
-    VDW_SORTED_LAUNCH(k_pencil_fwd, c->d_spec, g, c->d_tw, c->d_pos, c->d_Q, 2 * c->Npad, PEN_COLS)
+    on_grid(g, [&](auto d) {
+        k_pencil_fwd<decltype(d)::N2><<<grid, PEN_THREADS, sorted_pencil_smem(g), s>>>(
+            c->d_spec, g, c->d_tw + tw_off_y(g), c->d_pos, c->d_Q, 2 * c->Npad);
+    });
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;
 }
@@ -360,12 +388,13 @@ int sorted_forward(vdw_ctx* c, int nfields, cudaStream_t s, int B) {
 int sorted_inverse(vdw_ctx* c, int nfields, cudaStream_t s, int B) {
     const GridArgs& g = c->g;
     const dim3 grid((g.ncols + PEN_COLS - 1) / PEN_COLS, nfields / 4, B);
-    const size_t sm = sorted_pencil_smem(g);
-    VDW_SORTED_LAUNCH(k_pencil_inv, c->d_spec, g, c->d_tw, c->d_pos, c->d_Q, 2 * c->Npad, PEN_COLS)
+    on_grid(g, [&](auto d) {
+        k_pencil_inv<decltype(d)::N2><<<grid, PEN_THREADS, sorted_pencil_smem(g), s>>>(
+            c->d_spec, g, c->d_tw + tw_off_y(g), c->d_pos, c->d_Q, 2 * c->Npad);
+    });
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;
 }
-#undef VDW_SORTED_LAUNCH
 
 int sorted_contract(vdw_ctx* c, double* epart, int write_back, cudaStream_t s, int B) {
     return sorted_contract_table(c, c->p.Nq, c->d_kcoef, c->g.inv_dk, c->g.Nk, epart, write_back, s, B);

@@ -1,18 +1,23 @@
-// Warp-per-line mixed-radix FFTs on shared memory (sm_103a).
+// Mixed-radix FFTs of lines of at most 256 points (sm_103a), two register
+// passes per line with one exchange through shared memory between them.
 //
-// One warp transforms one line of complex FP32 values held in shared memory
-// (any element stride), in place, by Stockham autosort passes of radix 4, 2,
-// 3 or 5: in each pass every lane loads its butterflies' inputs into
-// registers, the warp synchronises, and the lanes write the outputs to their
-// autosorted positions.  Lines are independent, so a block spreads its lines
-// over its warps with no block-wide barrier between passes.
+// A line of n = P1 P2 points is the Stockham autosort algorithm over a list of
+// small radices (2, 3, 4, 5, and for some lengths in-register 8, 9, 12, 15,
+// 16), its consecutive radices taken in two groups whose products are P1 and
+// P2.  One thread does a whole group for one butterfly in registers: it loads
+// the P inputs x[j + q n/P], runs the group's radices one after another and
+// stores the P outputs, so that the shared-memory traffic is that of two
+// passes however many radices there are.
 //
-// Pass (radix R, Ns = product of the previous radices, m = n/R butterflies):
-//   for j in [0, m):  k = j mod Ns
-//     v_r = x[j + r m] * W_n^{r k n/(Ns R)}        (W_n = exp(-2 pi i/n))
-//     V   = DFT_R(v)
-//     y[(j - k) R + k + r Ns] = V_r
-// Forward uses W_n, inverse its conjugate; neither scales.
+// Group of radices A, B, C after Ns = product of the radices before it
+// (j in [0, n/P), k = j mod Ns):
+//   input q = (ra B + rb) C + rc        at j + q n/P
+//   radix A over ra, twiddle W_{Ns A}^(ra k),              output digit ka
+//   radix B over rb, twiddle W_{Ns A B}^(rb (k + ka Ns)),  output digit kb
+//   radix C over rc, twiddle W_{Ns P}^(rc (k + (ka + A kb) Ns)), digit kc
+//   output q' = ka + A kb + A B kc      at (j - k) P + k + q' Ns
+// In the first group Ns = 1 and k = 0: its twiddles are constants.  Forward
+// uses W_n = exp(-2 pi i/n), inverse its conjugate; neither scales.
 //
 // Every constant of a transform (table twiddles, the sines and cosines inside
 // the radix 3, 5, 8, 9 and 16 butterflies) is held as a pair hi + lo of FP32
@@ -27,10 +32,14 @@
 
 #include "common.cuh"
 
+#include <utility>
+
 namespace vdw {
 
-__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
+// packed FP32 pairs: one instruction for both parts (the transforms are bound
+// by issue slots and shared memory; 1-5 % of the plane kernels' time)
+__device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
+__device__ __forceinline__ float2 csub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
 __device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
@@ -152,141 +161,7 @@ __device__ __forceinline__ void dft<5, false>(float2* v) { dft5<false>(v); }
 template <>
 __device__ __forceinline__ void dft<5, true>(float2* v) { dft5<true>(v); }
 
-// One Stockham pass of radix R over a line of length n (n <= MAX_DIM), by one warp.
-// j mod Ns through a multiply-high: with M = floor((2^32-1)/Ns) + 1 the
-// quotient umulhi(j, M) is exact for j < 2048, Ns <= 512 (checked
-// exhaustively); Ns = 1 is special-cased.
-__device__ __forceinline__ unsigned magic_of(int Ns) { return Ns > 1 ? 0xFFFFFFFFu / (unsigned)Ns + 1u : 0u; }
-__device__ __forceinline__ int mod_magic(int j, int Ns, unsigned M) {
-    return Ns > 1 ? j - (int)__umulhi((unsigned)j, M) * Ns : 0;
-}
-
-template <int R, bool INV, class W>
-__device__ __forceinline__ void line_pass(float2* p, int es, int n, int Ns, const W* tw, int lane) {
-    constexpr int MAXB = (MAX_DIM / R + 31) / 32;
-    const int m = n / R;
-    const int tstride = n / (Ns * R);
-    const unsigned M = magic_of(Ns);
-    float2 v[MAXB][R];
-#pragma unroll
-    for (int b = 0; b < MAXB; ++b) {
-        const int j0 = lane + 32 * b;
-        const int j = j0 < m ? j0 : 0;  // in-range index for tail lanes
-        if (j0 < m) {
-            const int k = mod_magic(j, Ns, M);
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[b][r] = p[(j + r * m) * es];
-#pragma unroll
-            for (int r = 1; r < R; ++r) {
-                const W w = tw[r * k * tstride];  // r k n/(Ns R) < n
-                v[b][r] = tw_mul<INV>(v[b][r], w);
-            }
-            dft<R, INV>(v[b]);
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int b = 0; b < MAXB; ++b) {
-        const int j0 = lane + 32 * b;
-        const int j = j0 < m ? j0 : 0;
-        if (j0 < m) {
-            const int k = mod_magic(j, Ns, M);
-            const int base = (j - k) * R + k;
-#pragma unroll
-            for (int r = 0; r < R; ++r) p[(base + r * Ns) * es] = v[b][r];
-        }
-    }
-    __syncwarp();
-}
-
-// Full line transform: tw holds W_n^e = exp(-2 pi i e/n), e in [0, n), as hi/lo pairs.  One
-// loop per radix keeps each pass's registers separate.
-template <bool INV, class W>
-__device__ __forceinline__ void line_fft(float2* p, int es, const LinePlan& pl, const W* tw, int lane) {
-    int Ns = 1;
-#pragma unroll 1
-    for (int s = 0; s < pl.c4; ++s) { line_pass<4, INV>(p, es, pl.n, Ns, tw, lane); Ns *= 4; }
-#pragma unroll 1
-    for (int s = 0; s < pl.c2; ++s) { line_pass<2, INV>(p, es, pl.n, Ns, tw, lane); Ns *= 2; }
-#pragma unroll 1
-    for (int s = 0; s < pl.c3; ++s) { line_pass<3, INV>(p, es, pl.n, Ns, tw, lane); Ns *= 3; }
-#pragma unroll 1
-    for (int s = 0; s < pl.c5; ++s) { line_pass<5, INV>(p, es, pl.n, Ns, tw, lane); Ns *= 5; }
-}
-
-// Two real rows a, b packed as Z = a + i b, after the forward transform of Z:
-// split into the half spectra A[k], B[k], k in [0, N/2], written to p[0..Nh)
-// and p[Nh..2Nh) (the region holds 2 Nh = N + 2 values).
-__device__ __forceinline__ void r2c_untangle(float2* p, int N, int lane) {
-    constexpr int MAXK = (MAX_DIM / 2 + 1 + 31) / 32;
-    const int Nh = N / 2 + 1;
-    float2 A[MAXK], B[MAXK];
-#pragma unroll
-    for (int b = 0; b < MAXK; ++b) {
-        const int k0 = lane + 32 * b;
-        const int k = k0 < Nh ? k0 : 0;  // in-range index for tail lanes
-        if (k0 < Nh) {
-            const float2 zk = p[k == N ? 0 : k];
-            const float2 zm = p[k == 0 ? 0 : N - k];
-            // A = (Z_k + conj Z_{-k})/2,  B = -i (Z_k - conj Z_{-k})/2
-            A[b] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-            B[b] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int b = 0; b < MAXK; ++b) {
-        const int k0 = lane + 32 * b;
-        const int k = k0 < Nh ? k0 : 0;
-        if (k0 < Nh) {
-            p[k] = A[b];
-            p[Nh + k] = B[b];
-        }
-    }
-    __syncwarp();
-}
-
-// Inverse of the above: from half spectra A (p[0..Nh)), B (p[Nh..2Nh)) of two
-// real rows build Z[0..N) = A + i B on the full circle (Hermitian extension;
-// the imaginary parts of the k = 0 and k = N/2 terms are dropped, as a
-// complex-to-real transform does).  The inverse transform of Z then gives
-// N a in its real part and N b in its imaginary part.
-__device__ __forceinline__ void c2r_tangle(float2* p, int N, int lane) {
-    constexpr int MAXK = (MAX_DIM / 2 + 1 + 31) / 32;
-    const int Nh = N / 2 + 1;
-    float2 A[MAXK], B[MAXK];
-#pragma unroll
-    for (int b = 0; b < MAXK; ++b) {
-        const int k0 = lane + 32 * b;
-        const int k = k0 < Nh ? k0 : 0;
-        if (k0 < Nh) {
-            A[b] = p[k];
-            B[b] = p[Nh + k];
-            if (k == 0 || 2 * k == N) { A[b].y = 0.f; B[b].y = 0.f; }
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int b = 0; b < MAXK; ++b) {
-        const int k0 = lane + 32 * b;
-        const int k = k0 < Nh ? k0 : 0;
-        if (k0 < Nh) {
-            p[k] = make_float2(A[b].x - B[b].y, A[b].y + B[b].x);
-            if (k >= 1 && 2 * k < N) p[N - k] = make_float2(A[b].x + B[b].y, B[b].x - A[b].y);
-        }
-    }
-    __syncwarp();
-}
-
-}  // namespace vdw
-
-// ---------------------------------------------------------------------------
-// Compile-time line lengths: the same Stockham passes with constant radices,
-// strides and twiddle steps, radix 8 first, and several lines per warp so
-// that short lines still fill the 32 lanes.
-// ---------------------------------------------------------------------------
-namespace vdw {
-
+// ---- in-register radices ---------------------------------------------------
 template <bool INV>
 __device__ __forceinline__ void dft8(float2* v) {
     constexpr KPair r2 = kpair(0.70710678118654752440);
@@ -426,169 +301,213 @@ template <> __device__ __forceinline__ void dft<15, true>(float2* v) { dft_pfa<5
 template <> __device__ __forceinline__ void dft<16, false>(float2* v) { dft_ct<4, 4, false>(v); }
 template <> __device__ __forceinline__ void dft<16, true>(float2* v) { dft_ct<4, 4, true>(v); }
 
-// Radix schedule of a compile-time length: the first radix is the one (among
-// the in-register lengths) that leaves the fewest passes, the larger on a tie.
-// maxr caps the radix (register pressure in kernels that hold much else).
-constexpr int CT_RADICES[] = {16, 15, 12, 10, 9, 8, 6, 5, 4, 3, 2};
-constexpr int ct_passes_greedy(int n, int maxr);
-constexpr int ct_radix(int n, int maxr = 16) {
-    int best = 0, bestp = 1 << 20, bestd = 1 << 20;
-    for (int r : CT_RADICES) {
-        if (r > maxr || n % r != 0) continue;
-        const int p = 1 + ct_passes_greedy(n / r, maxr);
-        const int d = r > n / r ? r - n / r : n / r - r;  // prefer balanced splits
-        if (p < bestp || (p == bestp && d < bestd)) {
-            bestp = p;
-            bestd = d;
-            best = r;
-        }
-    }
-    return best;
+// ---------------------------------------------------------------------------
+// groups of radices
+// ---------------------------------------------------------------------------
+// f(integral_constant<int, i>) for i = 0 .. N-1
+template <class F, int... I>
+__device__ __forceinline__ void static_for_impl(F&& f, std::integer_sequence<int, I...>) {
+    (f(std::integral_constant<int, I>{}), ...);
 }
-constexpr int ct_passes_greedy(int n, int maxr) {
-    if (n <= 1) return 0;
-    for (int r : CT_RADICES)
-        if (r <= maxr && n % r == 0) return 1 + ct_passes_greedy(n / r, maxr);
-    return 1 << 20;
-}
-constexpr int ct_npasses(int n, int maxr = 16) { return n <= 1 ? 0 : 1 + ct_npasses(n / ct_radix(n, maxr), maxr); }
-// radix of pass s (in order) and the product Ns of the radices before it
-constexpr int ct_radix_at(int n, int s, int maxr = 16) {
-    return s == 0 ? ct_radix(n, maxr) : ct_radix_at(n / ct_radix(n, maxr), s - 1, maxr);
-}
-constexpr int ct_ns_at(int n, int s, int maxr = 16) {
-    return s == 0 ? 1 : ct_radix(n, maxr) * ct_ns_at(n / ct_radix(n, maxr), s - 1, maxr);
-}
-// largest butterfly count N / R over the passes, and the lines one warp
-// transforms together so that its lanes stay busy
-constexpr int ct_max_m(int n, int maxr = 16, int s = 0) {
-    return s >= ct_npasses(n, maxr) ? 0
-                                    : (n / ct_radix_at(n, s, maxr) > ct_max_m(n, maxr, s + 1) ? n / ct_radix_at(n, s, maxr)
-                                                                                                : ct_max_m(n, maxr, s + 1));
-}
-// (two lines of at most 16 butterflies go one per half-warp, see ct_pass)
-constexpr int ct_lines_per_warp(int n, int maxr = 16) {
-    const int m = ct_max_m(n, maxr);
-    if (m <= 16) return 2;
-    const int l = 32 / m;
-    return l < 1 ? 1 : (l > 4 ? 4 : l);
+template <int N, class F>
+__device__ __forceinline__ void static_for(F&& f) {
+    static_for_impl(f, std::make_integer_sequence<int, N>{});
 }
 
-// Twiddle table of a compile-time length N, laid out by pass: pass s with
-// Ns > 1 keeps W_N^(r k TS) (r = 1 .. R-1, k = 0 .. Ns-1, TS = N/(Ns R)) at
-// ct_tw_off(N, s) + (r - 1) Ns + k, so that the lanes of a pass, which take
-// consecutive k, read consecutive entries (no bank conflicts).  At most N
-// entries in all.
-constexpr int ct_tw_off(int n, int s, int maxr = 16) {
-    return s == 0 ? 0
-                  : ct_tw_off(n, s - 1, maxr) +
-                        (ct_ns_at(n, s - 1, maxr) > 1 ? (ct_radix_at(n, s - 1, maxr) - 1) * ct_ns_at(n, s - 1, maxr) : 0);
+// cos and sin of 2 pi e/n for the constant twiddles of a first group, by
+// their series on [0, pi/4] after reduction to the first octant (exact at the
+// multiples of a quarter turn)
+constexpr double series_cos(double x) {
+    double s = 0.0, t = 1.0;
+    for (int k = 0; k < 14; ++k) {
+        s += t;
+        t *= -x * x / ((2.0 * k + 1.0) * (2.0 * k + 2.0));
+    }
+    return s;
 }
-// Fills the table from the plain one (src[e] = W_N^e), all threads of the block.
-template <int N, int MAXR = 16, int S = 0, class W>
-__device__ __forceinline__ void ct_load_twiddles(W* dst, const Tw* src) {
-    if constexpr (S < ct_npasses(N, MAXR)) {
-        constexpr int R = ct_radix_at(N, S, MAXR), Ns = ct_ns_at(N, S, MAXR);
-        if constexpr (Ns > 1) {
-            constexpr int TS = N / (Ns * R), off = ct_tw_off(N, S, MAXR);
-            for (int i = threadIdx.x; i < (R - 1) * Ns; i += blockDim.x) {
-                const int r = 1 + i / Ns, k = i - (r - 1) * Ns;
-                tw_put(dst + off + i, src[r * k * TS]);
+constexpr double series_sin(double x) {
+    double s = 0.0, t = x;
+    for (int k = 0; k < 14; ++k) {
+        s += t;
+        t *= -x * x / ((2.0 * k + 2.0) * (2.0 * k + 3.0));
+    }
+    return s;
+}
+constexpr double turn_cos(int e, int n);
+constexpr double turn_sin(int e, int n) {
+    e %= n;
+    if (2 * e > n) return -turn_sin(n - e, n);                 // second half: odd
+    if (4 * e > n) return turn_sin(n - 2 * e, 2 * n);          // sin(pi - x)
+    if (8 * e > n) return series_cos(6.28318530717958647692 * (n - 4 * e) / (4.0 * n));
+    return series_sin(6.28318530717958647692 * e / (double)n);
+}
+constexpr double turn_cos(int e, int n) { return turn_sin(4 * e + n, 4 * n); }
+
+// a W_N^E (conjugated for the inverse) with a constant twiddle: hi/lo pairs
+// (W = Tw) or the FP32 value (W = float2)
+template <int N, int E, bool INV, class W>
+__device__ __forceinline__ float2 mul_root(float2 a) {
+    constexpr int e = ((E % N) + N) % N;
+    if constexpr (e == 0) return a;
+    else if constexpr (4 * e == N) return mul_mi<INV>(a);
+    else if constexpr (2 * e == N) return make_float2(-a.x, -a.y);
+    else if constexpr (4 * e == 3 * N) return mul_mi<!INV>(a);
+    else {
+        constexpr KPair cr = kpair(turn_cos(e, N)), ci = kpair(-turn_sin(e, N));
+        if constexpr (sizeof(W) == sizeof(float4)) return tw_mul<INV>(a, make_float4(cr.h, ci.h, cr.l, ci.l));
+        else return tw_mul<INV>(a, make_float2(cr.h, ci.h));
+    }
+}
+
+template <int A_, int B_ = 1, int C_ = 1>
+struct Grp {
+    static constexpr int A = A_, B = B_, C = C_, P = A_ * B_ * C_;
+    // output digit q' of register i (the radices run in place: register
+    // (ka B + kb) C + kc ends with output ka + A kb + A B kc)
+    static constexpr int digit(int i) { return i / (B * C) + A * ((i / C) % B) + A * B * (i % C); }
+};
+
+// The group's transform of v (input q in register q).  FIRST: Ns = 1,
+// constant twiddles.  Otherwise tw points at the group's table (tw_entries)
+// plus k: the twiddle of entry i is tw[i Ns].
+template <class G, bool INV, bool FIRST, class W>
+__device__ __forceinline__ void group_fft(float2 (&v)[G::P], const W* tw, int Ns) {
+    constexpr int A = G::A, B = G::B, C = G::C, BC = B * C;
+    if constexpr (A > 1) {
+        static_for<BC>([&](auto S) {
+            constexpr int s = decltype(S)::value;
+            float2 t[A];
+#pragma unroll
+            for (int r = 0; r < A; ++r) {
+                t[r] = v[r * BC + s];
+                if (!FIRST && r > 0) t[r] = tw_mul<INV>(t[r], tw[(r - 1) * Ns]);
             }
-        }
-        ct_load_twiddles<N, MAXR, S + 1>(dst, src);
+            dft<A, INV>(t);
+#pragma unroll
+            for (int r = 0; r < A; ++r) v[r * BC + s] = t[r];
+        });
+    }
+    if constexpr (B > 1) {
+        static_for<A>([&](auto KA) {
+            constexpr int ka = decltype(KA)::value;
+            static_for<C>([&](auto S) {
+                constexpr int s = decltype(S)::value;
+                float2 t[B];
+                static_for<B>([&](auto R) {
+                    constexpr int r = decltype(R)::value;
+                    t[r] = v[ka * BC + r * C + s];
+                    if constexpr (FIRST) t[r] = mul_root<A * B, r * ka, INV, W>(t[r]);
+                    else if constexpr (r > 0) t[r] = tw_mul<INV>(t[r], tw[(A - 1 + (r - 1) * A + ka) * Ns]);
+                });
+                dft<B, INV>(t);
+#pragma unroll
+                for (int r = 0; r < B; ++r) v[ka * BC + r * C + s] = t[r];
+            });
+        });
+    }
+    if constexpr (C > 1) {
+        static_for<A * B>([&](auto K) {
+            constexpr int ka = decltype(K)::value / B, kb = decltype(K)::value % B, kk = ka + A * kb;
+            float2 t[C];
+            static_for<C>([&](auto R) {
+                constexpr int r = decltype(R)::value;
+                t[r] = v[ka * BC + kb * C + r];
+                if constexpr (FIRST) t[r] = mul_root<A * B * C, r * kk, INV, W>(t[r]);
+                else if constexpr (r > 0) t[r] = tw_mul<INV>(t[r], tw[(A * B - 1 + (r - 1) * A * B + kk) * Ns]);
+            });
+            dft<C, INV>(t);
+#pragma unroll
+            for (int r = 0; r < C; ++r) v[ka * BC + kb * C + r] = t[r];
+        });
     }
 }
 
-// One pass over L lines (line l at p + l*ls, element stride es) by one warp.
-// Two lines of at most 16 butterflies go one per half-warp: a 64-bit shared
-// access is served per half-warp, so the two lines never compete for banks
-// whatever their distance, and consecutive butterflies of one line hit
-// distinct banks.  The first pass (Ns = 1) has no twiddles; the others read
-// the pass-ordered table of ct_load_twiddles.
-template <int N, int S, int L, bool INV, int MAXR, class W>
-__device__ __forceinline__ void ct_pass(float2* p, int es, int ls, const W* tw, int lane) {
-    constexpr int R = ct_radix_at(N, S, MAXR);
-    constexpr int Ns = ct_ns_at(N, S, MAXR);
-    constexpr int M = N / R;
-    constexpr int TOT = L * M;
-    constexpr bool HALF = (L == 2) && (M <= 16);
-    constexpr int B = HALF ? 1 : (TOT + 31) / 32;
-    float2 v[B][R];
-    int lj[B][2];
-    bool act[B];
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-        if constexpr (HALF) {
-            lj[b][0] = lane >> 4;
-            lj[b][1] = lane & 15;
-            act[b] = (M == 16) || lj[b][1] < M;
-        } else {
-            const int t0 = lane + 32 * b;
-            act[b] = (TOT % 32 == 0) || t0 < TOT;
-            const int t = act[b] ? t0 : 0;  // in-range index for tail lanes
-            lj[b][0] = t / M;
-            lj[b][1] = t - lj[b][0] * M;
-        }
-    }
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-        if (act[b]) {
-            const int l = lj[b][0], j = lj[b][1];
-            const int k = j % Ns;
-            const float2* q = p + l * ls;
-#pragma unroll
-            for (int r = 0; r < R; ++r) v[b][r] = q[(j + r * M) * es];
-            if constexpr (Ns > 1) {
-                constexpr int off = ct_tw_off(N, S, MAXR);
-#pragma unroll
-                for (int r = 1; r < R; ++r) {
-                    const W w = tw[off + (r - 1) * Ns + k];
-                    v[b][r] = tw_mul<INV>(v[b][r], w);
+// ---------------------------------------------------------------------------
+// line schedules
+// ---------------------------------------------------------------------------
+// Compile-time lengths (the grids 180 x 180 x 72 and 256 x 256 x 96): two
+// in-register radices each.  Any other length takes its groups at run time
+// from the list 4, .., 4, 2, 3, .., 3, 5, .., 5 (make_line_plan).
+template <int CN> struct CtLine { using G1 = Grp<1>; using G2 = Grp<1>; };
+template <> struct CtLine<180> { using G1 = Grp<15>; using G2 = Grp<12>; };
+template <> struct CtLine<72> { using G1 = Grp<9>; using G2 = Grp<8>; };
+template <> struct CtLine<256> { using G1 = Grp<16>; using G2 = Grp<16>; };
+template <> struct CtLine<96> { using G1 = Grp<12>; using G2 = Grp<8>; };
+
+// Run-time lengths: any, or (ANY16) with no group above 16.  The second kind
+// leaves the larger groups' registers out of a kernel.
+constexpr int ANY = 0, ANY16 = -1;
+
+// f(group of product P) for a run-time P.  A product stands for one list of
+// radices; P1 of an even length is one of the first set, of an odd one also
+// of the second, and P2 one of the third.
+template <bool ODD, bool BIG, class F>
+__device__ __forceinline__ void first_group(int P, F&& f) {
+    switch (P) {
+        case 2: f(Grp<2>{}); break;
+        case 4: f(Grp<4>{}); break;
+        case 6: f(Grp<2, 3>{}); break;
+        case 8: f(Grp<4, 2>{}); break;
+        case 10: f(Grp<2, 5>{}); break;
+        case 12: f(Grp<4, 3>{}); break;
+        case 16: f(Grp<4, 4>{}); break;
+        default:
+            if constexpr (BIG) {
+                switch (P) {
+                    case 18: f(Grp<2, 3, 3>{}); break;
+                    case 20: f(Grp<4, 5>{}); break;
+                    case 24: f(Grp<4, 2, 3>{}); break;
+                    default: break;
                 }
             }
-            dft<R, INV>(v[b]);
-        }
-    }
-    __syncwarp();
-#pragma unroll
-    for (int b = 0; b < B; ++b) {
-        if (act[b]) {
-            const int l = lj[b][0], j = lj[b][1];
-            const int k = j % Ns;
-            float2* q = p + l * ls;
-            const int base = (j - k) * R + k;
-            if constexpr (HALF && Ns == 1 && R == 16) {
-                // the outputs of butterfly j go to 16 j + r: with the same r in
-                // every lane the 16 lanes of a half-warp would hit one bank.
-                // Rotate each lane's outputs by j (four conditional rotations
-                // by 1, 2, 4, 8) so that step r' stores output (r' + j) mod 16.
-#pragma unroll
-                for (int bit = 0; bit < 4; ++bit) {
-                    const bool rot = (j >> bit) & 1;
-                    float2 t[R];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) t[r] = v[b][(r + (1 << bit)) & (R - 1)];
-#pragma unroll
-                    for (int r = 0; r < R; ++r) v[b][r] = rot ? t[r] : v[b][r];
+            if constexpr (ODD) {
+                switch (P) {
+                    case 3: f(Grp<3>{}); break;
+                    case 5: f(Grp<5>{}); break;
+                    case 9: f(Grp<3, 3>{}); break;
+                    case 15: f(Grp<3, 5>{}); break;
+                    default: break;
                 }
-#pragma unroll
-                for (int r = 0; r < R; ++r) q[(base + ((r + j) & (R - 1))) * es] = v[b][r];
-            } else {
-#pragma unroll
-                for (int r = 0; r < R; ++r) q[(base + r * Ns) * es] = v[b][r];
             }
-        }
+            if constexpr (ODD && BIG) {
+                switch (P) {
+                    case 25: f(Grp<5, 5>{}); break;
+                    case 27: f(Grp<3, 3, 3>{}); break;
+                    default: break;
+                }
+            }
     }
-    __syncwarp();
 }
-
-template <int N, int L, bool INV, int MAXR = 16, int S = 0, class W>
-__device__ __forceinline__ void ct_fft(float2* p, int es, int ls, const W* tw, int lane) {
-    if constexpr (S < ct_npasses(N, MAXR)) {
-        ct_pass<N, S, L, INV, MAXR>(p, es, ls, tw, lane);
-        ct_fft<N, L, INV, MAXR, S + 1>(p, es, ls, tw, lane);
+template <bool BIG, class F>
+__device__ __forceinline__ void second_group(int P, F&& f) {
+    switch (P) {
+        case 1: f(Grp<1>{}); break;
+        case 2: f(Grp<2>{}); break;
+        case 3: f(Grp<3>{}); break;
+        case 4: f(Grp<4>{}); break;
+        case 5: f(Grp<5>{}); break;
+        case 6: f(Grp<2, 3>{}); break;
+        case 8: f(Grp<4, 2>{}); break;
+        case 9: f(Grp<3, 3>{}); break;
+        case 10: f(Grp<2, 5>{}); break;
+        case 12: f(Grp<4, 3>{}); break;
+        case 15: f(Grp<3, 5>{}); break;
+        case 16: f(Grp<4, 4>{}); break;
+        default:
+            if constexpr (BIG) {
+                if (P == 25) f(Grp<5, 5>{});
+            }
     }
+}
+template <int CN, bool ODD, class F>
+__device__ __forceinline__ void on_first(const LinePlan& lp, F&& f) {
+    if constexpr (CN > 0) f(typename CtLine<CN>::G1{});
+    else first_group<ODD, CN == ANY>(lp.P1, f);
+}
+template <int CN, class F>
+__device__ __forceinline__ void on_second(const LinePlan& lp, F&& f) {
+    if constexpr (CN > 0) f(typename CtLine<CN>::G2{});
+    else second_group<CN == ANY>(lp.P2, f);
 }
 
 }  // namespace vdw

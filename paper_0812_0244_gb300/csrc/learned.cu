@@ -844,8 +844,8 @@ __global__ void __launch_bounds__(SORTED_BLOCK) k_learned_contract_gradk(float4*
 // ---------------------------------------------------------------------------
 // L3: assembly of Eq. (Vi), one thread per point (packed order)
 // ---------------------------------------------------------------------------
-// The inverse plane transforms of u_m have left N3 x N1 real rows at the start
-// of each plane of the spectrum buffer.  Per point: v_loc and g from the 8 u
+// The inverse plane transforms of u_m have left packed real rows in each plane
+// of the spectrum buffer.  Per point: v_loc and g from the 8 u
 // values and the coefficients the network pass stored in lw.
 // mode 0: v_loc to v, w = g grad n to w_out; mode 1: v_loc to v, g to g_out
 // (the plane transforms of w follow in k_w_planes).
@@ -859,7 +859,7 @@ __global__ void __launch_bounds__(256, 6) k_learned_usum(const float* __restrict
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < N; q += (long long)gridDim.x * blockDim.x) {
         int y, z, x, j;
         const long long gi = packed_point(q, g, y, z, x, j);
-        const float* up = uf + 2LL * y * g.ncols + (long long)z * g.N1 + x;
+        const float* up = uf + 2LL * y * g.ncols + packed_offset(x, j, z & 1, g.Nh);
         float vl = lw[2 * LRN_M * N + q], gg = lw[(2 * LRN_M + 1) * N + q];
 #pragma unroll
         for (int m = 0; m < LRN_M; ++m) {
@@ -885,7 +885,7 @@ __global__ void __launch_bounds__(256) k_u_fields(const float* __restrict__ uf, 
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
         int x, y, z;
         flat_point(i, g, x, y, z);
-        const float* up = uf + 2LL * y * g.ncols + (long long)z * g.N1 + x;
+        const float* up = uf + 2LL * y * g.ncols + packed_offset(x, z >> 1, z & 1, g.Nh);
 #pragma unroll
         for (int m = 0; m < LRN_M; ++m) U[m * N + i] = up[m * fstride];
     }
@@ -1108,97 +1108,128 @@ __global__ void __launch_bounds__(256) k_basis_weights(const float* __restrict__
 // spectral gradient: grad f = IFFT(i G f(G)), Nyquist components removed
 // ---------------------------------------------------------------------------
 template <int CN1, int CN3>
-__global__ void __launch_bounds__(PLANE_THREADS, 2) k_field_plane(const float* __restrict__ f, GridArgs g,
-                                                                   const Tw* __restrict__ tw,
-                                                                   float2* __restrict__ spec) {
+__global__ void __launch_bounds__(PLANE_THREADS, 2)
+    k_field_plane(const float* __restrict__ f, GridArgs g, const Tw* __restrict__ tw, float2* __restrict__ spec) {
     extern __shared__ float2 sm[];
-    float2* plane = sm;
-    Tw* tw1 = twiddles_after(plane, (size_t)(g.N3 * g.Nh));
-    Tw* tw3 = tw1 + g.N1;
-    const int y = blockIdx.x;
-    load_line_twiddles<CN1>(tw1, tw, g.N1);
-    load_line_twiddles<CN3>(tw3, tw + g.N1 + g.N2, g.N3);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const long long zs = (long long)g.N1 * g.N2;  // flat distance between rows z and z + 1
-    for (int jr = warp; jr < (g.N3 >> 1); jr += nw) {
-        const long long row = (long long)g.N1 * (y + (long long)g.N2 * 2 * jr);
-        float2* crow = plane + jr * 2 * g.Nh;
-        for (int x = lane; x < g.N1; x += 32) crow[x] = make_float2(f[row + x], f[row + zs + x]);
-    }
-    __syncthreads();
-    plane_forward<CN1, CN3>(plane, g, tw1, tw3);
+    const int N1 = CN1 > 0 ? CN1 : g.N1, Nh = N1 / 2 + 1;
+    const int y = blockIdx.x, zs = N1 * g.N2;  // flat distance between rows z and z + 1
+    const float* fp = f + (long long)N1 * y;
     float2* dst = spec + (long long)y * g.ncols;
-    for (int i = threadIdx.x; i < g.ncols; i += blockDim.x) dst[i] = plane[i];
+    plane_forward<CN1, CN3, Tw>(
+        sm, g, tw,
+        [&](int row, int x) {
+            const long long i = 2LL * row * zs + x;
+            return make_float2(fp[i], fp[i + zs]);
+        },
+        [&](int kz, int kx, float2 c) { dst[kz * Nh + kx] = c; });
 }
 
+// Block: 8 columns; the field's lines, transformed, then each derivative's.
+constexpr int GRAD_COLS = 8;
 template <int CN2>
 __global__ void __launch_bounds__(256, 2) k_pencil_grad(const float2* __restrict__ spec, float2* __restrict__ wspec,
-                                                        GridArgs g, const Tw* __restrict__ tw, int C) {
+                                                        GridArgs g, const Tw* __restrict__ tw) {
     extern __shared__ float2 sm[];
-    const int N2 = CN2 > 0 ? CN2 : g.N2;
-    float2* lines = sm;  // [4][C][N2]: the field, then its three derivatives
-    Tw* tw2 = twiddles_after(lines, (size_t)(4 * C * N2));
-    load_line_twiddles<CN2>(tw2, tw + g.N1, N2);
+    constexpr int C = GRAD_COLS;
+    LinePlan L = g.p2;
+    if constexpr (CN2 > 0) L = LinePlan{CN2, CtLine<CN2>::G1::P, CtLine<CN2>::G2::P};
+    const int N2 = L.n, P1 = L.P1, ps = P1 | 1;
+    const int S = pencil_stride(L);
+    Tw* tw2 = twiddles_after(sm, (size_t)4 * C * S);  // lines [4][C][S]: the field, then its three derivatives
+    load_twiddles(tw2, tw, N2 - P1);
     const int c0 = blockIdx.x * C;
-    const SmallDiv sC = small_div(C);  // i / C in the staging loops
-    for (int i = threadIdx.x; i < N2 * C; i += blockDim.x) {
-        const int yy = sdiv(i, sC), cc = i - yy * C;
-        const int col = c0 + cc;
-        lines[cc * N2 + yy] = col < g.ncols ? spec[(long long)yy * g.ncols + col] : make_float2(0.f, 0.f);
-    }
-    __syncthreads();
-    pencils_fft<CN2, false>(lines, C, N2, g.p2, tw2);
-    __syncthreads();
-    for (int pt = threadIdx.x; pt < C * N2; pt += blockDim.x) {
-        const int cc = pt / N2, yy = pt % N2;
-        const int col = c0 + cc;
-        const int kx = col % g.Nh, kz = col / g.Nh;
-        const int mx = (2 * kx == g.N1) ? 0 : kx;
-        const int my = (2 * yy == N2) ? 0 : ((2 * yy < N2) ? yy : yy - N2);
-        const int mz = (2 * kz == g.N3) ? 0 : ((2 * kz < g.N3) ? kz : kz - g.N3);
-        const float2 fv = lines[cc * N2 + yy];
-        const float G[3] = {g.gx * mx, g.gy * my, g.gz * mz};
+    const SmallDiv dP = small_div(P1);
+    on_first<CN2, true>(L, [&](auto tag) {
+        using R = decltype(tag);
+        const int m = N2 / R::P;
+        for (int it = threadIdx.x; it < C * m; it += blockDim.x) {
+            const int cc = it & (C - 1), j = it / C, col = c0 + cc;
+            float2 v[R::P];
 #pragma unroll
-        for (int c = 0; c < 3; ++c)  // i G f / N
-            lines[((1 + c) * C + cc) * N2 + yy] = make_float2(-G[c] * fv.y * g.invN, G[c] * fv.x * g.invN);
-    }
+            for (int i = 0; i < R::P; ++i)
+                v[i] = col < g.ncols ? spec[(long long)(j + i * m) * g.ncols + col] : make_float2(0.f, 0.f);
+            group_fft<R, false, true, Tw>(v, (const Tw*)nullptr, 1);
+            float2* d = sm + cc * S + ps * j;
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) d[R::digit(i)] = v[i];
+        }
+    });
     __syncthreads();
-    pencils_fft<CN2, true>(lines + C * N2, 3 * C, N2, g.p2, tw2);
+    on_second<CN2>(L, [&](auto tag) {
+        using R = decltype(tag);
+        for (int it = threadIdx.x; it < C * P1; it += blockDim.x) {
+            const int cc = it & (C - 1), k1 = it / C;
+            float2* d = sm + cc * S + k1;
+            float2 v[R::P];
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) v[i] = d[i * ps];
+            group_fft<R, false, false, Tw>(v, tw2 + k1, P1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) d[R::digit(i) * ps] = v[i];
+        }
+    });
     __syncthreads();
-    for (int i = threadIdx.x; i < 3 * N2 * C; i += blockDim.x) {
-        const int rr = sdiv(i, sC), cc = i - rr * C, yy = rr % N2, c = rr / N2;
-        const int col = c0 + cc;
-        if (col < g.ncols) wspec[((long long)c * N2 + yy) * g.ncols + col] = lines[((1 + c) * C + cc) * N2 + yy];
-    }
+    on_first<CN2, true>(L, [&](auto tag) {
+        using R = decltype(tag);
+        const int m = N2 / R::P;
+        const SmallDiv dm = small_div(m);
+        for (int it = threadIdx.x; it < 3 * C * m; it += blockDim.x) {
+            const int cc = it & (C - 1), t = it / C, c = sdiv(t, dm), j = t - c * m;
+            const int col = min(c0 + cc, g.ncols - 1);
+            const int kx = col % g.Nh, kz = col / g.Nh;
+            const int mx = (2 * kx == g.N1) ? 0 : kx;
+            const int mz = (2 * kz == g.N3) ? 0 : ((2 * kz < g.N3) ? kz : kz - g.N3);
+            float2 v[R::P];
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) {
+                const int k = j + i * m;
+                const int my = (2 * k == N2) ? 0 : ((2 * k < N2) ? k : k - N2);
+                const float G = c == 0 ? g.gx * mx : c == 1 ? g.gy * my : g.gz * mz;
+                const float2 fv = sm[cc * S + k + sdiv(k, dP) * (ps - P1)];
+                v[i] = make_float2(-G * fv.y * g.invN, G * fv.x * g.invN);  // i G f / N
+            }
+            group_fft<R, true, true, Tw>(v, (const Tw*)nullptr, 1);
+            float2* d = sm + ((1 + c) * C + cc) * S + ps * j;
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) d[R::digit(i)] = v[i];
+        }
+    });
+    __syncthreads();
+    on_second<CN2>(L, [&](auto tag) {
+        using R = decltype(tag);
+        const SmallDiv dp = small_div(P1);
+        for (int it = threadIdx.x; it < 3 * C * P1; it += blockDim.x) {
+            const int cc = it & (C - 1), t = it / C, c = sdiv(t, dp), k1 = t - c * P1;
+            const int col = c0 + cc;
+            const float2* d = sm + ((1 + c) * C + cc) * S + k1;
+            float2 v[R::P];
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) v[i] = d[i * ps];
+            group_fft<R, true, false, Tw>(v, tw2 + k1, P1);
+            if (col < g.ncols) {
+#pragma unroll
+                for (int i = 0; i < R::P; ++i)
+                    wspec[((long long)c * N2 + k1 + P1 * R::digit(i)) * g.ncols + col] = v[i];
+            }
+        }
+    });
 }
 
 template <int CN1, int CN3>
-__global__ void __launch_bounds__(PLANE_THREADS, 2) k_plane_inv3(const float2* __restrict__ wspec, GridArgs g,
-                                                                  const Tw* __restrict__ tw,
-                                                                  float* __restrict__ out) {
+__global__ void __launch_bounds__(PLANE_THREADS, 2)
+    k_plane_inv3(const float2* __restrict__ wspec, GridArgs g, const Tw* __restrict__ tw, float* __restrict__ out) {
     extern __shared__ float2 sm[];
-    float2* plane = sm;
-    Tw* tw1 = twiddles_after(plane, (size_t)(g.N3 * g.Nh));
-    Tw* tw3 = tw1 + g.N1;
-    const int y = blockIdx.x, c = blockIdx.y;
-    load_line_twiddles<CN1>(tw1, tw, g.N1);
-    load_line_twiddles<CN3>(tw3, tw + g.N1 + g.N2, g.N3);
+    const int N1 = CN1 > 0 ? CN1 : g.N1, Nh = N1 / 2 + 1;
+    const int y = blockIdx.x, c = blockIdx.y, zs = N1 * g.N2;
     const float2* src = wspec + ((long long)c * g.N2 + y) * g.ncols;
-    for (int i = threadIdx.x; i < g.ncols; i += blockDim.x) plane[i] = src[i];
-    __syncthreads();
-    plane_inverse<CN1, CN3>(plane, g, tw1, tw3);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const long long zs = (long long)g.N1 * g.N2;
-    float* oc = out + c * g.N;
-    for (int jr = warp; jr < (g.N3 >> 1); jr += nw) {
-        const long long row = (long long)g.N1 * (y + (long long)g.N2 * 2 * jr);
-        const float2* crow = plane + jr * 2 * g.Nh;
-        for (int x = lane; x < g.N1; x += 32) {
-            const float2 d = crow[x];
-            oc[row + x] = d.x;
-            oc[row + zs + x] = d.y;
-        }
-    }
+    float* oc = out + c * g.N + (long long)N1 * y;
+    plane_inverse<CN1, CN3, Tw>(
+        sm, g, tw, [&](int kz, int kx) { return src[kz * Nh + kx]; },
+        [&](int row, int x, float2 d) {
+            const long long i = 2LL * row * zs + x;
+            oc[i] = d.x;
+            oc[i + zs] = d.y;
+        });
 }
 
 // ---------------------------------------------------------------------------
@@ -1248,18 +1279,14 @@ int lookup_blocks(vdw_ctx* c) {
 }
 // knot-gradient bins of k_learned_contract_gradk
 size_t smem_gradk(int J) { return sizeof(float) * (size_t)LRN_P * J; }
-size_t smem_plane1(const GridArgs& g) {
-    return sizeof(float2) * tw_offset((size_t)g.N3 * g.Nh) + sizeof(Tw) * (g.N1 + g.N3);
-}
 size_t smem_pgrad() {
     return sizeof(float) * ((size_t)LRN_H * LRN_H + LRN_M * LRN_H + 2 * LRN_H + 2 * LRN_H + LRN_M +
                             3 * (size_t)PG_TILE * PG_LD + PG_TILE * LRN_M + 2 * PG_TILE);
 }
-constexpr int GRAD_COLS = 8;
 size_t smem_pgrad_pencil(const GridArgs& g) {
-    return sizeof(float2) * tw_offset((size_t)4 * GRAD_COLS * g.N2) + sizeof(Tw) * g.N2;
+    return sizeof(float2) * tw_offset((size_t)4 * GRAD_COLS * pencil_stride(g.p2)) + sizeof(Tw) * (g.N2 - g.p2.P1);
 }
-const size_t SMEM_LIMIT = 227 * 1024 - 4 * 1024;
+const size_t SMEM_LIMIT = 227 * 1024 - 1024;
 
 template <class K>
 int set_smem(K kernel, size_t bytes, const char* name) {
@@ -1275,18 +1302,18 @@ int configure(vdw_ctx* c) {
     const GridArgs& g = c->g;
     int rc = set_smem(k_learned_net, smem_net(), "k_learned_net");
     if (!rc) rc = set_smem(k_learned_contract_gradk, smem_gradk(c->lrn_J), "k_learned_contract_gradk");
-    if (!rc) rc = set_smem(k_field_plane<CN1, CN3>, smem_plane1(g), "k_field_plane");
-    if (!rc) rc = set_smem(k_plane_inv3<CN1, CN3>, smem_plane1(g), "k_plane_inv3");
+    if (!rc) rc = set_smem(k_field_plane<CN1, CN3>, smem_plane(g), "k_field_plane");
+    if (!rc) rc = set_smem(k_plane_inv3<CN1, CN3>, smem_plane(g), "k_plane_inv3");
     if (!rc) rc = set_smem(k_pencil_grad<CN2>, smem_pgrad_pencil(g), "k_pencil_grad");
     if (!rc) rc = set_smem(k_learned_param_grad, smem_pgrad(), "k_learned_param_grad");
     return rc;
 }
 
 int configure_all(vdw_ctx* c) {
-    const GridArgs& g = c->g;
-    if (g.N1 == 180 && g.N2 == 180 && g.N3 == 72) return configure<180, 180, 72>(c);
-    if (g.N1 == 256 && g.N2 == 256 && g.N3 == 96) return configure<256, 256, 96>(c);
-    return configure<0, 0, 0>(c);
+    return on_grid(c->g, [&](auto d) {
+        using D = decltype(d);
+        return configure<D::N1, D::N2, D::N3>(c);
+    });
 }
 
 // learned scratch: partial sums [N2 * 8 + nb_sorted]
@@ -1296,7 +1323,6 @@ double* lrn_epart(vdw_ctx* c) {
 
 enum RunKind { RUN_ENERGY = 0, RUN_GRAD = 1 };
 
-template <int CN1, int CN2, int CN3>
 int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, float* w, int kind, double coef,
         double* gout, cudaStream_t s) {
     const GridArgs& g = c->g;
@@ -1330,7 +1356,7 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
         k_learned_net<<<nb0, L_NET_THREADS, smem_net(), s>>>(n, grad, g, P, la, specf, ep, c->d_invalid,
                                                          (want_pot && kind != RUN_GRAD) ? c->d_lw : nullptr);
     mark(ST_POINTWISE);
-    int rc = pipeline_planes_inplace(c, LRN_M, false, s);
+    int rc = planes_inplace(c, LRN_M, false, s);
     if (rc) return rc;
     mark(ST_PLANES_FWD);
     rc = sorted_forward(c, LRN_M, s);
@@ -1383,7 +1409,7 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
         mark(ST_PENCILS_INV);
     }
     if (kind == RUN_GRAD) {
-        rc = pipeline_planes_inplace(c, LRN_M, true, s);
+        rc = planes_inplace(c, LRN_M, true, s);
         if (rc) return rc;
         k_u_fields<<<nb_pt, 256, 0, s>>>(specf, g, c->d_U);
         const double dOmega = Omega / (double)g.N;
@@ -1395,7 +1421,7 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
         k_axpy<<<36, 256, 0, s>>>(gout + LRN_OFF_K, c->d_gK, coef, LRN_P * c->lrn_J);
     } else if (want_pot) {
         const int mode = (w != nullptr) ? 0 : 1;
-        rc = pipeline_planes_inplace(c, LRN_M, true, s);
+        rc = planes_inplace(c, LRN_M, true, s);
         if (!rc) {
             mark(ST_PLANES_INV);
             k_learned_usum<<<nb_pt, 256, 0, s>>>(specf, grad, g, c->d_lw, v, w, c->d_gg, mode);
@@ -1417,21 +1443,13 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
     return VDW_OK;
 }
 
-int run_any(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, float* w, int kind, double coef,
-            double* gout, cudaStream_t s) {
-    const GridArgs& g = c->g;
-    if (g.N1 == 180 && g.N2 == 180 && g.N3 == 72) return run<180, 180, 72>(c, n, grad, E, v, w, kind, coef, gout, s);
-    if (g.N1 == 256 && g.N2 == 256 && g.N3 == 96) return run<256, 256, 96>(c, n, grad, E, v, w, kind, coef, gout, s);
-    return run<0, 0, 0>(c, n, grad, E, v, w, kind, coef, gout, s);
-}
-
 template <int CN1, int CN2, int CN3>
 void spectral_gradient(vdw_ctx* c, const float* f, float* out, cudaStream_t s) {
     const GridArgs& g = c->g;
-    k_field_plane<CN1, CN3><<<g.N2, PLANE_THREADS, smem_plane1(g), s>>>(f, g, c->d_tw, c->d_spec);
+    k_field_plane<CN1, CN3><<<g.N2, plane_block(c, g.N2), smem_plane(g), s>>>(f, g, c->d_tw, c->d_spec);
     k_pencil_grad<CN2><<<(g.ncols + GRAD_COLS - 1) / GRAD_COLS, 256, smem_pgrad_pencil(g), s>>>(
-        c->d_spec, c->d_wspec, g, c->d_tw, GRAD_COLS);
-    k_plane_inv3<CN1, CN3><<<dim3(g.N2, 3), PLANE_THREADS, smem_plane1(g), s>>>(c->d_wspec, g, c->d_tw, out);
+        c->d_spec, c->d_wspec, g, c->d_tw + tw_off_y(g));
+    k_plane_inv3<CN1, CN3><<<dim3(g.N2, 3), plane_block(c, 3LL * g.N2), smem_plane(g), s>>>(c->d_wspec, g, c->d_tw, out);
 }
 
 bool lrn_ready(vdw_ctx* c) {
@@ -1497,7 +1515,7 @@ void learned_free(vdw_ctx* c) {
 int learned_run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, float* w, cudaStream_t s) {
     if (!lrn_ready(c)) return VDW_ERR_STATE;
     if ((v || w) && !c->d_lw) VDW_CUDA(cudaMalloc(&c->d_lw, sizeof(float) * (2 * LRN_M + 2) * (size_t)c->g.N));
-    return run_any(c, n, grad, E, v, w, RUN_ENERGY, 0.0, nullptr, s);
+    return run(c, n, grad, E, v, w, RUN_ENERGY, 0.0, nullptr, s);
 }
 
 }  // namespace vdw
@@ -1607,7 +1625,7 @@ int vdw_learned_param_grad(vdw_handle c, const float* n, const float* grad, doub
     if (!lrn_ready(c)) return VDW_ERR_STATE;
     if (const int rw = check_wait(c)) return rw;
     if (!c->d_U) VDW_CUDA(cudaMalloc(&c->d_U, sizeof(float) * LRN_M * (size_t)c->g.N));
-    return run_any(c, n, grad, E, nullptr, nullptr, RUN_GRAD, coef, g_params, (cudaStream_t)stream);
+    return run(c, n, grad, E, nullptr, nullptr, RUN_GRAD, coef, g_params, (cudaStream_t)stream);
 }
 
 int vdw_learned_fit_grad(vdw_handle c, const float* n, const float* grad, const float* target, const float* weight,
@@ -1691,23 +1709,14 @@ int vdw_spectral_gradient(vdw_handle c, const float* f, float* grad, void* strea
     if (!c->planned) return VDW_ERR_STATE;
     const GridArgs& g = c->g;
     cudaStream_t s = (cudaStream_t)stream;
-    int rc = VDW_OK;
-    if (g.N1 == 180 && g.N2 == 180 && g.N3 == 72) {
-        rc = set_smem(k_field_plane<180, 72>, smem_plane1(g), "k_field_plane");
-        if (!rc) rc = set_smem(k_plane_inv3<180, 72>, smem_plane1(g), "k_plane_inv3");
-        if (!rc) rc = set_smem(k_pencil_grad<180>, smem_pgrad_pencil(g), "k_pencil_grad");
-        if (!rc) spectral_gradient<180, 180, 72>(c, f, grad, s);
-    } else if (g.N1 == 256 && g.N2 == 256 && g.N3 == 96) {
-        rc = set_smem(k_field_plane<256, 96>, smem_plane1(g), "k_field_plane");
-        if (!rc) rc = set_smem(k_plane_inv3<256, 96>, smem_plane1(g), "k_plane_inv3");
-        if (!rc) rc = set_smem(k_pencil_grad<256>, smem_pgrad_pencil(g), "k_pencil_grad");
-        if (!rc) spectral_gradient<256, 256, 96>(c, f, grad, s);
-    } else {
-        rc = set_smem(k_field_plane<0, 0>, smem_plane1(g), "k_field_plane");
-        if (!rc) rc = set_smem(k_plane_inv3<0, 0>, smem_plane1(g), "k_plane_inv3");
-        if (!rc) rc = set_smem(k_pencil_grad<0>, smem_pgrad_pencil(g), "k_pencil_grad");
-        if (!rc) spectral_gradient<0, 0, 0>(c, f, grad, s);
-    }
+    const int rc = on_grid(g, [&](auto d) {
+        using D = decltype(d);
+        int r = set_smem(k_field_plane<D::N1, D::N3>, smem_plane(g), "k_field_plane");
+        if (!r) r = set_smem(k_plane_inv3<D::N1, D::N3>, smem_plane(g), "k_plane_inv3");
+        if (!r) r = set_smem(k_pencil_grad<D::N2>, smem_pgrad_pencil(g), "k_pencil_grad");
+        if (!r) spectral_gradient<D::N1, D::N2, D::N3>(c, f, grad, s);
+        return r;
+    });
     if (rc) return rc;
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;

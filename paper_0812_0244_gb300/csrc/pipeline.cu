@@ -4,14 +4,14 @@
 //                       Eq. fofx), theta_a = n p_a(q) (text after Eq. Eoffk)
 //                       into packed real planes; Delta E partial sums
 //                       (Eqs. DEnl, Depsnl)
-//   P1 k_planes_inplace forward plane transforms of theta_a in place: R2C
-//                       along x and C2C along z in shared memory
+//   P1 (planes.cu)      forward plane transforms of theta_a in place: R2C
+//                       along x and C2C along z through shared memory
 //   P2 (contract.cu)    C2C along y of all Nq fields, points written in |G|
 //                       order; per G: u_a(G) = sum_b phi_ab(|G|) theta_b(G)
 //                       with phi_ab from the radial table, energy of Eq.
 //                       (Eoffk) in FP64; inverse C2C along y (Eqs. epsilon,
 //                       epsofk)
-//   P3 k_planes_inplace inverse plane transform of u_a (in place)
+//   P3 (planes.cu)      inverse plane transform of u_a (in place)
 //      k_u_sum          Eq. (Vi) per point: v_loc and g of w = g grad n
 //      k_w_planes       forward plane transform of w
 //   P4 k_pencil_div     y transform of w, i G' . w(G), inverse y transform
@@ -21,9 +21,9 @@
 // [field][N2][N3][Nh] with Nh = N1/2+1 (a y plane of the half spectrum is one
 // contiguous block, a pencil along y strides by N3 Nh).
 //
-// Every kernel is a template over the line lengths (CN1, CN2, CN3): the
-// grids 180 x 180 x 72 and 256 x 256 x 96 get compile-time transforms, any
-// other size (0) the runtime-length engine.
+// The transform kernels are templates over the line lengths (CN1, CN2, CN3):
+// the grids 180 x 180 x 72 and 256 x 256 x 96 get compile-time lengths, any
+// other size one of the two run-time kinds of fft.cuh.
 #include "plane.cuh"
 #include "pointwise.cuh"
 
@@ -128,116 +128,14 @@ __global__ void __launch_bounds__(256, 6) k_pointwise(const float* __restrict__ 
     if (threadIdx.x == 0 && b > 0.0) atomicAdd(invalid, (unsigned long long)b);
 }
 
-// P1 (the forward plane transforms of theta_a) is k_planes_inplace below; P2
-// (y transforms and the contraction) is in contract.cu.
+// P1 (the forward plane transforms of theta_a) is in planes.cu; P2 (y
+// transforms and the contraction) in contract.cu.
 
 // ---------------------------------------------------------------------------
-// P3: inverse plane transforms of u_a, in place
+// P3': the assembly of Eq. (Vi)
 // ---------------------------------------------------------------------------
-// One block per (y plane, field): the plane arrives by one bulk asynchronous
-// copy (completion counted on an mbarrier) while the twiddles load.
-// Inverse: the plane of u_a(G) goes through the inverse z and x transforms,
-// and its N3 x N1 real values (unscaled: 1/N is folded into the contraction)
-// overwrite the start of the same plane of the spectrum buffer, rows of N1
-// floats.  Forward: the plane holds real rows in the packed layout of the
-// plane transforms (real rows 2j and 2j+1 as the real and imaginary parts of
-// complex row j, rows of 2 Nh complex values) and is replaced by its half
-// spectrum.
-__device__ __forceinline__ void mbar_init1(uint64_t* bar) {
-    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"((uint32_t)__cvta_generic_to_shared(bar)) : "memory");
-}
-// Bulk copy of `bytes` (multiple of 16, both addresses 16-byte aligned) from
-// global memory into this block's shared memory, counted on bar.
-__device__ __forceinline__ void bulk_load(void* dst, const void* src, uint32_t bytes, uint64_t* bar) {
-    const uint32_t b = (uint32_t)__cvta_generic_to_shared(bar);
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(dst);
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(b), "r"(bytes) : "memory");
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(d),
-                 "l"(src), "r"(bytes), "r"(b)
-                 : "memory");
-}
-// Bounded wait for the phase of the given parity; false if it gave up.
-__device__ __forceinline__ bool mbar_wait_parity(uint64_t* bar, uint32_t parity) {
-    const uint32_t a = (uint32_t)__cvta_generic_to_shared(bar);
-    for (int i = 0; i < (1 << 20); ++i) {
-        uint32_t done;
-        asm volatile(
-            "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-            "selp.u32 %0, 1, 0, p;\n\t}\n"
-            : "=r"(done)
-            : "r"(a), "r"(parity)
-            : "memory");
-        if (done) return true;
-    }
-    return false;
-}
-
-// Three blocks per SM at N1 = 180 (80 registers, a few spilled: 0.160 and
-// 0.157 ms for the forward and inverse stage against 0.171 and 0.165 ms at
-// two blocks); two elsewhere.
-template <int CN1, int CN3, bool INV>
-__global__ void __launch_bounds__(PLANE_THREADS, CN1 == 180 ? 3 : 2)
-    k_planes_inplace(float2* __restrict__ spec, GridArgs g, const Tw* __restrict__ tw, int bulk,
-                     int* __restrict__ wait_err) {
-    extern __shared__ float2 sm[];
-    __shared__ uint64_t bar;
-    float2* plane = sm;
-    // the forward transforms of theta feed the energy: hi/lo twiddles there
-    using W = TwOf<!INV>;
-    W* tw1 = twiddles_after<W>(plane, (size_t)(g.N3 * g.Nh));
-    W* tw3 = tw1 + g.N1;
-    const int y = blockIdx.x, a = blockIdx.y;
-    float2* src = spec + blockIdx.z * g.bs_spec + ((long long)a * g.N2 + y) * g.ncols;
-    // bulk: one copy of the whole plane (16-byte aligned, a multiple of 16
-    // bytes), in flight while the twiddles load
-    if (bulk) {
-        if (threadIdx.x == 0) mbar_init1(&bar);
-        __syncthreads();
-        if (threadIdx.x == 0) bulk_load(plane, src, (uint32_t)(sizeof(float2) * (size_t)g.ncols), &bar);
-    } else {
-        for (int i = threadIdx.x; i < g.ncols; i += blockDim.x) plane[i] = src[i];
-    }
-    load_line_twiddles<CN1>(tw1, tw, g.N1);
-    load_line_twiddles<CN3>(tw3, tw + g.N1 + g.N2, g.N3);
-    __syncthreads();
-    const bool got = !bulk || mbar_wait_parity(&bar, 0u);
-    if (__syncthreads_or(!got)) {
-        // a wait gave up: record it for the next entry point, give the copy in
-        // flight (it writes this block's shared memory) a second bounded wait,
-        // and leave the plane as it is rather than transform a partial one
-        if (threadIdx.x == 0) {
-            *(volatile int*)wait_err = 1;
-            __threadfence_system();
-        }
-        mbar_wait_parity(&bar, 0u);
-        return;
-    }
-    if constexpr (INV) {
-        plane_inverse<CN1, CN3>(plane, g, tw1, tw3);
-        float* dst = reinterpret_cast<float*>(src);
-        const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-        // complex row jr holds real rows 2 jr (real parts) and 2 jr + 1 (imaginary parts)
-        for (int jr = warp; jr < (g.N3 >> 1); jr += nw) {
-            const float2* crow = plane + jr * 2 * g.Nh;
-            float* d0 = dst + 2 * jr * g.N1;
-            for (int x = lane; x < g.N1; x += 32) {
-                const float2 u = crow[x];
-                d0[x] = u.x;
-                d0[g.N1 + x] = u.y;
-            }
-        }
-    } else {
-        plane_forward<CN1, CN3>(plane, g, tw1, tw3);
-        for (int i = threadIdx.x; i < g.ncols; i += blockDim.x) src[i] = plane[i];
-    }
-}
-
-// ---------------------------------------------------------------------------
-// P3': the assembly of Eq. (Vi), one thread per point
-// ---------------------------------------------------------------------------
-// S0 = sum_a u_a p_a(q), S1 = sum_a u_a p_a'(q) from the real u_a planes left
-// in the spectrum buffer by the inverse k_planes_inplace.  On interval k with
+// S0 = sum_a u_a p_a(q), S1 = sum_a u_a p_a'(q) from the packed real u_a planes
+// left in the spectrum buffer by the inverse k_planes_inplace.  On interval k with
 // A = 1 - t, B = t, p_a = A d_ak + B d_a,k+1 + [(A^3 - A) M_ak + (B^3 - B)
 // M_a,k+1] h^2/6 is linear in the second derivatives M, so both sums need
 // only u_k, u_k+1 and the two dot products m0 = sum_a u_a M_ak, m1 = sum_a
@@ -247,8 +145,10 @@ __global__ void __launch_bounds__(PLANE_THREADS, CN1 == 180 ? 3 : 2)
 // g_out (the plane transforms of w follow in k_w_planes).
 constexpr int USUM_THREADS = 256;
 
+// One thread takes the two points z = 2 j, 2 j + 1 of a packed row, so that a
+// field's two values come by one 8-byte load.
 template <int NQ>
-__global__ void __launch_bounds__(USUM_THREADS) k_u_sum(const float* __restrict__ uf, const float* __restrict__ grad,
+__global__ void __launch_bounds__(USUM_THREADS) k_u_sum(const float2* __restrict__ uf, const float* __restrict__ grad,
                                                         const float* __restrict__ tk, const uint8_t* __restrict__ kk,
                                                         const float4* __restrict__ aux, GridArgs g, PointParams P,
                                                         float* __restrict__ v, float* __restrict__ w_out,
@@ -257,7 +157,7 @@ __global__ void __launch_bounds__(USUM_THREADS) k_u_sum(const float* __restrict_
     {
         // density blockIdx.y of a batch
         const long long b = blockIdx.y;
-        uf += 2 * b * g.bs_spec;
+        uf += b * g.bs_spec;
         grad += 3 * b * g.N;
         tk += b * g.N;
         kk += b * g.N;
@@ -269,41 +169,49 @@ __global__ void __launch_bounds__(USUM_THREADS) k_u_sum(const float* __restrict_
     load_spline_smem(&sp, P);
     __syncthreads();
     const long long N = g.N;
-    const long long fstride = 2LL * g.N2 * g.ncols;  // floats between the planes of two fields
-    const int N1 = g.N1;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N; i += (long long)gridDim.x * blockDim.x) {
-        int x, y, z;
-        flat_point(i, g, x, y, z);
-        const float* up = uf + 2LL * y * g.ncols + (long long)z * N1 + x;
-        const int k = kk[i];
-        float vl = 0.f, gg = 0.f;
-        if (k != K_INVALID) {
-            float u[NQ];
+    const long long fstride = (long long)g.N2 * g.ncols;  // values between the planes of two fields
+    const long long zs = (long long)g.N1 * g.N2;
+    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < N / 2; i += (long long)gridDim.x * blockDim.x) {
+        int x, y, j;
+        flat_point(i, g, x, y, j);  // (x, y) of the plane z = 2 j
+        const float2* up = uf + (long long)y * g.ncols + (2 * j * g.Nh + x);
+        const long long i0 = i + j * zs;
+        const int k0 = kk[i0], k1 = kk[i0 + zs];
+        const int c0 = k0 == K_INVALID ? 0 : k0, c1 = k1 == K_INVALID ? 0 : k1;
+        float2 uk = make_float2(0.f, 0.f), uk1 = uk, m0 = uk, m1 = uk;
 #pragma unroll
-            for (int a = 0; a < NQ; ++a) u[a] = up[a * fstride];
-            const float t = tk[i];
-            const float4 ax = aux[i];
-            float uk = 0.f, uk1 = 0.f, m0 = 0.f, m1 = 0.f;
+        for (int a = 0; a < NQ; ++a) {
+            const float2 u = up[a * fstride];
+            const float* Ma = sp.Mq + a * MAX_NQ;
+            m0.x = fmaf(u.x, Ma[c0], m0.x);
+            m1.x = fmaf(u.x, Ma[c0 + 1], m1.x);
+            m0.y = fmaf(u.y, Ma[c1], m0.y);
+            m1.y = fmaf(u.y, Ma[c1 + 1], m1.y);
+            uk.x = (a == c0) ? u.x : uk.x;
+            uk1.x = (a == c0 + 1) ? u.x : uk1.x;
+            uk.y = (a == c1) ? u.y : uk.y;
+            uk1.y = (a == c1 + 1) ? u.y : uk1.y;
+        }
 #pragma unroll
-            for (int a = 0; a < NQ; ++a) {
-                m0 = fmaf(u[a], sp.Mq[a * MAX_NQ + k], m0);
-                m1 = fmaf(u[a], sp.Mq[a * MAX_NQ + k + 1], m1);
-                uk = (a == k) ? u[a] : uk;
-                uk1 = (a == k + 1) ? u[a] : uk1;
-            }
+        for (int s = 0; s < 2; ++s) {
+            const long long ii = i0 + s * zs;
+            const int k = s ? c1 : c0;
+            const float t = tk[ii];
+            const float4 ax = aux[ii];
+            const float a0 = s ? uk.y : uk.x, a1 = s ? uk1.y : uk1.x, b0 = s ? m0.y : m0.x, b1 = s ? m1.y : m1.x;
             const float A = 1.f - t, B = t;
-            const float s0 = A * uk + B * uk1 + ((A * A * A - A) * m0 + (B * B * B - B) * m1) * sp.h26[k];
-            const float s1 = (uk1 - uk) * sp.ih[k] + ((3.f * B * B - 1.f) * m1 - (3.f * A * A - 1.f) * m0) * sp.h6[k];
-            vl = s0 + ax.x * s1 + ax.z;
-            gg = ax.y * s1 + ax.w;
+            const float s0 = A * a0 + B * a1 + ((A * A * A - A) * b0 + (B * B * B - B) * b1) * sp.h26[k];
+            const float s1 = (a1 - a0) * sp.ih[k] + ((3.f * B * B - 1.f) * b1 - (3.f * A * A - 1.f) * b0) * sp.h6[k];
+            const bool ok = (s ? k1 : k0) != K_INVALID;
+            const float vl = ok ? s0 + ax.x * s1 + ax.z : 0.f, gg = ok ? ax.y * s1 + ax.w : 0.f;
+            if (v) v[ii] = vl;
+            if (mode == 0 && w_out) {
+                w_out[ii] = gg * grad[ii];
+                w_out[N + ii] = gg * grad[N + ii];
+                w_out[2 * N + ii] = gg * grad[2 * N + ii];
+            }
+            if (mode == 1) g_out[ii] = gg;
         }
-        if (v) v[i] = vl;
-        if (mode == 0 && w_out) {
-            w_out[i] = gg * grad[i];
-            w_out[N + i] = gg * grad[N + i];
-            w_out[2 * N + i] = gg * grad[2 * N + i];
-        }
-        if (mode == 1) g_out[i] = gg;
     }
 }
 
@@ -311,119 +219,145 @@ __global__ void __launch_bounds__(USUM_THREADS) k_u_sum(const float* __restrict_
 // P3b: forward plane transforms of the three components of w = g grad n
 // ---------------------------------------------------------------------------
 template <int CN1, int CN3>
-__global__ void __launch_bounds__(PLANE_THREADS, 2) k_w_planes(const float* __restrict__ gfield,
-                                                                const float* __restrict__ grad, GridArgs g,
-                                                                const Tw* __restrict__ tw,
-                                                                float2* __restrict__ wspec) {
+__global__ void __launch_bounds__(PLANE_THREADS, 2)
+    k_w_planes(const float* __restrict__ gfield, const float* __restrict__ grad, GridArgs g, const Tw* __restrict__ tw,
+               float2* __restrict__ wspec) {
     extern __shared__ float2 sm[];
-    float2* plane = sm;
-    float2* tw1 = twiddles_after<float2>(plane, (size_t)(g.N3 * g.Nh));
-    float2* tw3 = tw1 + g.N1;
+    const int N1 = CN1 > 0 ? CN1 : g.N1, Nh = N1 / 2 + 1;
     const int y = blockIdx.x, c = blockIdx.y;
-    gfield += blockIdx.z * g.N;  // density blockIdx.z of a batch
-    grad += 3 * blockIdx.z * g.N;
-    wspec += blockIdx.z * g.bs_wspec;
-    load_line_twiddles<CN1>(tw1, tw, g.N1);
-    load_line_twiddles<CN3>(tw3, tw + g.N1 + g.N2, g.N3);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const float* gc = grad + c * g.N;
-    const long long zs = (long long)g.N1 * g.N2;  // flat distance between rows z and z + 1
-    for (int jr = warp; jr < (g.N3 >> 1); jr += nw) {
-        const long long row = (long long)g.N1 * (y + (long long)g.N2 * 2 * jr);
-        float2* crow = plane + jr * 2 * g.Nh;
-        for (int x = lane; x < g.N1; x += 32)
-            crow[x] = make_float2(gfield[row + x] * gc[row + x], gfield[row + zs + x] * gc[row + zs + x]);
-    }
-    __syncthreads();
-    plane_forward<CN1, CN3>(plane, g, tw1, tw3);
-    float2* dst = wspec + ((long long)c * g.N2 + y) * g.ncols;
-    for (int i = threadIdx.x; i < g.ncols; i += blockDim.x) dst[i] = plane[i];
+    const int zs = N1 * g.N2;  // flat distance between rows z and z + 1
+    // density blockIdx.z of a batch
+    const float* gf = gfield + blockIdx.z * g.N + (long long)N1 * y;
+    const float* gc = grad + (3 * blockIdx.z + c) * g.N + (long long)N1 * y;
+    float2* dst = wspec + blockIdx.z * g.bs_wspec + ((long long)c * g.N2 + y) * g.ncols;
+    plane_forward<CN1, CN3, float2>(
+        sm, g, tw,
+        [&](int row, int x) {
+            const long long i = 2LL * row * zs + x;
+            return make_float2(gf[i] * gc[i], gf[i + zs] * gc[i + zs]);
+        },
+        [&](int kz, int kx, float2 w) { dst[kz * Nh + kx] = w; });
 }
 
 // ---------------------------------------------------------------------------
 // P4: spectral divergence along pencils
 // ---------------------------------------------------------------------------
-constexpr int DIV_COLS_CT = 8;  // columns per divergence block
+// Block: the three components of 8 columns.  The forward transform's second
+// group, d = i G' . w / N and the inverse transform's first group (the same
+// radices: the inverse takes the two groups in the other order) stay in one
+// thread's registers.  180 x 180 x 72: 26 -> 18 us; 100^3: 29 -> 25 us.
+constexpr int DIV_COLS = 8;
+constexpr int DIV_THREADS = 128;
 
 template <int CN2>
-__global__ void __launch_bounds__(256, 2) k_pencil_div(float2* __restrict__ wspec, GridArgs g,
-                                                       const Tw* __restrict__ tw, int C) {
+__global__ void __launch_bounds__(DIV_THREADS) k_pencil_div(float2* __restrict__ wspec, GridArgs g,
+                                                            const Tw* __restrict__ tw, const Tw* __restrict__ tw_swap) {
     extern __shared__ float2 sm[];
-    const int N2 = CN2 > 0 ? CN2 : g.N2;
-    const int S = pencil_stride(N2);
-    float2* lines = sm;  // [3][C][S]
-    float2* tw2 = twiddles_after<float2>(lines, (size_t)(3 * C * S));
+    constexpr int C = DIV_COLS;
+    LinePlan L = g.p2;
+    if constexpr (CN2 > 0) L = LinePlan{CN2, CtLine<CN2>::G1::P, CtLine<CN2>::G2::P};
+    const int N2 = L.n, P1 = L.P1, P2 = L.P2, ps = P1 | 1;
+    const int S = pencil_stride(L);
+    float2* tw2 = twiddles_after<float2>(sm, (size_t)3 * C * S);
+    float2* tw2s = tw2 + (N2 - P1);
+    load_twiddles(tw2, tw, N2 - P1);
+    load_twiddles(tw2s, tw_swap, N2 - P2);
     wspec += blockIdx.y * g.bs_wspec;  // density blockIdx.y of a batch
-    load_line_twiddles<CN2>(tw2, tw + g.N1, N2);
     const int c0 = blockIdx.x * C;
-    const SmallDiv sC = small_div(C);  // i / C in the staging loops
-    const int tot = 3 * N2 * C;
-    for (int i = threadIdx.x; i < tot; i += blockDim.x) {
-        const int r = sdiv(i, sC), cc = i - r * C, yy = r % N2, c = r / N2;
-        const int col = c0 + cc;
-        const bool ok = col < g.ncols;
-        cp_async8(lines + (c * C + cc) * S + yy, ok ? wspec + ((long long)c * N2 + yy) * g.ncols + col : wspec, ok);
-    }
-    cp_async_wait_all();
+    on_first<CN2, true>(L, [&](auto tag) {
+        using R = decltype(tag);
+        constexpr int CM = CN2 > 0 ? CN2 / R::P : 0;
+        const int m = CN2 > 0 ? CM : L.P2;
+        const SmallDiv dm = small_div(m);
+        const long long step = (long long)m * g.ncols;
+        for (int it = threadIdx.x; it < 3 * C * m; it += blockDim.x) {
+            const int cc = it & (C - 1), t = it / C, c = cdiv<CM>(t, dm), j = t - c * m;
+            const int col = c0 + cc;
+            float2 v[R::P];
+            const float2* src = wspec + (long long)(c * N2 + j) * g.ncols + col;
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) v[i] = col < g.ncols ? src[i * step] : make_float2(0.f, 0.f);
+            group_fft<R, false, true, float2>(v, (const float2*)nullptr, 1);
+            float2* d = sm + (c * C + cc) * S + ps * j;
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) d[R::digit(i)] = v[i];
+        }
+    });
     __syncthreads();
-    pencils_fft<CN2, false>(lines, 3 * C, N2, g.p2, tw2, S);
+    on_second<CN2>(L, [&](auto tag) {
+        using R = decltype(tag);
+        for (int it = threadIdx.x; it < C * P1; it += blockDim.x) {
+            const int cc = it & (C - 1), k1 = it / C;
+            const int col = min(c0 + cc, g.ncols - 1);
+            const int kx = col % g.Nh, kz = col / g.Nh;
+            // derivative wave numbers with the Nyquist components removed
+            const int mx = (2 * kx == g.N1) ? 0 : kx;
+            const int mz = (2 * kz == g.N3) ? 0 : ((2 * kz < g.N3) ? kz : kz - g.N3);
+            const float Gx = g.gx * mx, Gz = g.gz * mz;
+            float2* l = sm + cc * S + k1;
+            float2 dv[R::P];  // i G . w / N at k = k1 + P1 i
+#pragma unroll 1
+            for (int c = 0; c < 3; ++c) {
+                float2 v[R::P];
+#pragma unroll
+                for (int i = 0; i < R::P; ++i) v[i] = l[c * C * S + i * ps];
+                group_fft<R, false, false, float2>(v, tw2 + k1, P1);
+#pragma unroll
+                for (int i = 0; i < R::P; ++i) {
+                    const int k = k1 + P1 * R::digit(i);
+                    const int my = (2 * k == N2) ? 0 : ((2 * k < N2) ? k : k - N2);
+                    const float G = (c == 0 ? Gx : c == 1 ? g.gy * my : Gz) * g.invN;
+                    float2& d = dv[R::digit(i)];
+                    d.x = c == 0 ? -G * v[i].y : fmaf(-G, v[i].y, d.x);
+                    d.y = c == 0 ? G * v[i].x : fmaf(G, v[i].x, d.y);
+                }
+            }
+            group_fft<R, true, true, float2>(dv, (const float2*)nullptr, 1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) l[R::digit(i) * ps] = dv[i];
+        }
+    });
     __syncthreads();
-    for (int pt = threadIdx.x; pt < C * N2; pt += blockDim.x) {
-        const int cc = pt / N2, yy = pt % N2;
-        const int col = c0 + cc;
-        if (col >= g.ncols) continue;
-        const int kx = col % g.Nh, kz = col / g.Nh;
-        // derivative wave numbers with the Nyquist components removed
-        const int mx = (2 * kx == g.N1) ? 0 : kx;
-        const int my = (2 * yy == N2) ? 0 : ((2 * yy < N2) ? yy : yy - N2);
-        const int mz = (2 * kz == g.N3) ? 0 : ((2 * kz < g.N3) ? kz : kz - g.N3);
-        const float2 wx = lines[(0 * C + cc) * S + yy];
-        const float2 wy = lines[(1 * C + cc) * S + yy];
-        const float2 wz = lines[(2 * C + cc) * S + yy];
-        const float Gx = g.gx * mx, Gy = g.gy * my, Gz = g.gz * mz;
-        // i G . w / N
-        const float re = Gx * wx.x + Gy * wy.x + Gz * wz.x;
-        const float im = Gx * wx.y + Gy * wy.y + Gz * wz.y;
-        lines[(0 * C + cc) * S + yy] = make_float2(-im * g.invN, re * g.invN);
-    }
-    __syncthreads();
-    pencils_fft<CN2, true>(lines, C, N2, g.p2, tw2, S);
-    __syncthreads();
-    for (int i = threadIdx.x; i < N2 * C; i += blockDim.x) {
-        const int yy = sdiv(i, sC), cc = i - yy * C;
-        const int col = c0 + cc;
-        if (col < g.ncols) wspec[(long long)yy * g.ncols + col] = lines[cc * S + yy];
-    }
+    on_first<CN2, true>(L, [&](auto tag) {
+        using R = decltype(tag);
+        const long long step = (long long)P2 * g.ncols;
+        for (int it = threadIdx.x; it < C * P2; it += blockDim.x) {
+            const int cc = it & (C - 1), j = it / C;
+            const int col = c0 + cc;
+            const float2* l = sm + cc * S + ps * j;
+            float2 v[R::P];
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) v[i] = l[i];
+            group_fft<R, true, false, float2>(v, tw2s + j, P2);
+            float2* dst = wspec + (long long)j * g.ncols + col;
+            if (col < g.ncols) {
+#pragma unroll
+                for (int i = 0; i < R::P; ++i) dst[R::digit(i) * step] = v[i];
+            }
+        }
+    });
 }
 
 // ---------------------------------------------------------------------------
 // P5: inverse plane transform of D.w, v = v_loc - D.w
 // ---------------------------------------------------------------------------
 template <int CN1, int CN3>
-__global__ void __launch_bounds__(PLANE_THREADS, 2) k_div_final(const float2* __restrict__ wspec, GridArgs g,
-                                                      const Tw* __restrict__ tw, float* __restrict__ v) {
+__global__ void __launch_bounds__(PLANE_THREADS, 2)
+    k_div_final(const float2* __restrict__ wspec, GridArgs g, const Tw* __restrict__ tw, float* __restrict__ v) {
     extern __shared__ float2 sm[];
-    float2* plane = sm;
-    float2* tw1 = twiddles_after<float2>(plane, (size_t)(g.N3 * g.Nh));
-    float2* tw3 = tw1 + g.N1;
+    const int N1 = CN1 > 0 ? CN1 : g.N1, Nh = N1 / 2 + 1;
     const int y = blockIdx.x;
-    wspec += blockIdx.y * g.bs_wspec;  // density blockIdx.y of a batch
-    v += blockIdx.y * g.N;
-    load_line_twiddles<CN1>(tw1, tw, g.N1);
-    load_line_twiddles<CN3>(tw3, tw + g.N1 + g.N2, g.N3);
-    const float2* src = wspec + (long long)y * g.ncols;
-    for (int i = threadIdx.x; i < g.ncols; i += blockDim.x) plane[i] = src[i];
-    __syncthreads();
-    plane_inverse<CN1, CN3>(plane, g, tw1, tw3);
-    const float* pf = reinterpret_cast<const float*>(plane);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    // real row z: component z & 1 of complex row z / 2 (one row per warp: the
-    // read-modify-write of v keeps more rows in flight this way than by pairs)
-    for (int z = warp; z < g.N3; z += nw) {
-        const long long row = (long long)g.N1 * (y + (long long)g.N2 * z);
-        const float* srow = pf + 2 * ((z >> 1) * 2 * g.Nh) + (z & 1);
-        for (int x = lane; x < g.N1; x += 32) v[row + x] -= srow[2 * x];
-    }
+    const int zs = N1 * g.N2;
+    // density blockIdx.y of a batch
+    const float2* src = wspec + blockIdx.y * g.bs_wspec + (long long)y * g.ncols;
+    float* vp = v + blockIdx.y * g.N + (long long)N1 * y;
+    plane_inverse<CN1, CN3, float2>(
+        sm, g, tw, [&](int kz, int kx) { return src[kz * Nh + kx]; },
+        [&](int row, int x, float2 d) {
+            const long long i = 2LL * row * zs + x;
+            vp[i] -= d.x;
+            vp[i + zs] -= d.y;
+        });
 }
 
 // ---------------------------------------------------------------------------
@@ -589,61 +523,168 @@ __global__ void __launch_bounds__(EPART_SPLIT) k_energy_final(const double* __re
     }
 }
 
-// W_n^e = exp(-2 pi i e / n) in FP64, stored as the hi/lo FP32 pair of each part
-__global__ void k_twiddles(Tw* tw, int n, int off) {
-    for (int e = threadIdx.x + blockIdx.x * blockDim.x; e < n; e += blockDim.x * gridDim.x) {
+// Twiddle table of a line's second group with radices A, B, C after Ns (order
+// as group_fft reads it): W_n^e = exp(-2 pi i e / n) in FP64, stored as the
+// hi/lo FP32 pair of each part.
+__global__ void k_twiddles(Tw* tw, int n, int Ns, int A, int B, int C) {
+    const int tot = (A * B * C - 1) * Ns;
+    for (int i = threadIdx.x + blockIdx.x * blockDim.x; i < tot; i += blockDim.x * gridDim.x) {
+        int q = i / Ns;
+        const int k = i - q * Ns;
+        int e;
+        if (q < A - 1) {
+            e = (q + 1) * k * (n / (Ns * A));
+        } else if (q < A * B - 1) {
+            q -= A - 1;
+            e = (q / A + 1) * (k + (q % A) * Ns) * (n / (Ns * A * B));
+        } else {
+            q -= A * B - 1;
+            e = (q / (A * B) + 1) * (k + (q % (A * B)) * Ns) * (n / (Ns * A * B * C));
+        }
         double s, c;
         sincospi(-2.0 * (double)e / (double)n, &s, &c);
         const float ch = (float)c, sh = (float)s;
-        tw[off + e] = make_float4(ch, sh, (float)(c - (double)ch), (float)(s - (double)sh));
+        tw[i] = make_float4(ch, sh, (float)(c - (double)ch), (float)(s - (double)sh));
     }
 }
 
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-int make_line_plan(int n, LinePlan* lp) {
-    lp->n = n;
-    int m = n;
-    lp->c4 = lp->c2 = lp->c3 = lp->c5 = 0;
-    while (m % 4 == 0) { m /= 4; ++lp->c4; }
-    while (m % 2 == 0) { m /= 2; ++lp->c2; }
-    while (m % 3 == 0) { m /= 3; ++lp->c3; }
-    while (m % 5 == 0) { m /= 5; ++lp->c5; }
-    return m == 1 ? VDW_OK : VDW_ERR_SIZE;
+// The groups fft.cuh has (second_group / first_group): the radices of a
+// product, {1, 1, 1} where it has none.
+struct Radices {
+    int a, b, c;
+};
+static Radices radices_of(int P) {
+    switch (P) {
+        case 6: return {2, 3, 1};
+        case 8: return {4, 2, 1};
+        case 9: return {3, 3, 1};
+        case 10: return {2, 5, 1};
+        case 12: return {4, 3, 1};
+        case 15: return {3, 5, 1};
+        case 16: return {4, 4, 1};
+        case 18: return {2, 3, 3};
+        case 20: return {4, 5, 1};
+        case 24: return {4, 2, 3};
+        case 25: return {5, 5, 1};
+        case 27: return {3, 3, 3};
+        default: return {P, 1, 1};  // 1 .. 5
+    }
 }
 
-static size_t smem_plane(const GridArgs& g) {
-    return sizeof(float2) * tw_offset((size_t)g.N3 * g.Nh) + sizeof(Tw) * (g.N1 + g.N3);
+// The radices of n are 4, .., 4, 2, 3, .., 3, 5, .., 5 in this order.  Of the
+// places where that list can be cut into two groups that exist, the one with
+// the smallest larger group is taken (registers and work per thread), the
+// larger second group on a tie (longer runs in the first pass's loads).
+int make_line_plan(int n, bool sized, LinePlan* lp) {
+    lp->n = n;
+    lp->P1 = lp->P2 = 0;
+    if (sized) {
+        lp->P1 = n == 180 ? 15 : n == 72 ? 9 : n == 256 ? 16 : 12;
+        lp->P2 = n / lp->P1;
+        return VDW_OK;
+    }
+    int rad[16], nr = 0, m = n;
+    for (int r : {4, 2, 3, 5})
+        while (m % r == 0) {
+            rad[nr++] = r;
+            m /= r;
+        }
+    if (m != 1) return VDW_ERR_SIZE;
+    const auto is_group = [&](int i0, int i1, bool first) {
+        int P = 1;
+        for (int i = i0; i < i1; ++i) P *= rad[i];
+        if (P > 27 || i1 - i0 > 3) return 0;
+        if (P == 1) return first ? 0 : 1;
+        const Radices r = radices_of(P);
+        const int want[3] = {r.a, r.b, r.c};
+        for (int i = 0; i < 3; ++i)
+            if ((i0 + i < i1 ? rad[i0 + i] : 1) != want[i]) return 0;
+        if (!first && (P == 18 || P == 20 || P == 24 || P == 27)) return 0;
+        return P;
+    };
+    for (int cut = 1; cut <= nr; ++cut) {
+        const int a = is_group(0, cut, true), b = is_group(cut, nr, false);
+        if (!a || !b) continue;
+        const int big = std::max(a, b), cur = std::max(lp->P1, lp->P2);
+        if (lp->P1 == 0 || big < cur || (big == cur && b > lp->P2)) {
+            lp->P1 = a;
+            lp->P2 = b;
+        }
+    }
+    return lp->P1 ? VDW_OK : VDW_ERR_SIZE;
 }
-static size_t smem_pencil(const GridArgs& g, int nq, int C) {
-    return sizeof(float2) * tw_offset((size_t)nq * C * pencil_stride(g.N2)) + sizeof(Tw) * g.N2;
+
+// Block size in [lo, hi] (whole warps) with the fewest thread slots over
+// passes of the given numbers of items, the largest on a tie.
+int best_threads(std::initializer_list<int> items, int lo, int hi) {
+    int best = hi;
+    long long cost = -1;
+    for (int t = hi; t >= lo; t -= 32) {
+        long long c = 0;
+        for (int n : items) c += (long long)((n + t - 1) / t) * t;
+        if (cost < 0 || c < cost) {
+            cost = c;
+            best = t;
+        }
+    }
+    return best;
 }
-static size_t smem_pencil_run(const GridArgs& g, int nq, int C) { return smem_pencil(g, nq, C); }
+
+// shared memory of the plane kernels, forward or inverse
+static size_t smem_plane_of(const GridArgs& g, bool inverse, bool pad) {
+    const PlaneGeo p = plane_geo(g.p1.P1, g.p1.P2, inverse, pad);
+    return sizeof(float2) * tw_offset((size_t)(g.N3 / 2) * p.S) +
+           sizeof(Tw) * ((size_t)(g.N1 - g.p1.P1) + (g.N3 - g.p3.P1));
+}
+size_t smem_plane(const GridArgs& g) {
+    return std::max(smem_plane_of(g, false, g.pad_fwd), smem_plane_of(g, true, g.pad_inv));
+}
+// Block size of a plane kernel launched on nblocks planes: about 1024 threads
+// per SM over the blocks that shared memory and the grid allow there, and
+// among the sizes near that the one that wastes the fewest thread slots over
+// the five passes.
+int plane_block(const vdw_ctx* c, long long nblocks) {
+    const GridArgs& g = c->g;
+    const int nr = g.N3 / 2, nsm = std::max(c->nsm, 1);
+    const long long fit = std::max<long long>(1, 228 * 1024 / (long long)(smem_plane(g) + 1024));
+    const long long per_sm = std::max<long long>(1, std::min<long long>(fit, (nblocks + nsm - 1) / nsm));
+    const int hi = std::max(64, (int)std::min<long long>(PLANE_THREADS, 1024 / per_sm) / 32 * 32);
+    return best_threads({nr * g.p1.P2, nr * g.p1.P1, g.Nh * nr, g.Nh * g.p3.P2, g.Nh * g.p3.P1},
+                        std::max(64, hi * 3 / 4 / 32 * 32), hi);
+}
+static size_t smem_div(const GridArgs& g) {
+    return sizeof(float2) * tw_offset((size_t)3 * DIV_COLS * pencil_stride(g.p2)) +
+           sizeof(float2) * ((size_t)2 * g.N2 - g.p2.P1 - g.p2.P2);
+}
 
 // dynamic shared memory per block, leaving room for the kernels' static arrays
-static const size_t SMEM_MAX = 227 * 1024 - 5 * 1024;
-static const int DIV_COLS = DIV_COLS_CT;
+static const size_t SMEM_MAX = 227 * 1024 - 1024;
 
-int pipeline_plan_check(vdw_ctx* c, size_t* sp, size_t* spen, size_t* sa, size_t* sd) {
-    const GridArgs& g = c->g;
-    *sp = smem_plane(g);
-    *spen = sorted_pencil_smem(g);
-    // the inverse plane transforms of u take their planes by one bulk copy when
-    // a plane is a whole multiple of 16 bytes (every plane then starts 16-byte aligned)
-    c->bulk_planes = (sizeof(float2) * (size_t)g.ncols) % 16 == 0;
-    *sa = *sp;
-    *sd = smem_pencil_run(g, 3, DIV_COLS);
-    if (*sp > SMEM_MAX || *spen > SMEM_MAX || *sd > SMEM_MAX)
+int pipeline_plan_check(vdw_ctx* c) {
+    GridArgs& g = c->g;
+    g.pad_fwd = smem_plane_of(g, false, true) <= SMEM_MAX;
+    g.pad_inv = smem_plane_of(g, true, true) <= SMEM_MAX;
+    // the whole-plane limit of the unpadded rows
+    if (sizeof(float2) * (size_t)g.N3 * g.Nh + sizeof(Tw) * (g.N1 + g.N3) > 222 * 1024 ||
+        smem_plane(g) > SMEM_MAX || sorted_pencil_smem(g) > SMEM_MAX || smem_div(g) > SMEM_MAX)
         return VDW_ERR_SIZE;
     return VDW_OK;
 }
 
 int pipeline_make_twiddles(vdw_ctx* c) {
     const GridArgs& g = c->g;
-    k_twiddles<<<4, 256>>>(c->d_tw, g.N1, 0);
-    k_twiddles<<<4, 256>>>(c->d_tw, g.N2, g.N1);
-    k_twiddles<<<4, 256>>>(c->d_tw, g.N3, g.N1 + g.N2);
+    const bool sized = sized_grid(g.N1, g.N2, g.N3);
+    const auto make = [&](int off, int n, int Ns, int P) {
+        const Radices r = sized ? Radices{P, 1, 1} : radices_of(P);
+        if (P > 1) k_twiddles<<<4, 256>>>(c->d_tw + off, n, Ns, r.a, r.b, r.c);
+    };
+    make(0, g.N1, g.p1.P1, g.p1.P2);
+    make(tw_off_y(g), g.N2, g.p2.P1, g.p2.P2);
+    make(g.N1 + g.N2, g.N3, g.p3.P1, g.p3.P2);
+    make(tw_off_swap(g), g.N2, g.p2.P2, g.p2.P1);
     VDW_CUDA(cudaGetLastError());
     VDW_CUDA(cudaDeviceSynchronize());
     return VDW_OK;
@@ -665,17 +706,16 @@ int pipeline_stencil_gradient(vdw_ctx* c, const float* f, float* grad, cudaStrea
 // spline table is staged once per block
 static int u_sum_blocks(const vdw_ctx* c) {
     const GridArgs& g = c->g;
-    return (int)std::min<long long>((g.N + USUM_THREADS - 1) / USUM_THREADS,
+    return (int)std::min<long long>((g.N / 2 + USUM_THREADS - 1) / USUM_THREADS,
                                     (long long)std::max(c->usum_per_sm, 1) * std::max(c->nsm, 1));
 }
 
 static int launch_u_sum(vdw_ctx* c, const float* n, const float* grad, float* v, float* w, int mode, cudaStream_t s,
                         int B) {
     const GridArgs& g = c->g;
-    const float* uf = reinterpret_cast<const float*>(c->d_spec);
     const int nb = u_sum_blocks(c);
 #define VDW_U_SUM(NQ) \
-    k_u_sum<NQ><<<dim3(nb, B), USUM_THREADS, 0, s>>>(uf, grad, c->d_t, c->d_k, c->d_aux, g, c->pp, v, w, c->d_gg, mode)
+    k_u_sum<NQ><<<dim3(nb, B), USUM_THREADS, 0, s>>>(c->d_spec, grad, c->d_t, c->d_k, c->d_aux, g, c->pp, v, w, c->d_gg, mode)
     switch (c->pp.Nq) {
         case 20: VDW_U_SUM(20); break;
         case 8: VDW_U_SUM(8); break;
@@ -727,12 +767,12 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
     mark(ST_POINTWISE);
 
     const size_t sp = smem_plane(g);
-    k_planes_inplace<CN1, CN3, false><<<dim3(g.N2, P.Nq, B), PLANE_THREADS, sp, s>>>(c->d_spec, g, c->d_tw,
-                                                                                     c->bulk_planes, c->d_flags);
+    int rc = planes_inplace(c, P.Nq, false, s, B);
+    if (rc) return rc;
     mark(ST_PLANES_FWD);
 
     // y transforms, contraction in |G| order, inverse y transforms (contract.cu)
-    int rc = sorted_forward(c, P.Nq, s, B);
+    rc = sorted_forward(c, P.Nq, s, B);
     if (rc) return rc;
     mark(ST_PENCILS_FWD);
     rc = sorted_contract(c, c->d_epart + c->nb_point, want_pot ? 1 : 0, s, B);
@@ -776,8 +816,11 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
         }
         mark(ST_PENCILS_INV);
         const int mode = (w != nullptr) ? 0 : 1;
-        k_planes_inplace<CN1, CN3, true><<<dim3(g.N2, P.Nq, B), PLANE_THREADS, sp, s>>>(c->d_spec, g, c->d_tw,
-                                                                                        c->bulk_planes, c->d_flags);
+        rc = planes_inplace(c, P.Nq, true, s, B);
+        if (rc) {
+            join();
+            return rc;
+        }
         mark(ST_PLANES_INV);
         const int rcs = launch_u_sum(c, n, grad, v, w, mode, s, B);
         if (rcs) {
@@ -793,13 +836,12 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
             k_stencil_div_sub<<<stencil_blocks(g), 256, 0, s>>>(c->d_gg, grad, g, stencil_ih2(c), v);
             mark(ST_DIV_FINAL);
         } else if (mode == 1) {
-            k_w_planes<CN1, CN3><<<dim3(g.N2, 3, B), PLANE_THREADS, sp, s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
+            k_w_planes<CN1, CN3><<<dim3(g.N2, 3, B), plane_block(c, 3LL * g.N2 * B), sp, s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
             mark(ST_W_PLANES);
-            const size_t sd = smem_pencil_run(g, 3, DIV_COLS);
-            k_pencil_div<CN2><<<dim3((g.ncols + DIV_COLS - 1) / DIV_COLS, B), 256, sd, s>>>(c->d_wspec, g, c->d_tw,
-                                                                                          DIV_COLS);
+            k_pencil_div<CN2><<<dim3((g.ncols + DIV_COLS - 1) / DIV_COLS, B), DIV_THREADS, smem_div(g), s>>>(
+                c->d_wspec, g, c->d_tw + tw_off_y(g), c->d_tw + tw_off_swap(g));
             mark(ST_PENCIL_DIV);
-            k_div_final<CN1, CN3><<<dim3(g.N2, B), PLANE_THREADS, sp, s>>>(c->d_wspec, g, c->d_tw, v);
+            k_div_final<CN1, CN3><<<dim3(g.N2, B), plane_block(c, (long long)g.N2 * B), sp, s>>>(c->d_wspec, g, c->d_tw, v);
             mark(ST_DIV_FINAL);
         }
     }
@@ -808,31 +850,13 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
     return VDW_OK;
 }
 
-// Dynamic shared-memory limits of the kernels a plan uses (set once per plan).
-// Sets a kernel's dynamic shared-memory limit and checks that the block size
-// it will be launched with fits its register use.
-template <class K>
-static int set_and_check(K kernel, const char* name, int smem, int threads) {
-    if (const int rs = raise_smem_limit(kernel, (size_t)smem)) return rs;
-    cudaFuncAttributes fa;
-    VDW_CUDA(cudaFuncGetAttributes(&fa, kernel));
-    if (fa.maxThreadsPerBlock < threads) {
-        set_error(std::string(name) + ": " + std::to_string(threads) + " threads requested, " +
-                  std::to_string(fa.maxThreadsPerBlock) + " possible with " + std::to_string(fa.numRegs) +
-                  " registers");
-        return VDW_ERR_UNSUPPORTED;
-    }
-    return VDW_OK;
-}
-
 template <int CN1, int CN2, int CN3>
 static int configure_sized(vdw_ctx* c) {
     const GridArgs& g = c->g;
     const int sp = (int)smem_plane(g);
-    const int sd = (int)smem_pencil_run(g, 3, DIV_COLS);
-    int rc = set_and_check(k_planes_inplace<CN1, CN3, true>, "k_planes_inplace", sp, PLANE_THREADS);
-    if (!rc) rc = set_and_check(k_planes_inplace<CN1, CN3, false>, "k_planes_inplace", sp, PLANE_THREADS);
-    if (!rc) rc = set_and_check(k_pencil_div<CN2>, "k_pencil_div", sd, 256);
+    const int sd = (int)smem_div(g);
+    int rc = planes_configure(c);
+    if (!rc) rc = set_and_check(k_pencil_div<CN2>, "k_pencil_div", sd, DIV_THREADS);
     if (!rc) rc = set_and_check(k_div_final<CN1, CN3>, "k_div_final", sp, PLANE_THREADS);
     if (!rc) rc = set_and_check(k_w_planes<CN1, CN3>, "k_w_planes", sp, PLANE_THREADS);
     if (rc) return rc;
@@ -851,60 +875,40 @@ static int configure_sized(vdw_ctx* c) {
 }
 
 int pipeline_configure(vdw_ctx* c) {
-    const GridArgs& g = c->g;
-    if (g.N1 == 180 && g.N2 == 180 && g.N3 == 72) return configure_sized<180, 180, 72>(c);
-    if (g.N1 == 256 && g.N2 == 256 && g.N3 == 96) return configure_sized<256, 256, 96>(c);
-    return configure_sized<0, 0, 0>(c);
+    return on_grid(c->g, [&](auto d) {
+        using D = decltype(d);
+        return configure_sized<D::N1, D::N2, D::N3>(c);
+    });
 }
 
 template <int CN1, int CN2, int CN3>
 static void launch_divergence(vdw_ctx* c, float* v, cudaStream_t s) {
     const GridArgs& g = c->g;
-    const size_t sd = smem_pencil_run(g, 3, DIV_COLS);
-    k_pencil_div<CN2><<<(g.ncols + DIV_COLS - 1) / DIV_COLS, 256, sd, s>>>(c->d_wspec, g, c->d_tw, DIV_COLS);
-    k_div_final<CN1, CN3><<<g.N2, PLANE_THREADS, smem_plane(g), s>>>(c->d_wspec, g, c->d_tw, v);
+    k_pencil_div<CN2><<<(g.ncols + DIV_COLS - 1) / DIV_COLS, DIV_THREADS, smem_div(g), s>>>(
+        c->d_wspec, g, c->d_tw + tw_off_y(g), c->d_tw + tw_off_swap(g));
+    k_div_final<CN1, CN3><<<g.N2, plane_block(c, g.N2), smem_plane(g), s>>>(c->d_wspec, g, c->d_tw, v);
 }
 
 template <int CN1, int CN3>
 static void launch_w_planes(vdw_ctx* c, const float* grad, cudaStream_t s) {
     const GridArgs& g = c->g;
-    k_w_planes<CN1, CN3><<<dim3(g.N2, 3), PLANE_THREADS, smem_plane(g), s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
+    k_w_planes<CN1, CN3><<<dim3(g.N2, 3), plane_block(c, 3LL * g.N2), smem_plane(g), s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
 }
 
 int pipeline_w_planes(vdw_ctx* c, const float* grad, cudaStream_t s) {
-    const GridArgs& g = c->g;
-    if (g.N1 == 180 && g.N2 == 180 && g.N3 == 72) launch_w_planes<180, 72>(c, grad, s);
-    else if (g.N1 == 256 && g.N2 == 256 && g.N3 == 96) launch_w_planes<256, 96>(c, grad, s);
-    else launch_w_planes<0, 0>(c, grad, s);
-    VDW_CUDA(cudaGetLastError());
-    return VDW_OK;
-}
-
-template <int CN1, int CN3>
-static void launch_planes_inplace(vdw_ctx* c, int nfields, bool inverse, cudaStream_t s) {
-    const GridArgs& g = c->g;
-    if (inverse)
-        k_planes_inplace<CN1, CN3, true><<<dim3(g.N2, nfields), PLANE_THREADS, smem_plane(g), s>>>(
-            c->d_spec, g, c->d_tw, c->bulk_planes, c->d_flags);
-    else
-        k_planes_inplace<CN1, CN3, false><<<dim3(g.N2, nfields), PLANE_THREADS, smem_plane(g), s>>>(
-            c->d_spec, g, c->d_tw, c->bulk_planes, c->d_flags);
-}
-
-int pipeline_planes_inplace(vdw_ctx* c, int nfields, bool inverse, cudaStream_t s) {
-    const GridArgs& g = c->g;
-    if (g.N1 == 180 && g.N2 == 180 && g.N3 == 72) launch_planes_inplace<180, 72>(c, nfields, inverse, s);
-    else if (g.N1 == 256 && g.N2 == 256 && g.N3 == 96) launch_planes_inplace<256, 96>(c, nfields, inverse, s);
-    else launch_planes_inplace<0, 0>(c, nfields, inverse, s);
+    on_grid(c->g, [&](auto d) {
+        using D = decltype(d);
+        launch_w_planes<D::N1, D::N3>(c, grad, s);
+    });
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;
 }
 
 int pipeline_divergence(vdw_ctx* c, float* v, cudaStream_t s) {
-    const GridArgs& g = c->g;
-    if (g.N1 == 180 && g.N2 == 180 && g.N3 == 72) launch_divergence<180, 180, 72>(c, v, s);
-    else if (g.N1 == 256 && g.N2 == 256 && g.N3 == 96) launch_divergence<256, 256, 96>(c, v, s);
-    else launch_divergence<0, 0, 0>(c, v, s);
+    on_grid(c->g, [&](auto d) {
+        using D = decltype(d);
+        launch_divergence<D::N1, D::N2, D::N3>(c, v, s);
+    });
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;
 }
@@ -922,12 +926,10 @@ int pipeline_energy_final(vdw_ctx* c, const double* epart, int nb0, int nb2, dou
 
 int pipeline_run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, float* w, cudaStream_t s,
                  int fd, int xc, const cudaEvent_t* slab_ready, int B) {
-    const GridArgs& g = c->g;
-    if (g.N1 == 180 && g.N2 == 180 && g.N3 == 72)
-        return run_sized<180, 180, 72>(c, n, grad, E, v, w, s, fd, xc, slab_ready, B);
-    if (g.N1 == 256 && g.N2 == 256 && g.N3 == 96)
-        return run_sized<256, 256, 96>(c, n, grad, E, v, w, s, fd, xc, slab_ready, B);
-    return run_sized<0, 0, 0>(c, n, grad, E, v, w, s, fd, xc, slab_ready, B);
+    return on_grid(c->g, [&](auto d) {
+        using D = decltype(d);
+        return run_sized<D::N1, D::N2, D::N3>(c, n, grad, E, v, w, s, fd, xc, slab_ready, B);
+    });
 }
 
 int pipeline_xc_final(vdw_ctx* c, double* E, cudaStream_t s) {

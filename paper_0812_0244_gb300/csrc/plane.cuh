@@ -1,7 +1,6 @@
-// Shared pieces of the transform kernels: block reductions, twiddle loads,
-// dispatch between the compile-time and runtime line transforms, and the
-// forward / inverse transform of one y plane (N3 rows of N1 reals <-> N3 x Nh
-// half spectrum) held in shared memory.
+// Shared pieces of the transform kernels: block reductions, twiddle loads, and
+// the forward / inverse transform of one y plane (N3 rows of N1 reals <->
+// N3 x Nh half spectrum) through shared memory.
 #pragma once
 #include <type_traits>
 
@@ -31,17 +30,11 @@ __device__ inline double block_sum(double v, double* red) {
     return s;
 }
 
-template <class W>
-__device__ __forceinline__ void load_twiddles(W* dst, const Tw* src, int n) {
-    for (int i = threadIdx.x; i < n; i += blockDim.x) tw_put(dst + i, src[i]);
-}
-// Shared-memory twiddles of a line length: the pass-ordered table of the
-// compile-time transforms when CN > 0 (CN == n), the plain table otherwise;
+// A line's second-group twiddle table (n - P1 entries) into shared memory;
 // W = Tw keeps the hi/lo pairs, W = float2 the FP32 values only.
-template <int CN, class W>
-__device__ __forceinline__ void load_line_twiddles(W* dst, const Tw* src, int n) {
-    if constexpr (CN > 0) ct_load_twiddles<CN>(dst, src);
-    else load_twiddles(dst, src, n);
+template <class W>
+__device__ __forceinline__ void load_twiddles(W* dst, const Tw* __restrict__ src, int n) {
+    for (int i = threadIdx.x; i < n; i += blockDim.x) tw_put(dst + i, src[i]);
 }
 
 // i / d for a small divisor (1 <= d < 256) and 0 <= i < 2^24 by one
@@ -58,61 +51,12 @@ __device__ __forceinline__ SmallDiv small_div(int d) {
     return s;
 }
 __device__ __forceinline__ int sdiv(int i, SmallDiv s) { return s.d == 1 ? i : (int)__umulhi((unsigned)i, s.m); }
-
-// 8-byte asynchronous copy global -> shared memory (cp.async), zero-filled
-// instead when !valid (src is then not read; it must still be a mapped
-// address).  A thread issues all its copies without waiting on any;
-// cp_async_wait_all then waits for the thread's own copies.
-__device__ __forceinline__ void cp_async8(void* smem_dst, const void* src, bool valid) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(d), "l"(src), "r"(valid ? 8 : 0) : "memory");
+// the same with the divisor known at compile time when C > 0
+template <int C>
+__device__ __forceinline__ int cdiv(int i, SmallDiv s) {
+    if constexpr (C > 0) return (int)((unsigned)i / (unsigned)C);
+    else return sdiv(i, s);
 }
-// 4-byte form of the same
-__device__ __forceinline__ void cp_async4(void* smem_dst, const void* src, bool valid) {
-    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(valid ? 4 : 0) : "memory");
-}
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
-
-// ---------------------------------------------------------------------------
-// line-transform dispatch: compile-time length when CN > 0
-// ---------------------------------------------------------------------------
-// the Nh columns of a plane (element stride Nh), several columns per warp for short lines
-template <int CN, bool INV, int MAXR = 16, class W>
-__device__ __forceinline__ void columns_fft(float2* plane, int Nh, const LinePlan& pl, const W* tw) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if constexpr (CN > 0) {
-        constexpr int L = ct_lines_per_warp(CN, MAXR);
-        const int full = (Nh / L) * L;
-        for (int col = warp * L; col < full; col += nw * L) ct_fft<CN, L, INV, MAXR>(plane + col, Nh, 1, tw, lane);
-        for (int col = full + warp; col < Nh; col += nw) ct_fft<CN, 1, INV, MAXR>(plane + col, Nh, 1, tw, lane);
-    } else {
-        for (int col = warp; col < Nh; col += nw) line_fft<INV>(plane + col, Nh, pl, tw, lane);
-    }
-}
-
-// lines of length N2 (pencils) at a stride of ls values (ls = N2: contiguous),
-// several lines per warp for short lines
-template <int CN, bool INV, class W>
-__device__ __forceinline__ void pencils_fft(float2* lines, int nlines, int N2, const LinePlan& pl, const W* tw,
-                                            int ls = 0) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    if (ls == 0) ls = N2;
-    if constexpr (CN > 0) {
-        constexpr int L = ct_lines_per_warp(CN);
-        const int full = (nlines / L) * L;
-        for (int l = warp * L; l < full; l += nw * L) ct_fft<CN, L, INV>(lines + l * ls, 1, ls, tw, lane);
-        for (int l = full + warp; l < nlines; l += nw) ct_fft<CN, 1, INV>(lines + l * ls, 1, 0, tw, lane);
-    } else {
-        for (int l = warp; l < nlines; l += nw) line_fft<INV>(lines + l * ls, 1, pl, tw, lane);
-    }
-}
-
-// Line stride of the pencil kernels' shared-memory lines [field][column][y]:
-// the staging loops give the 16 lanes of a half-warp 8 columns x 2 rows, at
-// (column S + y) float2 values; with S = 2 (mod 16) those are the 16
-// distinct 8-byte banks.
-__host__ __device__ __forceinline__ int pencil_stride(int N2) { return N2 + ((2 - N2) % 16 + 16) % 16; }
 
 // ---------------------------------------------------------------------------
 // plane helpers (one y plane, N3 rows of N1 reals <-> N3 x Nh half spectrum)
@@ -160,60 +104,57 @@ __device__ __forceinline__ void flat_point(long long i, const GridArgs& g, int& 
 // This is the float offset, within its plane, of real point (x, z = 2j + s).
 __device__ __forceinline__ int packed_offset(int x, int j, int s, int Nh) { return 4 * j * Nh + 2 * x + s; }
 
-// Rows of a plane (complex row j holds real rows 2j and 2j+1) through the
-// x transform, several rows per warp at compile-time lengths; each row is
-// then untangled into the two half spectra (forward), or tangled before the
-// transform (inverse).
-template <int CN1, bool INV, int MAXR = 16, class W>
-__device__ __forceinline__ void plane_rows(float2* plane, const GridArgs& g, const W* tw1) {
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const int nrows = g.N3 / 2, rs = 2 * g.Nh;
+// ---------------------------------------------------------------------------
+// y lines (pencils)
+// ---------------------------------------------------------------------------
+// Shared-memory lines of the pencil kernels: point k1 + P1 k2 of a line sits
+// at k1 + (P1 | 1) k2, a line takes pencil_stride values, and the C lines of
+// a field C pencil_stride values plus a pad.  The stride is 2 (mod 16): the
+// lanes that take 8 columns and 2 neighbouring points of each then hit the
+// 16 distinct 8-byte banks, and the field pads do the same for lanes that
+// take 4 fields and 4 neighbouring points.
+__host__ __device__ __forceinline__ int pencil_stride(const LinePlan& p) {
+    const int n = (p.P1 | 1) * p.P2;
+    return n + ((2 - n) % 16 + 16) % 16;
+}
+
+// ---------------------------------------------------------------------------
+// one y plane
+// ---------------------------------------------------------------------------
+// Shared memory of a plane transform: N3/2 rows, row j holding the complex
+// row j = (real row 2j) + i (real row 2j + 1), and later the half spectra of
+// those two rows.  Element k of a row sits at slot(k) = k + (k / P)(stride - P)
+// with a run length P and stride = P or P + 1 (padded so that steps of P
+// elements change the bank); a row takes an odd number of slots, so that
+// lanes on consecutive rows hit distinct banks.  Half spectra: real row 2j's
+// value at kx takes slot(kx) of row j, real row 2j + 1's takes slot(N1 - kx)
+// (two extra slots at the row's end for kx = 0 and N1/2), so that every pass
+// writes where the same thread read and no pass needs a second buffer.
+struct PlaneGeo {
+    int run, stride;  // slot(k) = k + (k / run)(stride - run)
+    int len;          // slots of a row before the two extra ones
+    int S;            // slots of a row
+};
+// forward: run P1 (the row transform's first group stores steps of P1);
+// inverse: run P2 (its second group reads steps of P2).  Without the pads
+// where they would not fit in shared memory (wide planes).
+__host__ __device__ constexpr PlaneGeo plane_geo(int P1, int P2, bool inverse, bool pad) {
+    const int run = inverse ? P2 : P1;
+    const int stride = pad ? (run | 1) : run;
+    const int len = stride * (inverse ? P1 : P2);
+    return PlaneGeo{run, stride, len, pad ? ((len + 2) | 1) : len + 2};
+}
+template <int CN1, bool INVERSE>
+__device__ __forceinline__ PlaneGeo geo_of(const GridArgs& g) {
     if constexpr (CN1 > 0) {
-        constexpr int L = ct_lines_per_warp(CN1, MAXR);
-        const int full = (nrows / L) * L;
-        for (int row = warp * L; row < full; row += nw * L) {
-            float2* p = plane + row * rs;
-            if (INV)
-                for (int l = 0; l < L; ++l) c2r_tangle(p + l * rs, g.N1, lane);
-            ct_fft<CN1, L, INV, MAXR>(p, 1, rs, tw1, lane);
-            if (!INV)
-                for (int l = 0; l < L; ++l) r2c_untangle(p + l * rs, g.N1, lane);
-        }
-        for (int row = full + warp; row < nrows; row += nw) {
-            float2* p = plane + row * rs;
-            if (INV) c2r_tangle(p, g.N1, lane);
-            ct_fft<CN1, 1, INV, MAXR>(p, 1, 0, tw1, lane);
-            if (!INV) r2c_untangle(p, g.N1, lane);
-        }
+        constexpr PlaneGeo p = plane_geo(CtLine<CN1>::G1::P, CtLine<CN1>::G2::P, INVERSE, true);
+        return p;
     } else {
-        for (int row = warp; row < nrows; row += nw) {
-            float2* p = plane + row * rs;
-            if (INV) c2r_tangle(p, g.N1, lane);
-            line_fft<INV>(p, 1, g.p1, tw1, lane);
-            if (!INV) r2c_untangle(p, g.N1, lane);
-        }
+        return plane_geo(g.p1.P1, g.p1.P2, INVERSE, INVERSE ? g.pad_inv : g.pad_fwd);
     }
 }
-
-// Forward: packed real rows -> half spectrum (x R2C, then z C2C).
-template <int CN1, int CN3, int MAXR = 16, class W>
-__device__ void plane_forward(float2* plane, const GridArgs& g, const W* tw1, const W* tw3) {
-    plane_rows<CN1, false, MAXR>(plane, g, tw1);
-    __syncthreads();
-    columns_fft<CN3, false, MAXR>(plane, g.Nh, g.p3, tw3);
-    __syncthreads();
-}
-
-// Inverse: half spectrum -> packed real rows (z C2C inverse, then x C2R), unscaled.
-template <int CN1, int CN3, int MAXR = 16, class W>
-__device__ void plane_inverse(float2* plane, const GridArgs& g, const W* tw1, const W* tw3) {
-    columns_fft<CN3, true, MAXR>(plane, g.Nh, g.p3, tw3);
-    __syncthreads();
-    plane_rows<CN1, true, MAXR>(plane, g, tw1);
-    __syncthreads();
-}
-
-constexpr int PLANE_THREADS = 256;  // threads of the plane kernels (P1, P5)
+// position of (z, kx): even and odd real rows of a complex row at slots se, so
+__device__ __forceinline__ int zpos(int z, int S, int se, int so) { return (z >> 1) * S + ((z & 1) ? so : se); }
 
 // Twiddles in shared memory after n float2 values, on a 16-byte boundary.
 __host__ __device__ __forceinline__ size_t tw_offset(size_t n) { return (n + 1) & ~(size_t)1; }
@@ -224,5 +165,237 @@ __device__ __forceinline__ W* twiddles_after(float2* base, size_t n) {
 // The twiddle kind of a transform: hi/lo pairs (EXACT) or FP32 values.
 template <bool EXACT>
 using TwOf = typename std::conditional<EXACT, Tw, float2>::type;
+
+// Forward transform of one plane: complex rows from ld(row, x) (R2C along x
+// of the two real rows in each, C2C along z), results to st(kz, kx, value).
+// Each phase is one register pass over all lines of the plane; a block-wide
+// barrier separates the phases.  The x passes' first group takes neighbouring
+// x in neighbouring lanes (the loads), the second neighbouring rows (one
+// twiddle for all lanes), the z passes neighbouring kx (the same, and the
+// stores).
+template <int CN1, int CN3, class W, class LD, class ST>
+__device__ __forceinline__ void plane_forward(float2* sm, const GridArgs& g, const Tw* __restrict__ tw, LD ld, ST st) {
+    const int N1 = CN1 > 0 ? CN1 : g.N1, N3 = CN3 > 0 ? CN3 : g.N3;
+    const int Nh = N1 / 2 + 1, nr = N3 / 2;
+    const PlaneGeo G = geo_of<CN1, false>(g);
+    const int S = G.S;
+    const int P1 = G.run, Q1 = CN3 > 0 ? CtLine<CN3>::G1::P : g.p3.P1;
+    W* tw1 = twiddles_after<W>(sm, (size_t)nr * S);
+    W* tw3 = tw1 + (N1 - P1);
+    load_twiddles(tw1, tw, N1 - P1);
+    load_twiddles(tw3, tw + g.N1 + g.N2, N3 - Q1);
+    const int t0 = threadIdx.x, nt = blockDim.x;
+    on_first<CN1, false>(g.p1, [&](auto tag) {
+        using R = decltype(tag);
+        constexpr int CM = CN1 > 0 ? CN1 / R::P : 0;
+        const int m = CN1 > 0 ? CM : g.p1.P2;
+        const SmallDiv dm = small_div(m);
+        for (int it = t0; it < nr * m; it += nt) {
+            const int row = cdiv<CM>(it, dm), j = it - row * m;
+            float2 v[R::P];
+#pragma unroll
+            for (int q = 0; q < R::P; ++q) v[q] = ld(row, j + q * m);
+            group_fft<R, false, true, W>(v, (const W*)nullptr, 1);
+            float2* d = sm + row * S + G.stride * j;
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) d[R::digit(i)] = v[i];
+        }
+    });
+    __syncthreads();
+    constexpr int CR = CN3 > 0 ? CN3 / 2 : 0;
+    const SmallDiv dr = small_div(nr);
+    on_second<CN1>(g.p1, [&](auto tag) {
+        using R = decltype(tag);
+        for (int it = t0; it < P1 * nr; it += nt) {
+            const int k1 = cdiv<CR>(it, dr), row = it - k1 * nr;
+            float2* d = sm + row * S + k1;
+            float2 v[R::P];
+#pragma unroll
+            for (int q = 0; q < R::P; ++q) v[q] = d[q * G.stride];
+            group_fft<R, false, false, W>(v, tw1 + k1, P1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) d[R::digit(i) * G.stride] = v[i];
+        }
+    });
+    __syncthreads();
+    // the two half spectra of each complex row: A = (Z_k + conj Z_{-k})/2,
+    // B = -i (Z_k - conj Z_{-k})/2
+    const SmallDiv dP = small_div(G.run);
+    for (int it = t0; it < Nh * nr; it += nt) {
+        const int k = cdiv<CR>(it, dr), row = it - k * nr;
+        const int km = k == 0 ? 0 : N1 - k;
+        float2* d = sm + row * S;
+        const int sk = k + sdiv(k, dP) * (G.stride - G.run), sm_ = km + sdiv(km, dP) * (G.stride - G.run);
+        const float2 zk = d[sk], zm = d[sm_];
+        d[sk] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
+        d[k == 0 ? G.len : (k == km ? G.len + 1 : sm_)] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+    }
+    __syncthreads();
+    constexpr int CH = CN1 > 0 ? CN1 / 2 + 1 : 0;
+    const SmallDiv dh = small_div(Nh);
+    const auto slots = [&](int kx, int& se, int& so) {
+        const int km = N1 - kx;
+        se = kx + sdiv(kx, dP) * (G.stride - G.run);
+        so = kx == 0 ? G.len : (kx == km ? G.len + 1 : km + sdiv(km, dP) * (G.stride - G.run));
+    };
+    on_first<CN3, false>(g.p3, [&](auto tag) {
+        using R = decltype(tag);
+        const int m = CN3 > 0 ? CN3 / R::P : g.p3.P2;
+        for (int it = t0; it < m * Nh; it += nt) {
+            const int j = cdiv<CH>(it, dh), kx = it - j * Nh;
+            int se, so;
+            slots(kx, se, so);
+            float2* d0 = sm + zpos(j, S, se, so);
+            float2* d1 = sm + zpos(j + m, S, se, so);
+            float2 v[R::P];
+#pragma unroll
+            for (int q = 0; q < R::P; ++q) v[q] = (q & 1 ? d1 : d0)[(q >> 1) * m * S];
+            group_fft<R, false, true, W>(v, (const W*)nullptr, 1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) (R::digit(i) & 1 ? d1 : d0)[(R::digit(i) >> 1) * m * S] = v[i];
+        }
+    });
+    __syncthreads();
+    on_second<CN3>(g.p3, [&](auto tag) {
+        using R = decltype(tag);
+        for (int it = t0; it < Q1 * Nh; it += nt) {
+            const int k1 = cdiv<CH>(it, dh), kx = it - k1 * Nh;
+            int se, so;
+            slots(kx, se, so);
+            const float2* d0 = sm + zpos(k1 * R::P, S, se, so);
+            const float2* d1 = sm + zpos(k1 * R::P + 1, S, se, so);
+            float2 v[R::P];
+#pragma unroll
+            for (int q = 0; q < R::P; ++q) v[q] = (q & 1 ? d1 : d0)[(q >> 1) * S];
+            group_fft<R, false, false, W>(v, tw3 + k1, Q1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) st(k1 + Q1 * R::digit(i), kx, v[i]);
+        }
+    });
+}
+
+// Inverse transform of one plane (unscaled): half spectrum from ld(kz, kx),
+// C2C along z, C2R along x of the two real rows of each complex row (the
+// imaginary parts at kx = 0 and N1/2 are dropped, as a complex-to-real
+// transform does), st(row, x, {real row 2 row, real row 2 row + 1}).
+template <int CN1, int CN3, class W, class LD, class ST>
+__device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, const Tw* __restrict__ tw, LD ld, ST st) {
+    const int N1 = CN1 > 0 ? CN1 : g.N1, N3 = CN3 > 0 ? CN3 : g.N3;
+    const int Nh = N1 / 2 + 1, nr = N3 / 2;
+    const PlaneGeo G = geo_of<CN1, true>(g);
+    const int S = G.S;
+    const int P1 = CN1 > 0 ? CtLine<CN1>::G1::P : g.p1.P1, Q1 = CN3 > 0 ? CtLine<CN3>::G1::P : g.p3.P1;
+    W* tw1 = twiddles_after<W>(sm, (size_t)nr * S);
+    W* tw3 = tw1 + (N1 - P1);
+    load_twiddles(tw1, tw, N1 - P1);
+    load_twiddles(tw3, tw + g.N1 + g.N2, N3 - Q1);
+    const int t0 = threadIdx.x, nt = blockDim.x;
+    constexpr int CH = CN1 > 0 ? CN1 / 2 + 1 : 0;
+    const SmallDiv dh = small_div(Nh), dP = small_div(G.run);
+    const auto slots = [&](int kx, int& se, int& so) {
+        const int km = N1 - kx;
+        se = kx + sdiv(kx, dP) * (G.stride - G.run);
+        so = kx == 0 ? G.len : (kx == km ? G.len + 1 : km + sdiv(km, dP) * (G.stride - G.run));
+    };
+    on_first<CN3, false>(g.p3, [&](auto tag) {
+        using R = decltype(tag);
+        const int m = CN3 > 0 ? CN3 / R::P : g.p3.P2;
+        for (int it = t0; it < m * Nh; it += nt) {
+            const int j = cdiv<CH>(it, dh), kx = it - j * Nh;
+            float2 v[R::P];
+#pragma unroll
+            for (int q = 0; q < R::P; ++q) v[q] = ld(j + q * m, kx);
+            int se, so;
+            slots(kx, se, so);
+            float2* d0 = sm + zpos(R::P * j, S, se, so);
+            float2* d1 = sm + zpos(R::P * j + 1, S, se, so);
+            group_fft<R, true, true, W>(v, (const W*)nullptr, 1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) (R::digit(i) & 1 ? d1 : d0)[(R::digit(i) >> 1) * S] = v[i];
+        }
+    });
+    __syncthreads();
+    on_second<CN3>(g.p3, [&](auto tag) {
+        using R = decltype(tag);
+        for (int it = t0; it < Q1 * Nh; it += nt) {
+            const int k1 = cdiv<CH>(it, dh), kx = it - k1 * Nh;
+            int se, so;
+            slots(kx, se, so);
+            float2* d0 = sm + zpos(k1, S, se, so);
+            float2* d1 = sm + zpos(k1 + Q1, S, se, so);
+            float2 v[R::P];
+#pragma unroll
+            for (int q = 0; q < R::P; ++q) v[q] = (q & 1 ? d1 : d0)[(q >> 1) * Q1 * S];
+            group_fft<R, true, false, W>(v, tw3 + k1, Q1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) (R::digit(i) & 1 ? d1 : d0)[(R::digit(i) >> 1) * Q1 * S] = v[i];
+        }
+    });
+    __syncthreads();
+    // Z = A + i B on the full circle from the two half spectra
+    constexpr int CR = CN3 > 0 ? CN3 / 2 : 0;
+    const SmallDiv dr = small_div(nr);
+    for (int it = t0; it < Nh * nr; it += nt) {
+        const int k = cdiv<CR>(it, dr), row = it - k * nr;
+        int se, so;
+        slots(k, se, so);
+        float2* d = sm + row * S;
+        float2 a = d[se], b = d[so];
+        const bool edge = k == 0 || 2 * k == N1;
+        if (edge) a.y = b.y = 0.f;
+        d[se] = make_float2(a.x - b.y, a.y + b.x);
+        if (!edge) d[so] = make_float2(a.x + b.y, b.x - a.y);
+    }
+    __syncthreads();
+    on_first<CN1, false>(g.p1, [&](auto tag) {
+        using R = decltype(tag);
+        const int m = CN1 > 0 ? CN1 / R::P : g.p1.P2;
+        for (int it = t0; it < m * nr; it += nt) {
+            const int j = cdiv<CR>(it, dr), row = it - j * nr;
+            float2* d = sm + row * S + j;
+            float2 v[R::P];
+#pragma unroll
+            for (int q = 0; q < R::P; ++q) v[q] = d[q * G.stride];
+            group_fft<R, true, true, W>(v, (const W*)nullptr, 1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) d[R::digit(i) * G.stride] = v[i];
+        }
+    });
+    __syncthreads();
+    const SmallDiv dk = small_div(P1);
+    constexpr int CK = CN1 > 0 ? CtLine<CN1>::G1::P : 0;
+    on_second<CN1>(g.p1, [&](auto tag) {
+        using R = decltype(tag);
+        for (int it = t0; it < P1 * nr; it += nt) {
+            const int row = cdiv<CK>(it, dk), k1 = it - row * P1;
+            const float2* d = sm + row * S + k1 * G.stride;
+            float2 v[R::P];
+#pragma unroll
+            for (int q = 0; q < R::P; ++q) v[q] = d[q];
+            group_fft<R, true, false, W>(v, tw1 + k1, P1);
+#pragma unroll
+            for (int i = 0; i < R::P; ++i) st(row, k1 + P1 * R::digit(i), v[i]);
+        }
+    });
+}
+
+// Threads of the plane kernels at most; two such blocks (64 registers per
+// thread) or more smaller ones per SM, plane_block (pipeline.cu).
+constexpr int PLANE_THREADS = 512;
+
+// f(Dims) with the line kinds of a plan: the compile-time grids, else per
+// plane (x and z together) and per y line the run-time kind.
+template <int N1_, int N2_, int N3_>
+struct Dims {
+    static constexpr int N1 = N1_, N2 = N2_, N3 = N3_;
+};
+template <class F>
+auto on_grid(const GridArgs& g, F&& f) {
+    if (sized_grid(g.N1, g.N2, g.N3)) return g.N1 == 180 ? f(Dims<180, 180, 72>{}) : f(Dims<256, 256, 96>{});
+    const auto small = [](const LinePlan& l) { return l.P1 <= 16 && l.P2 <= 16; };
+    if (small(g.p1) && small(g.p3))
+        return small(g.p2) ? f(Dims<ANY16, ANY16, ANY16>{}) : f(Dims<ANY16, ANY, ANY16>{});
+    return small(g.p2) ? f(Dims<ANY, ANY16, ANY>{}) : f(Dims<ANY, ANY, ANY>{});
+}
 
 }  // namespace vdw
