@@ -104,7 +104,6 @@ struct LearnedArgs {
     const float* b3;        // [M]
     const uint16_t* w2f;    // forward operand W2 [H out][H in]
     const uint16_t* w3f;    // forward operand W3 [16 (M padded)][H]
-    const float* w2r;       // W2 bf16-rounded values, row-major [H][H] (CUDA-core kernels)
     const float* w3r;       // W3 bf16-rounded values, row-major [M][H]
     const float4* knots;    // [J-1][P]: cubic coefficients in t of the Catmull-Rom piece on interval j
     int* err;               // set when a tensor-core wait gives up

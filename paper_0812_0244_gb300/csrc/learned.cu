@@ -22,7 +22,7 @@
 //   then the plain method's divergence kernels (P4, P5).
 //
 // Training kernels: the parameter gradient of E through the network
-// (k_learned_param_grad, CUDA cores, FP32 sums into FP64), a regression
+// (k_learned_param_grad, tensor cores, FP32 sums into FP64), a regression
 // gradient for fitting the channel weights to targets, and an Adam step.
 // Utilities: the plain cardinal weights p_a(q) and the spectral gradient.
 #include "plane.cuh"
@@ -46,7 +46,7 @@ constexpr int L_THREADS = 256;    // two warpgroups (channel kernel)
 constexpr int L_NET_WG = 3;       // warpgroups of the network kernel
 constexpr int L_NET_THREADS = 128 * L_NET_WG;
 constexpr int L_TILE = 128;       // points per warpgroup tile
-constexpr int L_MAXJ = 256;       // knots held in shared memory by the knot-gradient bins
+constexpr int L_MAXJ = 256;       // knots at most
 
 // ---------------------------------------------------------------------------
 // device helpers
@@ -318,10 +318,11 @@ __device__ bool mlp_forward(MlpShared* S, MlpWG* W, MlpCtl* ctl, int wg, int r, 
 // the first tangent into [64, 128); after their epilogue the second tangent
 // reuses [64, 128) while the layer-2 pre-activation stays in [0, 64) for its
 // SiLU derivative.  Layer 3 then writes [0, 16), [16, 32), [32, 48).
-// Returns o (8 outputs) and J1, J2 (d o / d x1, d o / d x2).
+// Returns o (8 outputs) and J1, J2 (d o / d x1, d o / d x2).  Without JAC the
+// tangents are left out (the outputs are the same to the bit).
 // overlap() runs on every thread of the warpgroup while the first layer-2
 // batch is in flight (work that does not depend on the network).
-template <class Overlap>
+template <bool JAC, class Overlap>
 __device__ bool mlp_forward_jac(MlpShared* S, MlpWG3* W, MlpCtl* ctl, int wg, int r, uint32_t& phase, float x1,
                                 float x2, float* o, float* J1, float* J2, int* err, Overlap overlap) {
 #pragma unroll
@@ -337,13 +338,15 @@ __device__ bool mlp_forward_jac(MlpShared* S, MlpWG3* W, MlpCtl* ctl, int wg, in
             t2[q] = sp * S->w1[2 * j + 1];
         }
         store8_bf16(W->A[0] + tc::kmaj(r, 8 * c, LRN_H), h);
-        store8_bf16(W->A[1] + tc::kmaj(r, 8 * c, LRN_H), t1);
-        store8_bf16(W->A[2] + tc::kmaj(r, 8 * c, LRN_H), t2);
+        if (JAC) {
+            store8_bf16(W->A[1] + tc::kmaj(r, 8 * c, LRN_H), t1);
+            store8_bf16(W->A[2] + tc::kmaj(r, 8 * c, LRN_H), t2);
+        }
     }
     {
         const uint16_t* As[2] = {W->A[0], W->A[1]};
         const uint32_t cols[2] = {0, 64};
-        wg_mma_issue(ctl, wg, r, As, cols, 2, S->w2f, LRN_H, LRN_H);
+        wg_mma_issue(ctl, wg, r, As, cols, JAC ? 2 : 1, S->w2f, LRN_H, LRN_H);
         overlap();
         if (!wg_mma_wait(ctl, wg, phase, err)) return false;
     }
@@ -351,17 +354,29 @@ __device__ bool mlp_forward_jac(MlpShared* S, MlpWG3* W, MlpCtl* ctl, int wg, in
     for (int c = 0; c < LRN_H / 16; ++c) {
         float z[16], d1[16];
         tc::tmem_ld16(lane_addr(ctl, wg, 16 * c), z);
-        tc::tmem_ld16(lane_addr(ctl, wg, 64 + 16 * c), d1);
+        if (JAC) tc::tmem_ld16(lane_addr(ctl, wg, 64 + 16 * c), d1);
 #pragma unroll
         for (int q = 0; q < 16; ++q) {
             float sp;
             silu_both(z[q] + S->b2[16 * c + q], z[q], sp);
-            d1[q] *= sp;
+            if (JAC) d1[q] *= sp;
         }
         store8_bf16(W->A[0] + tc::kmaj(r, 16 * c, LRN_H), z);
         store8_bf16(W->A[0] + tc::kmaj(r, 16 * c + 8, LRN_H), z + 8);
-        store8_bf16(W->A[1] + tc::kmaj(r, 16 * c, LRN_H), d1);
-        store8_bf16(W->A[1] + tc::kmaj(r, 16 * c + 8, LRN_H), d1 + 8);
+        if (JAC) {
+            store8_bf16(W->A[1] + tc::kmaj(r, 16 * c, LRN_H), d1);
+            store8_bf16(W->A[1] + tc::kmaj(r, 16 * c + 8, LRN_H), d1 + 8);
+        }
+    }
+    if constexpr (!JAC) {
+        const uint16_t* As[1] = {W->A[0]};
+        const uint32_t cols[1] = {64};
+        if (!wg_mma_n(ctl, wg, r, phase, As, cols, 1, S->w3f, LRN_H, LRN_N3, err)) return false;
+        float v[16];
+        tc::tmem_ld16(lane_addr(ctl, wg, 64), v);
+#pragma unroll
+        for (int m = 0; m < LRN_M; ++m) o[m] = v[m] + S->b3[m];
+        return true;
     }
     {
         // the first tangent's columns are read (tcgen05.wait::ld in tmem_ld16)
@@ -406,7 +421,6 @@ __global__ void k_learned_prepare(const float* __restrict__ flat, LearnedArgs la
     float* b1 = const_cast<float*>(la.b1);
     float* b2 = const_cast<float*>(la.b2);
     float* b3 = const_cast<float*>(la.b3);
-    float* w2r = const_cast<float*>(la.w2r);
     float* w3r = const_cast<float*>(la.w3r);
     uint16_t* w2f = const_cast<uint16_t*>(la.w2f);
     uint16_t* w3f = const_cast<uint16_t*>(la.w3f);
@@ -422,7 +436,6 @@ __global__ void k_learned_prepare(const float* __restrict__ flat, LearnedArgs la
     for (int i = t; i < LRN_H * LRN_H; i += nt) {
         const int o = i / LRN_H, j = i % LRN_H;  // W2[o][j]: output o, input j
         const float x = flat[LRN_OFF_W2 + i];
-        w2r[i] = bf16r(x);
         w2f[tc::kmaj(o, j, LRN_H)] = bfu(x);
     }
     for (int i = t; i < LRN_N3 * LRN_H; i += nt) {
@@ -461,6 +474,9 @@ __global__ void k_learned_prepare(const float* __restrict__ flat, LearnedArgs la
 //   lw[M + m] = n (dw_m/d|grad n|)/|grad n|
 //   lw[2M], lw[2M + 1] = the Delta E derivatives.
 // Delta E partial sums per block.
+// Training calls it without the Jacobian (JAC false, lw null): its parameter
+// gradient needs theta alone, 470 -> 270 us at 180 x 180 x 72.
+template <bool JAC>
 __global__ void __launch_bounds__(L_NET_THREADS, 1)
     k_learned_net(const float* __restrict__ n, const float* __restrict__ grad, GridArgs g, PointParams P,
                   LearnedArgs la, float* __restrict__ specf, double* __restrict__ epart,
@@ -523,7 +539,11 @@ __global__ void __launch_bounds__(L_NET_THREADS, 1)
             }
         };
         float o[LRN_M], J1[LRN_M], J2[LRN_M];
-        if (!mlp_forward_jac(S, W, &ctl, wg, r, phase, ok ? f.x1 : 0.f, ok ? f.x2 : 0.f, o, J1, J2, la.err, qwork))
+        if (!JAC) {
+#pragma unroll
+            for (int m = 0; m < LRN_M; ++m) J1[m] = J2[m] = 0.f;
+        }
+        if (!mlp_forward_jac<JAC>(S, W, &ctl, wg, r, phase, ok ? f.x1 : 0.f, ok ? f.x2 : 0.f, o, J1, J2, la.err, qwork))
             break;
         if (in) {
             float* dst = specf + 2LL * y * g.ncols + packed_offset(x, j, z & 1, g.Nh);
@@ -735,27 +755,28 @@ __global__ void __launch_bounds__(LOOKUP_THREADS, 3) k_learned_lookup(const floa
 // (contract.cu) with the knot table.  This form also accumulates
 //   dE/dK_p(k_i) = sum_G 1/2 Omega w_G (2 - delta_ab) Re(conj th_a th_b) c_i(|G|)
 // for the four Catmull-Rom weights c_i of the knots around |G| (Eq. Eoffk
-// differentiated through the interpolation), in shared-memory bins [P][J].
-// In |G| order the 32 points of a warp nearly always share their interval:
-// the warp then sums its contributions first and one lane adds them.
-__device__ __forceinline__ float warp_sum_f(float v) {
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    return v;
-}
+// differentiated through the interpolation).  In |G| order a block's 128
+// points lie in a few runs of equal interval (one or two, save for the blocks
+// at the smallest |G|): the block puts the 36 pair products and the four
+// weights of every point into shared memory, and for each run 36 threads (one
+// pair each, in GK_PARTS parts of the run) sum the products of its points
+// with the four weights; the totals go to gK by FP64 atomics.  (Summing each
+// product over the warp by shuffles, into bins of all 36 x J knots per block,
+// took 495 us at 180 x 180 x 72 against 73.)
+constexpr int GK_PARTS = SORTED_BLOCK / LRN_P;  // 3
+constexpr int GK_LD = LRN_P + 1;
 
-__global__ void __launch_bounds__(SORTED_BLOCK) k_learned_contract_gradk(float4* __restrict__ Q, long long qstride,
-                                                                       const float* __restrict__ gs, LearnedArgs la,
-                                                                       float invN, double* __restrict__ epart,
-                                                                       double* __restrict__ gK, float halfOmega) {
+__global__ void __launch_bounds__(SORTED_BLOCK, 6) k_learned_contract_gradk(
+    float4* __restrict__ Q, long long qstride, const float* __restrict__ gs, LearnedArgs la, float invN,
+    double* __restrict__ epart, double* __restrict__ gK, float halfOmega) {
     constexpr int NQ = LRN_M;
-    extern __shared__ float bins[];  // [P][J]
     __shared__ double red[32];
-    const int J = la.J;
-    for (int i = threadIdx.x; i < LRN_P * J; i += blockDim.x) bins[i] = 0.f;
-    __syncthreads();
-    const long long r = (long long)blockIdx.x * SORTED_BLOCK + threadIdx.x;
-    const int lane = threadIdx.x & 31;
+    __shared__ float rv_s[SORTED_BLOCK * GK_LD];
+    __shared__ float4 w_s[SORTED_BLOCK];
+    __shared__ int j_s[SORTED_BLOCK];
+    __shared__ float part[GK_PARTS][LRN_P][4];
+    const int J = la.J, tid = threadIdx.x;
+    const long long r = (long long)blockIdx.x * SORTED_BLOCK + tid;
     float2 th[NQ];
 #pragma unroll
     for (int q = 0; q < NQ / 4; ++q) {
@@ -772,13 +793,9 @@ __global__ void __launch_bounds__(SORTED_BLOCK) k_learned_contract_gradk(float4*
     const float t = sk - (float)j;
     const float4* cf = la.knots + (long long)j * LRN_P;
     // Catmull-Rom weights of the knots j-1 .. j+2
-    const float wm1 = 0.5f * t * (t * (2.f - t) - 1.f), w0 = 1.f + t * t * (1.5f * t - 2.5f);
-    const float w1 = 0.5f * t * (1.f + t * (4.f - 3.f * t)), w2 = 0.5f * t * t * (t - 1.f);
-    // knots of the four weights: the knot before k = 0 mirrors knot 1; past the
-    // last knot the linear extrapolation 2 K_{J-1} - K_{J-2}
-    const int km1 = j == 0 ? 1 : j - 1;
-    const bool tail = j + 2 > J - 1;
-    const bool uni = __all_sync(0xffffffffu, j == __shfl_sync(0xffffffffu, j, 0));
+    w_s[tid] = make_float4(0.5f * t * (t * (2.f - t) - 1.f), 1.f + t * t * (1.5f * t - 2.5f),
+                           0.5f * t * (1.f + t * (4.f - 3.f * t)), 0.5f * t * t * (t - 1.f));
+    j_s[tid] = j;
     float2 u[NQ];
 #pragma unroll
     for (int a = 0; a < NQ; ++a) u[a] = make_float2(0.f, 0.f);
@@ -795,40 +812,15 @@ __global__ void __launch_bounds__(SORTED_BLOCK) k_learned_contract_gradk(float4*
                 u[b].x = fmaf(phi, th[a].x, u[b].x);
                 u[b].y = fmaf(phi, th[a].y, u[b].y);
             }
-            const float rv = halfOmega * wgt * (b != a ? 2.f : 1.f) * (th[a].x * th[b].x + th[a].y * th[b].y);
-            float* bp = bins + p * J;
-            if (uni) {
-                const float s0 = warp_sum_f(wm1 * rv), s1 = warp_sum_f(w0 * rv);
-                const float s2 = warp_sum_f(w1 * rv), s3 = warp_sum_f(w2 * rv);
-                if (lane == 0) {
-                    atomicAdd(&bp[km1], s0);
-                    atomicAdd(&bp[j], s1);
-                    atomicAdd(&bp[j + 1], s2);
-                    if (!tail) {
-                        atomicAdd(&bp[j + 2], s3);
-                    } else {
-                        atomicAdd(&bp[J - 1], 2.f * s3);
-                        atomicAdd(&bp[J - 2], -s3);
-                    }
-                }
-            } else {
-                atomicAdd(&bp[km1], wm1 * rv);
-                atomicAdd(&bp[j], w0 * rv);
-                atomicAdd(&bp[j + 1], w1 * rv);
-                if (!tail) {
-                    atomicAdd(&bp[j + 2], w2 * rv);
-                } else {
-                    atomicAdd(&bp[J - 1], 2.f * w2 * rv);
-                    atomicAdd(&bp[J - 2], -w2 * rv);
-                }
-            }
+            rv_s[tid * GK_LD + p] =
+                halfOmega * wgt * (b != a ? 2.f : 1.f) * (th[a].x * th[b].x + th[a].y * th[b].y);
         }
     }
     float e = 0.f;
 #pragma unroll
     for (int a = 0; a < NQ; ++a) e = fmaf(th[a].x, u[a].x, fmaf(th[a].y, u[a].y, e));
     const double es = block_sum((double)(wgt * e), red);
-    if (threadIdx.x == 0) epart[blockIdx.x] = es;
+    if (tid == 0) epart[blockIdx.x] = es;
 #pragma unroll
     for (int q = 0; q < NQ / 4; ++q) {
         Q[q * qstride + 2 * r] =
@@ -836,9 +828,51 @@ __global__ void __launch_bounds__(SORTED_BLOCK) k_learned_contract_gradk(float4*
         Q[q * qstride + 2 * r + 1] =
             make_float4(u[4 * q + 2].x * invN, u[4 * q + 2].y * invN, u[4 * q + 3].x * invN, u[4 * q + 3].y * invN);
     }
-    __syncthreads();
-    for (int i = threadIdx.x; i < LRN_P * J; i += blockDim.x)
-        if (bins[i] != 0.f) atomicAdd(&gK[i], (double)bins[i]);
+    // (block_sum's barriers order the writes above before these reads)
+    const int pair = tid % LRN_P, pt = tid / LRN_P;
+    for (int lo = 0; lo < SORTED_BLOCK;) {
+        const int jr = j_s[lo];
+        int hi = SORTED_BLOCK;
+        if (j_s[SORTED_BLOCK - 1] != jr) {  // the run's end: first point past it (j_s is non-decreasing)
+            int a = lo;
+            while (hi - a > 1) {
+                const int mid = (a + hi) >> 1;
+                if (j_s[mid] == jr) a = mid;
+                else hi = mid;
+            }
+        }
+        if (pt < GK_PARTS) {
+            float4 s = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int k = lo + pt; k < hi; k += GK_PARTS) {
+                const float rv = rv_s[k * GK_LD + pair];
+                const float4 w = w_s[k];
+                s.x = fmaf(rv, w.x, s.x);
+                s.y = fmaf(rv, w.y, s.y);
+                s.z = fmaf(rv, w.z, s.z);
+                s.w = fmaf(rv, w.w, s.w);
+            }
+            *reinterpret_cast<float4*>(part[pt][pair]) = s;
+        }
+        __syncthreads();
+        for (int o = tid; o < 4 * LRN_P; o += SORTED_BLOCK) {
+            const int pp = o >> 2, c = o & 3;
+            double s = 0.0;
+#pragma unroll
+            for (int k = 0; k < GK_PARTS; ++k) s += (double)part[k][pp][c];
+            // knots of the four weights: the knot before k = 0 mirrors knot 1;
+            // past the last knot the linear extrapolation 2 K_{J-1} - K_{J-2}
+            double* g = gK + pp * J;
+            const int kn = jr - 1 + c;
+            if (kn > J - 1) {
+                atomicAdd(g + J - 1, 2.0 * s);
+                atomicAdd(g + J - 2, -s);
+            } else {
+                atomicAdd(g + (kn < 0 ? 1 : kn), s);
+            }
+        }
+        __syncthreads();
+        lo = hi;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -939,151 +973,334 @@ __global__ void __launch_bounds__(L_THREADS, 1) k_learned_channels(const float* 
 }
 
 // ---------------------------------------------------------------------------
-// parameter gradient through the network (CUDA cores, FP32, FP64 totals)
+// parameter gradient through the network (tensor cores, FP64 totals)
 // ---------------------------------------------------------------------------
 // mode 0 (energy): cotangent of w_m at point i is coef dOmega n_i U[m][i];
 // mode 1 (fit):    coef 2 wt_i (w_m - T[m][i]) for the loss sum_i wt_i |w - T|^2.
+//
+// Persistent, one block per SM, two teams of 256 threads; a team takes tiles
+// of 128 points, two threads per point (32 hidden units each).  All products
+// are contractions and run on the tensor cores with FP32 accumulation:
+//   Z2 = h1 W2^T                                  (per point, 64 x 64)
+//   dh1 = dz2 W2                                  (per point, 64 x 64)
+//   sum over points of {h1, 1} dz2, dout h2, {x, 1} dz1
+// h1, h2 and the weights are bf16 values by definition of the network; the
+// FP32 factors (dz2, dz1, dout, x) enter as three bf16 terms whose sum is the
+// FP32 value to its last bit, so every product is exact and only the
+// accumulation rounds, as in an FP32 sum.  The sums over points read the
+// stored [point][unit] tiles transposed, with one 128-row operand
+//   H = [h1 (64) | dout in three terms (24) | x1, x2 in three terms (6) | 1 | 1]
+// against the columns dz2, h2 and dz1 (tensor memory: 256 columns per team,
+// scratch and one block of 64 per factor).  Each row of H is wanted with one
+// of the three factors only, so a thread adds 32 columns of its row to FP32
+// registers after every tile: the tensor cores' accumulation does not round
+// to nearest, and summed over all tiles there it left 1e-5 of relative error
+// against 64 bits (the smallest terms go first for the same reason).
+// Bound by the CUDA-core work per point (about 5 k instructions: SiLU and its
+// derivative for 64 + 64 units, the splits, dh2 = W3^T dout).
+// 180 x 180 x 72: 6828 us with one thread per point on the CUDA cores (each
+// product a shared-memory read and an FMA) -> 812 us; error against 64 bits,
+// norms of the blocks: 2e-7 to 2e-5 before, 6e-8 to 2e-5 now (the larger ones
+// are activations that round to bf16 the other way).
 constexpr int PG_TILE = 128;
-constexpr int PG_THREADS = 256;
-constexpr int PG_LD = LRN_H + 1;  // padded row of the per-point tiles
+constexpr int PG_TEAM = 256;
+constexpr int PG_THREADS = 2 * PG_TEAM;
+constexpr int PG_HK = 128;                // width of the H tile
+constexpr int PG_DOUT = 64, PG_X = 88, PG_ONE = 94;  // its columns after h1 (94: 1 with dz2, 95: 1 with dz1)
+
+struct __align__(128) PgTeam {
+    uint16_t H[PG_TILE * PG_HK];
+    uint16_t H2[PG_TILE * LRN_H];
+    uint16_t D[3][PG_TILE * LRN_H];  // the three terms of dz2, then of dz1
+};
+struct __align__(128) PgShared {
+    PgTeam team[2];
+    uint16_t w2f[LRN_H * LRN_H];  // [out][in]
+    uint16_t w2t[LRN_H * LRN_H];  // [in][out]
+    float w3[LRN_M * LRN_H];
+    float w1[2 * LRN_H], b1[LRN_H], b2[LRN_H], b3[LRN_M];
+};
+
+// v as three bf16 terms: a + b + c = v
+__device__ __forceinline__ void split3(float v, float& a, float& b, float& c) {
+    a = bf16r(v);
+    const float r = v - a;
+    b = bf16r(r);
+    c = r - b;
+}
+// 8 values in three terms to one 16-byte chunk of each of three tiles
+__device__ __forceinline__ void store8_split(uint16_t* d0, uint16_t* d1, uint16_t* d2, const float* v) {
+    float a[8], b[8], c[8];
+#pragma unroll
+    for (int i = 0; i < 8; ++i) split3(v[i], a[i], b[i], c[i]);
+    store8_bf16(d0, a);
+    store8_bf16(d1, b);
+    store8_bf16(d2, c);
+}
 
 __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
     const float* __restrict__ n, const float* __restrict__ grad, long long N, float n_min, LearnedArgs la,
     const float* __restrict__ cot, const float* __restrict__ wt, int mode, float coef, double* __restrict__ gout) {
-    extern __shared__ float smf[];
-    float* W2 = smf;                          // [H][H]
-    float* W3 = W2 + LRN_H * LRN_H;           // [M][H]
-    float* w1 = W3 + LRN_M * LRN_H;           // [H][2]
-    float* b1 = w1 + 2 * LRN_H;
-    float* b2 = b1 + LRN_H;
-    float* b3 = b2 + LRN_H;                   // [M] (padded to 8)
-    float* H1 = b3 + LRN_M;                   // [TILE][LD]
-    float* H2 = H1 + PG_TILE * PG_LD;         // [TILE][LD]; later delta z1
-    float* DZ2 = H2 + PG_TILE * PG_LD;        // [TILE][LD]
-    float* DO = DZ2 + PG_TILE * PG_LD;        // [TILE][M]
-    float* X = DO + PG_TILE * LRN_M;          // [TILE][2]
-    const int t = threadIdx.x;
-    for (int i = t; i < LRN_H * LRN_H; i += PG_THREADS) W2[i] = la.w2r[i];
-    for (int i = t; i < LRN_M * LRN_H; i += PG_THREADS) W3[i] = la.w3r[i];
-    for (int i = t; i < 2 * LRN_H; i += PG_THREADS) w1[i] = la.w1[i];
-    for (int i = t; i < LRN_H; i += PG_THREADS) {
-        b1[i] = la.b1[i];
-        b2[i] = la.b2[i];
+    extern __shared__ __align__(128) unsigned char smraw[];
+    __shared__ MlpCtl ctl;
+    PgShared* S = reinterpret_cast<PgShared*>(smraw);
+    const int team = threadIdx.x / PG_TEAM, t = threadIdx.x % PG_TEAM, p = t & (PG_TILE - 1), hf = t / PG_TILE;
+    PgTeam* T = &S->team[team];
+    for (int i = threadIdx.x; i < LRN_H * LRN_H; i += PG_THREADS) {
+        const int o = i / LRN_H, k = i % LRN_H;
+        const uint16_t w = la.w2f[tc::kmaj(o, k, LRN_H)];
+        S->w2f[tc::kmaj(o, k, LRN_H)] = w;
+        S->w2t[tc::kmaj(k, o, LRN_H)] = w;
     }
-    if (t < LRN_M) b3[t] = la.b3[t];
-    // accumulators: dW2[o][i0..i0+15] (o = t / 4, i0 = 16 (t % 4)), dW3[m][j0, j0+1]
-    // (m = t / 32, j0 = 2 (t % 32)), db2[o] (t % 4 == 0), db3 (t < M),
-    // dW1[j][c] and db1[j] for t < 64 (j = t)
-    float aW2[16], aW3[2], ab2 = 0.f, ab3 = 0.f, aW1[2] = {0.f, 0.f}, ab1 = 0.f;
+    for (int i = threadIdx.x; i < LRN_M * LRN_H; i += PG_THREADS) S->w3[i] = la.w3r[i];
+    for (int i = threadIdx.x; i < 2 * LRN_H; i += PG_THREADS) S->w1[i] = la.w1[i];
+    for (int i = threadIdx.x; i < LRN_H; i += PG_THREADS) {
+        S->b1[i] = la.b1[i];
+        S->b2[i] = la.b2[i];
+    }
+    if (threadIdx.x < LRN_M) S->b3[threadIdx.x] = la.b3[threadIdx.x];
+    // the unused columns of H stay zero
+    for (int i = t; i < PG_TILE * 4; i += PG_TEAM)
+        *reinterpret_cast<uint4*>(T->H + tc::kmaj(i >> 2, 96 + 8 * (i & 3), PG_HK)) = make_uint4(0, 0, 0, 0);
+    // one mbarrier and 256 tensor-memory columns per team (mlp_setup counts
+    // warpgroups: the block's four get 128 columns each, a team two of them)
+    mlp_setup(&ctl, 128);
+    const uint32_t tm = ctl.tmem + 256u * (uint32_t)team;
+    const uint32_t lane = tm + ((uint32_t)(p & ~31) << 16);
+    const uint32_t aH = tc::smem_u32(T->H), aH2 = tc::smem_u32(T->H2);
+    uint32_t aD[3];
 #pragma unroll
-    for (int q = 0; q < 16; ++q) aW2[q] = 0.f;
-    aW3[0] = aW3[1] = 0.f;
-    const float dOmegaCoef = coef;
+    for (int s = 0; s < 3; ++s) aD[s] = tc::smem_u32(T->D[s]);
+    const auto team_bar = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "r"(PG_TEAM) : "memory"); };
+    uint32_t phase = 0;
+    // sum of H^T B over the tile's points into the columns at col (B: a
+    // [point][64] tile; 8 steps of 16 points)
+    const auto mma_sum = [&](uint32_t col, uint32_t b, bool first) {
+        for (int k = 0; k < PG_TILE / 16; ++k)
+            tc::mma_bf16(tm + col, tc::operand_desc_t(aH, PG_HK, k, 0), tc::operand_desc_t(b, LRN_H, k, 0),
+                         tc::idesc_bf16_t(128, LRN_H), !(first && k == 0));
+    };
+    // all of the team's writes are done: one thread issues, then commits
+    const auto issue = [&](auto f) {
+        tc::fence_async_smem();
+        tc::fence_before_sync();
+        team_bar();
+        if (t == 0) {
+            tc::fence_after_sync();
+            f();
+            tc::mma_commit(&ctl.bar[team]);
+        }
+    };
+    const auto wait = [&]() {
+        const bool ok = tc::mbar_wait(&ctl.bar[team], phase);
+        if (!ok) {
+            atomicExch(&ctl.abort[team], 1);
+            *(volatile int*)la.err = 1;  // page-locked host word, read by the next entry point
+            __threadfence_system();
+            tc::mbar_wait(&ctl.bar[team], phase);  // a second bounded wait for the MMAs in flight
+        }
+        phase ^= 1u;
+        team_bar();
+        tc::fence_after_sync();
+        return ctl.abort[team] == 0;
+    };
+    // this row's sums over the tiles: columns 32 hf .. 32 hf + 31 of the
+    // factor its H column goes with
+    float acc[32];
+#pragma unroll
+    for (int q = 0; q < 32; ++q) acc[q] = 0.f;
+    const bool row3 = p >= PG_DOUT && p < PG_X, row1 = (p >= PG_X && p < PG_ONE) || p == PG_ONE + 1;
+    const auto flush = [&]() {
+        const int warp = p >> 5;
+        if (warp == 3) return;  // rows 96 .. 127 are zero
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            float v[16];
+            tc::tmem_ld16(lane + 64 + 32 * hf + 16 * c, v);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) acc[16 * c + q] += (row3 || row1) ? 0.f : v[q];
+            if (warp == 2) {
+                tc::tmem_ld16(lane + 128 + 32 * hf + 16 * c, v);
+#pragma unroll
+                for (int q = 0; q < 16; ++q) acc[16 * c + q] += row3 ? v[q] : 0.f;
+                tc::tmem_ld16(lane + 192 + 32 * hf + 16 * c, v);
+#pragma unroll
+                for (int q = 0; q < 16; ++q) acc[16 * c + q] += row1 ? v[q] : 0.f;
+            }
+        }
+    };
+    float ab3[LRN_M];
+#pragma unroll
+    for (int m = 0; m < LRN_M; ++m) ab3[m] = 0.f;
     const long long ntiles = (N + PG_TILE - 1) / PG_TILE;
-    for (long long T = blockIdx.x; T < ntiles; T += gridDim.x) {
-        __syncthreads();
-        if (t < PG_TILE) {
-            const long long i = T * PG_TILE + t;
-            const bool in = i < N;
-            float ni = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
-            if (in) {
-                ni = n[i];
-                gx = grad[i];
-                gy = grad[N + i];
-                gz = grad[2 * N + i];
+    bool first = true, good = true;
+    for (long long tile = 2 * (long long)blockIdx.x + team; tile < ntiles; tile += 2 * (long long)gridDim.x) {
+        const long long i = tile * PG_TILE + p;
+        const bool in = i < N;
+        float ni = 0.f, gx = 0.f, gy = 0.f, gz = 0.f;
+        if (in) {
+            ni = n[i];
+            gx = grad[i];
+            gy = grad[N + i];
+            gz = grad[2 * N + i];
+        }
+        const Feat f = features(ni, gx, gy, gz, la, n_min);
+        const bool ok = in && f.ok;
+        const float x1 = ok ? f.x1 : 0.f, x2 = ok ? f.x2 : 0.f;
+        float dout[LRN_M];
+#pragma unroll
+        for (int m = 0; m < LRN_M; ++m) dout[m] = (ok && mode == 0) ? coef * ni * cot[m * N + i] : 0.f;
+        // the last sums of the previous tile read H and D
+        if (!first) {
+            if (!(good = wait())) break;
+            flush();
+        }
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float h[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+                const int j = 32 * hf + 8 * c + q;
+                h[q] = silu(fmaf(S->w1[2 * j], x1, fmaf(S->w1[2 * j + 1], x2, S->b1[j])));
             }
-            const Feat f = features(ni, gx, gy, gz, la, n_min);
-            const bool ok = in && f.ok;
-            const float x1 = ok ? f.x1 : 0.f, x2 = ok ? f.x2 : 0.f;
-            X[2 * t] = x1;
-            X[2 * t + 1] = x2;
-            float* h1 = H1 + t * PG_LD;
-            for (int j = 0; j < LRN_H; ++j)
-                h1[j] = bf16r(silu(fmaf(w1[2 * j], x1, fmaf(w1[2 * j + 1], x2, b1[j]))));
-            float* h2 = H2 + t * PG_LD;
-            float* dz2 = DZ2 + t * PG_LD;
-            for (int o = 0; o < LRN_H; ++o) {
-                float z = b2[o];
-                for (int j = 0; j < LRN_H; ++j) z = fmaf(W2[o * LRN_H + j], h1[j], z);
-                dz2[o] = z;  // pre-activation, replaced by its delta below
-                h2[o] = bf16r(silu(z));
-            }
-            float dout[LRN_M];
-            for (int m = 0; m < LRN_M; ++m) {
-                float d = 0.f;
-                if (ok) {
-                    if (mode == 0) {
-                        d = dOmegaCoef * ni * cot[m * N + i];
-                    } else {
-                        float om = b3[m];
-                        for (int j = 0; j < LRN_H; ++j) om = fmaf(W3[m * LRN_H + j], h2[j], om);
-                        d = dOmegaCoef * 2.f * wt[i] * (om - cot[m * N + i]);
-                    }
+            store8_bf16(T->H + tc::kmaj(p, 32 * hf + 8 * c, PG_HK), h);
+        }
+        if (hf == 0) {
+            float x[8];
+            split3(x1, x[0], x[1], x[2]);
+            split3(x2, x[3], x[4], x[5]);
+            x[6] = 1.f;
+            x[7] = 1.f;
+            store8_bf16(T->H + tc::kmaj(p, PG_X, PG_HK), x);
+        }
+        issue([&]() {
+            for (int k = 0; k < LRN_H / 16; ++k)
+                tc::mma_bf16(tm, tc::operand_desc(aH, PG_HK, k), tc::operand_desc(tc::smem_u32(S->w2f), LRN_H, k),
+                             tc::idesc_bf16(128, LRN_H), k > 0);
+        });
+        if (!(good = wait())) break;
+        // h2 and silu'(z2) of this thread's 32 units
+        float sp[32];
+        float om[LRN_M];
+#pragma unroll
+        for (int m = 0; m < LRN_M; ++m) om[m] = 0.f;
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            float v[16];
+            tc::tmem_ld16(lane + 32 * hf + 16 * c, v);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) silu_both(v[q] + S->b2[32 * hf + 16 * c + q], v[q], sp[16 * c + q]);
+            store8_bf16(T->H2 + tc::kmaj(p, 32 * hf + 16 * c, LRN_H), v);
+            store8_bf16(T->H2 + tc::kmaj(p, 32 * hf + 16 * c + 8, LRN_H), v + 8);
+            if (mode == 1) {
+#pragma unroll
+                for (int q = 0; q < 16; ++q) {
+                    const float hq = bf16r(v[q]);
+#pragma unroll
+                    for (int m = 0; m < LRN_M; ++m)
+                        om[m] = fmaf(S->w3[m * LRN_H + 32 * hf + 16 * c + q], hq, om[m]);
                 }
-                dout[m] = d;
-                DO[t * LRN_M + m] = d;
-            }
-            for (int o = 0; o < LRN_H; ++o) {
-                float dh = 0.f;
-                for (int m = 0; m < LRN_M; ++m) dh = fmaf(W3[m * LRN_H + o], dout[m], dh);
-                dz2[o] = dh * silu_prime(dz2[o]);
             }
         }
-        __syncthreads();
-        {
-            const int o = t >> 2, i0 = 16 * (t & 3);
-            for (int p = 0; p < PG_TILE; ++p) {
-                const float d = DZ2[p * PG_LD + o];
-                const float* h1 = H1 + p * PG_LD + i0;
+        if (mode == 1) {
+            // the two halves' outputs, through the (free) D tile
+            float* ex = reinterpret_cast<float*>(T->D[0]);
 #pragma unroll
-                for (int q = 0; q < 16; ++q) aW2[q] = fmaf(d, h1[q], aW2[q]);
-                if ((t & 3) == 0) ab2 += d;
+            for (int m = 0; m < LRN_M; ++m) ex[(hf * LRN_M + m) * PG_TILE + p] = om[m];
+            team_bar();
+            if (ok) {
+#pragma unroll
+                for (int m = 0; m < LRN_M; ++m) {
+                    const float o = S->b3[m] + (ex[m * PG_TILE + p] + ex[(LRN_M + m) * PG_TILE + p]);
+                    dout[m] = coef * 2.f * wt[i] * (o - cot[m * N + i]);
+                }
             }
-            const int m = t >> 5, j0 = 2 * (t & 31);
-            for (int p = 0; p < PG_TILE; ++p) {
-                const float d = DO[p * LRN_M + m];
-                aW3[0] = fmaf(d, H2[p * PG_LD + j0], aW3[0]);
-                aW3[1] = fmaf(d, H2[p * PG_LD + j0 + 1], aW3[1]);
-                if (t < LRN_M) ab3 += DO[p * LRN_M + t];
+            team_bar();
+        }
+        if (hf == 1) {
+            uint16_t* h = T->H;
+            store8_split(h + tc::kmaj(p, PG_DOUT, PG_HK), h + tc::kmaj(p, PG_DOUT + 8, PG_HK),
+                         h + tc::kmaj(p, PG_DOUT + 16, PG_HK), dout);
+        } else {
+#pragma unroll
+            for (int m = 0; m < LRN_M; ++m) ab3[m] += dout[m];
+        }
+        // dz2 = (W3^T dout) silu'(z2)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            float d[8];
+#pragma unroll
+            for (int q = 0; q < 8; ++q) d[q] = 0.f;
+#pragma unroll
+            for (int m = 0; m < LRN_M; ++m) {
+                const float4* w = reinterpret_cast<const float4*>(S->w3 + m * LRN_H + 32 * hf + 8 * c);
+                const float4 w0 = w[0], w1 = w[1];
+                d[0] = fmaf(w0.x, dout[m], d[0]);
+                d[1] = fmaf(w0.y, dout[m], d[1]);
+                d[2] = fmaf(w0.z, dout[m], d[2]);
+                d[3] = fmaf(w0.w, dout[m], d[3]);
+                d[4] = fmaf(w1.x, dout[m], d[4]);
+                d[5] = fmaf(w1.y, dout[m], d[5]);
+                d[6] = fmaf(w1.z, dout[m], d[6]);
+                d[7] = fmaf(w1.w, dout[m], d[7]);
+            }
+#pragma unroll
+            for (int q = 0; q < 8; ++q) d[q] *= sp[8 * c + q];
+            const int at = tc::kmaj(p, 32 * hf + 8 * c, LRN_H);
+            store8_split(T->D[0] + at, T->D[1] + at, T->D[2] + at, d);
+        }
+        issue([&]() {
+            for (int s = 2; s >= 0; --s)
+                for (int k = 0; k < LRN_H / 16; ++k)
+                    tc::mma_bf16(tm, tc::operand_desc(aD[s], LRN_H, k),
+                                 tc::operand_desc(tc::smem_u32(S->w2t), LRN_H, k), tc::idesc_bf16(128, LRN_H),
+                                 s < 2 || k > 0);
+            for (int s = 2; s >= 0; --s) mma_sum(64, aD[s], s == 2);
+            mma_sum(128, aH2, true);
+        });
+        if (!(good = wait())) break;
+        // dz1 = dh1 silu'(z1)
+#pragma unroll
+        for (int c = 0; c < 2; ++c) {
+            float v[16];
+            tc::tmem_ld16(lane + 32 * hf + 16 * c, v);
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const int j = 32 * hf + 16 * c + q;
+                v[q] *= silu_prime(fmaf(S->w1[2 * j], x1, fmaf(S->w1[2 * j + 1], x2, S->b1[j])));
+            }
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const int at = tc::kmaj(p, 32 * hf + 16 * c + 8 * h, LRN_H);
+                store8_split(T->D[0] + at, T->D[1] + at, T->D[2] + at, v + 8 * h);
             }
         }
-        __syncthreads();
-        if (t < PG_TILE) {
-            // delta z1 = (W2^T delta z2) * silu'(z1), into this point's H2 row
-            const float x1 = X[2 * t], x2 = X[2 * t + 1];
-            const float* dz2 = DZ2 + t * PG_LD;
-            float* dz1 = H2 + t * PG_LD;
-            for (int j = 0; j < LRN_H; ++j) {
-                float dh = 0.f;
-                for (int o = 0; o < LRN_H; ++o) dh = fmaf(W2[o * LRN_H + j], dz2[o], dh);
-                dz1[j] = dh * silu_prime(fmaf(w1[2 * j], x1, fmaf(w1[2 * j + 1], x2, b1[j])));
-            }
+        issue([&]() {
+            for (int s = 2; s >= 0; --s) mma_sum(192, aD[s], s == 2);
+        });
+        first = false;
+    }
+    if (good && !first && wait()) {
+        flush();
+#pragma unroll
+        for (int q = 0; q < 32; ++q) {
+            const int j = 32 * hf + q;
+            const int at = p < PG_DOUT ? LRN_OFF_W2 + j * LRN_H + p
+                           : p < PG_X  ? LRN_OFF_W3 + ((p - PG_DOUT) % LRN_M) * LRN_H + j
+                           : p < PG_ONE ? LRN_OFF_W1 + 2 * j + (p - PG_X) / 3
+                           : p == PG_ONE ? LRN_OFF_B2 + j
+                                         : LRN_OFF_B1 + j;
+            if (p <= PG_ONE + 1) atomicAdd(&gout[at], (double)acc[q]);
         }
-        __syncthreads();
-        if (t < LRN_H) {
-            for (int p = 0; p < PG_TILE; ++p) {
-                const float d = H2[p * PG_LD + t];
-                aW1[0] = fmaf(d, X[2 * p], aW1[0]);
-                aW1[1] = fmaf(d, X[2 * p + 1], aW1[1]);
-                ab1 += d;
+        if (hf == 0) {
+#pragma unroll
+            for (int m = 0; m < LRN_M; ++m) {
+                const double s = warp_sum((double)ab3[m]);
+                if ((p & 31) == 0) atomicAdd(&gout[LRN_OFF_B3 + m], s);
             }
         }
     }
-    {
-        const int o = t >> 2, i0 = 16 * (t & 3);
-#pragma unroll
-        for (int q = 0; q < 16; ++q) atomicAdd(&gout[LRN_OFF_W2 + o * LRN_H + i0 + q], (double)aW2[q]);
-        if ((t & 3) == 0) atomicAdd(&gout[LRN_OFF_B2 + o], (double)ab2);
-        const int m = t >> 5, j0 = 2 * (t & 31);
-        atomicAdd(&gout[LRN_OFF_W3 + m * LRN_H + j0], (double)aW3[0]);
-        atomicAdd(&gout[LRN_OFF_W3 + m * LRN_H + j0 + 1], (double)aW3[1]);
-        if (t < LRN_M) atomicAdd(&gout[LRN_OFF_B3 + t], (double)ab3);
-        if (t < LRN_H) {
-            atomicAdd(&gout[LRN_OFF_W1 + 2 * t], (double)aW1[0]);
-            atomicAdd(&gout[LRN_OFF_W1 + 2 * t + 1], (double)aW1[1]);
-            atomicAdd(&gout[LRN_OFF_B1 + t], (double)ab1);
-        }
-    }
+    mlp_teardown(&ctl);
 }
 
 __global__ void k_axpy(double* __restrict__ y, const double* __restrict__ x, double a, int n) {
@@ -1277,12 +1494,7 @@ int lookup_blocks(vdw_ctx* c) {
     const long long wave = (long long)std::max(1, c->nsm) * per_sm;
     return (int)std::max(1LL, std::min(std::min(want, wave), (long long)c->g.N2 * L_SLOTS));
 }
-// knot-gradient bins of k_learned_contract_gradk
-size_t smem_gradk(int J) { return sizeof(float) * (size_t)LRN_P * J; }
-size_t smem_pgrad() {
-    return sizeof(float) * ((size_t)LRN_H * LRN_H + LRN_M * LRN_H + 2 * LRN_H + 2 * LRN_H + LRN_M +
-                            3 * (size_t)PG_TILE * PG_LD + PG_TILE * LRN_M + 2 * PG_TILE);
-}
+size_t smem_pgrad() { return sizeof(PgShared); }
 size_t smem_pgrad_pencil(const GridArgs& g) {
     return sizeof(float2) * tw_offset((size_t)4 * GRAD_COLS * pencil_stride(g.p2)) + sizeof(Tw) * (g.N2 - g.p2.P1);
 }
@@ -1300,8 +1512,8 @@ int set_smem(K kernel, size_t bytes, const char* name) {
 template <int CN1, int CN2, int CN3>
 int configure(vdw_ctx* c) {
     const GridArgs& g = c->g;
-    int rc = set_smem(k_learned_net, smem_net(), "k_learned_net");
-    if (!rc) rc = set_smem(k_learned_contract_gradk, smem_gradk(c->lrn_J), "k_learned_contract_gradk");
+    int rc = set_smem(k_learned_net<true>, smem_net(), "k_learned_net");
+    if (!rc) rc = set_smem(k_learned_net<false>, smem_net(), "k_learned_net");
     if (!rc) rc = set_smem(k_field_plane<CN1, CN3>, smem_plane(g), "k_field_plane");
     if (!rc) rc = set_smem(k_plane_inv3<CN1, CN3>, smem_plane(g), "k_plane_inv3");
     if (!rc) rc = set_smem(k_pencil_grad<CN2>, smem_pgrad_pencil(g), "k_pencil_grad");
@@ -1353,8 +1565,11 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
         k_learned_lookup<<<nb0, LOOKUP_THREADS, 0, s>>>(n, grad, g, P, la, specf, ep, c->d_invalid,
                                                        want_pot ? c->d_lw : nullptr);
     else
-        k_learned_net<<<nb0, L_NET_THREADS, smem_net(), s>>>(n, grad, g, P, la, specf, ep, c->d_invalid,
-                                                         (want_pot && kind != RUN_GRAD) ? c->d_lw : nullptr);
+    {
+        const bool lw = want_pot && kind != RUN_GRAD;
+        if (lw) k_learned_net<true><<<nb0, L_NET_THREADS, smem_net(), s>>>(n, grad, g, P, la, specf, ep, c->d_invalid, c->d_lw);
+        else k_learned_net<false><<<nb0, L_NET_THREADS, smem_net(), s>>>(n, grad, g, P, la, specf, ep, c->d_invalid, nullptr);
+    }
     mark(ST_POINTWISE);
     int rc = planes_inplace(c, LRN_M, false, s);
     if (rc) return rc;
@@ -1364,7 +1579,7 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
     mark(ST_PENCILS_FWD);
     if (kind == RUN_GRAD) {
         VDW_CUDA(cudaMemsetAsync(c->d_gK, 0, sizeof(double) * LRN_P * c->lrn_J, s));
-        k_learned_contract_gradk<<<c->nb_sorted, SORTED_BLOCK, smem_gradk(c->lrn_J), s>>>(
+        k_learned_contract_gradk<<<c->nb_sorted, SORTED_BLOCK, 0, s>>>(
             c->d_Q, 2 * c->Npad, c->d_gs, la, g.invN, ep + nb0, c->d_gK,
             (float)(0.5 * Omega / ((double)g.N * (double)g.N)));
         VDW_CUDA(cudaGetLastError());
@@ -1468,7 +1683,7 @@ bool lrn_ready(vdw_ctx* c) {
 
 // Size of the learned context's allocation and its layout (256-byte aligned pieces).
 struct LrnLayout {
-    size_t epart, w1, b1, b2, b3, w2r, w3r, w2f, w3f, knots, err, gK, total;
+    size_t epart, w1, b1, b2, b3, w3r, w2f, w3f, knots, err, gK, total;
 };
 static LrnLayout lrn_layout(const GridArgs& g, int J, int nb_sorted) {
     LrnLayout L{};
@@ -1485,7 +1700,6 @@ static LrnLayout lrn_layout(const GridArgs& g, int J, int nb_sorted) {
     L.b1 = take(sizeof(float) * LRN_H);
     L.b2 = take(sizeof(float) * LRN_H);
     L.b3 = take(sizeof(float) * LRN_M);
-    L.w2r = take(sizeof(float) * LRN_H * LRN_H);
     L.w3r = take(sizeof(float) * LRN_M * LRN_H);
     L.w2f = take(2 * LRN_H * LRN_H);
     L.w3f = take(2 * LRN_N3 * LRN_H);
@@ -1556,7 +1770,6 @@ int vdw_learned_load(vdw_handle c, int J, double k_max, const double feat[5], do
         la.b1 = reinterpret_cast<float*>(b + L.b1);
         la.b2 = reinterpret_cast<float*>(b + L.b2);
         la.b3 = reinterpret_cast<float*>(b + L.b3);
-        la.w2r = reinterpret_cast<float*>(b + L.w2r);
         la.w3r = reinterpret_cast<float*>(b + L.w3r);
         la.w2f = reinterpret_cast<uint16_t*>(b + L.w2f);
         la.w3f = reinterpret_cast<uint16_t*>(b + L.w3f);

@@ -41,6 +41,20 @@ __host__ __device__ constexpr uint32_t idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
 }
 
+// The same stored tile read the other way: a [R rows][K] tile as the operand
+// whose M (or N) index is the tile's k and whose contraction runs over the
+// tile's rows (MN-major, no swizzling: the stride-dimension offset is the
+// distance of core matrices adjacent in M or N, the leading-dimension offset
+// that of core matrices adjacent in the contraction).  Descriptor of step s
+// (16 rows) from column chunk c0 (8 columns each) on.
+__device__ __forceinline__ uint64_t operand_desc_t(uint32_t addr, int K, int s, int c0) {
+    return smem_desc(addr + 128u * (uint32_t)c0 + 32u * (uint32_t)K * (uint32_t)s, 16u * (uint32_t)K, 128u);
+}
+// instruction descriptor with both operands read that way
+__host__ __device__ constexpr uint32_t idesc_bf16_t(int M, int N) {
+    return idesc_bf16(M, N) | (1u << 15) | (1u << 16);
+}
+
 // D[tmem] (+)= A B^T for one 16-wide K step; issued by a single thread
 __device__ __forceinline__ void mma_bf16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc, uint32_t idesc,
                                          uint32_t accumulate) {
