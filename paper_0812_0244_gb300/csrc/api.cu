@@ -195,6 +195,7 @@ int vdw_create(vdw_handle* h, const vdw_params* p, const double* phi_k, double C
     delete[] table;
     if (rc != VDW_OK) {
         cudaFree(c->d_kcoef);
+        cudaFree(c->d_Mq);
         delete c;
         return rc;
     }
@@ -268,8 +269,13 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
         c->p0_chunks = (nh3 % 4 == 0) ? 4 : (nh3 % 3 == 0) ? 3 : (nh3 % 2 == 0) ? 2 : 1;
         c->p0_nj = nh3 / c->p0_chunks;
         c->p0_mnj = c->p0_nj > 1 ? 0xFFFFFFFFu / (unsigned)c->p0_nj + 1u : 0u;
-        const long long nb = std::min<long long>((g.N + 255) / 256, 4096);
-        c->nb_p0 = (int)((nb + c->p0_chunks - 1) / c->p0_chunks);
+        // per slab one wave of resident blocks at most, one pair of points per
+        // thread at a time: each block copies the spline table once
+        int dev = 0, nsm = 0;
+        VDW_CUDA(cudaGetDevice(&dev));
+        VDW_CUDA(cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev));
+        const long long pairs = (long long)c->p0_nj * n2 * n1;
+        c->nb_p0 = (int)std::min<long long>((pairs + 255) / 256, (long long)POINT_BLOCKS * nsm);
         c->nb_point = c->nb_p0 * c->p0_chunks;
     }
     VDW_CUDA(cudaMalloc(&c->d_tw, sizeof(float4) * (n1 + 2 * n2 + n3)));
@@ -475,6 +481,7 @@ int vdw_destroy(vdw_handle c) {
     cudaSetDevice(c->device);
     free_plan(c);
     cudaFree(c->d_kcoef);
+    cudaFree(c->d_Mq);
     for (int i = 0; i <= VDW_NSTAGES; ++i)
         if (c->ev[i]) cudaEventDestroy(c->ev[i]);
     delete c;

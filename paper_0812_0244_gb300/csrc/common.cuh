@@ -31,6 +31,7 @@ static_assert(ST_COUNT == VDW_NSTAGES, "stage list");
 constexpr int MAX_NQ = 32;     // largest interpolation mesh the kernels take
 constexpr int MAX_MC = 32;     // largest order m_c of the saturation sum of Eq. (Sat)
 constexpr int MAX_DIM = 256;   // largest grid dimension (FFT line length)
+constexpr int POINT_BLOCKS = 4;  // blocks of the pointwise kernel per SM
 constexpr uint8_t K_INVALID = 255;  // interval code of a point with theta = 0
 
 // Schedule of one line length n = P1 P2: the products of the two groups of
@@ -49,7 +50,9 @@ struct PointParams {
     float C_s;
     float inv_m[MAX_MC + 1];     // 1/m, m = 1 .. m_c (terms of the saturation sum)
     float qm[MAX_NQ];            // q mesh
-    float Mq[MAX_NQ][MAX_NQ];    // Mq[a][k]: second derivative of p_a at knot k
+    // device, [MAX_NQ][MAX_NQ]: Mq[a MAX_NQ + k] = second derivative of p_a at
+    // knot k (a block copies what it needs to shared memory)
+    const float* Mq;
 };
 
 // Grid geometry shared by the plane and pencil kernels.
@@ -129,6 +132,7 @@ struct vdw_ctx {
     vdw::PointParams pp;        // host copy of the pointwise constants
     double phi0, C_s;
     float4* d_kcoef;            // [Nk-1][npairs] cubic coefficients in local t
+    float* d_Mq;                // behind pp.Mq
     // plan
     int planned;
     vdw::GridArgs g;

@@ -55,14 +55,15 @@ constexpr int XC_BLOCKS = 1024;  // blocks (and partial-sum slots) of the semilo
 // 40 registers, six blocks of 256 threads per SM: 0.100 ms at 180 x 180 x 72
 // against 0.112 ms at 64 registers and four blocks.
 template <int NQ>
-__global__ void __launch_bounds__(256, 6) k_pointwise(const float* __restrict__ n, const float* __restrict__ grad,
+__global__ void __launch_bounds__(256, POINT_BLOCKS) k_pointwise(const float* __restrict__ n, const float* __restrict__ grad,
                                                    GridArgs g, PointParams P, int slab, int nj, unsigned mnj,
                                                    int nbs, float* __restrict__ t_out, uint8_t* __restrict__ k_out,
-                                                   float4* __restrict__ aux, float* __restrict__ specf,
+                                                   float4* __restrict__ aux, float2* __restrict__ spec,
                                                    double* __restrict__ epart,
                                                    unsigned long long* __restrict__ invalid) {
     __shared__ double red[32];
-    __shared__ SplineSmem sp;
+    __shared__ SplineMesh sp;
+    __shared__ float2 mp[NQ * MP_LD];
     {
         // density blockIdx.y of a batch
         const long long b = blockIdx.y;
@@ -71,54 +72,75 @@ __global__ void __launch_bounds__(256, 6) k_pointwise(const float* __restrict__ 
         t_out += b * g.N;
         k_out += b * g.N;
         aux += b * g.N;
-        specf += 2 * b * g.bs_spec;
+        spec += b * g.bs_spec;
         epart += b * g.bs_epart;
     }
-    load_spline_smem(&sp, P);
+    load_spline_mesh(&sp, P);
+    load_spline_pairs<NQ>(mp, P);
     __syncthreads();
     const int sl = slab >= 0 ? slab : (int)blockIdx.x / nbs;
     const int lb = slab >= 0 ? (int)blockIdx.x : (int)blockIdx.x - sl * nbs;
     const int j0 = sl * nj;
-    const long long N = g.N;
-    const long long Nc = 2LL * g.N2 * nj * g.N1;    // points of the slab
-    const long long fstride = 2LL * g.N2 * g.ncols;  // floats between the planes of two fields
+    const long long N = g.N, zs = (long long)g.N1 * g.N2;
+    const long long Nc = (long long)g.N2 * nj * g.N1;     // pairs of points of the slab
+    const long long fstride = (long long)g.N2 * g.ncols;  // values between the planes of two fields
     double acc = 0.0;
     unsigned int bad = 0;
     for (long long q = lb * (long long)blockDim.x + threadIdx.x; q < Nc; q += (long long)nbs * blockDim.x) {
         int y, x, jj;
-        const int s = (int)(q & 1);
         if (g.fast) {
-            const unsigned t = (unsigned)(q >> 1);
-            const unsigned rr = __umulhi(t, g.m1);
-            x = (int)(t - rr * (unsigned)g.N1);
+            const unsigned rr = __umulhi((unsigned)q, g.m1);
+            x = (int)((unsigned)q - rr * (unsigned)g.N1);
             y = nj == 1 ? (int)rr : (int)__umulhi(rr, mnj);
             jj = (int)(rr - (unsigned)y * (unsigned)nj);
         } else {
-            const long long t = q >> 1;
-            const long long rr = t / g.N1;
-            x = (int)(t - rr * g.N1);
+            const long long rr = q / g.N1;
+            x = (int)(q - rr * g.N1);
             y = (int)(rr / nj);
             jj = (int)(rr - (long long)y * nj);
         }
-        const int j = j0 + jj, z = 2 * j + s;
-        const long long i = ((long long)z * g.N2 + y) * g.N1 + x;
-        const float ni = n[i];
-        bad += (!(ni >= 0.f) || !isfinite(ni)) ? 1u : 0u;
-        const QPoint qp = q_point(ni, grad[i], grad[N + i], grad[2 * N + i], P, sp.qm);
-        t_out[i] = qp.t;
-        k_out[i] = (uint8_t)qp.k;
-        float* dst = specf + 2LL * y * g.ncols + packed_offset(x, j, z & 1, g.Nh);
-        if (qp.k != K_INVALID) {
-            const float q = qp.q, q3 = q * q * q, q4 = q3 * q;
-            acc += (double)(0.5f * P.C_s * ni * ni / q3);
-            const float cn = 1.5f * P.C_s * ni * ni / q4;
-            aux[i] = make_float4(ni * qp.dq_dn, ni * qp.dq_dg, P.C_s * ni / q3 - cn * qp.dq_dn, -cn * qp.dq_dg);
+        const int j = j0 + jj;
+        const long long i0 = (2LL * j * g.N2 + y) * g.N1 + x;
+        // per point: the spline's coefficients at its interval
+        float nn[2], A[2], B[2], cA[2], cB[2], h26[2];
+        int kk[2];
 #pragma unroll
-            for (int a = 0; a < NQ; ++a) dst[a * fstride] = ni * cardinal_value(&sp, a, qp.k, qp.t);
-        } else {
-            aux[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+        for (int s = 0; s < 2; ++s) {
+            const long long i = i0 + s * zs;
+            const float ni = n[i];
+            bad += (!(ni >= 0.f) || !isfinite(ni)) ? 1u : 0u;
+            const QPoint qp = q_point(ni, grad[i], grad[N + i], grad[2 * N + i], P, sp.qm);
+            t_out[i] = qp.t;
+            k_out[i] = (uint8_t)qp.k;
+            const bool ok = qp.k != K_INVALID;
+            float4 ax = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (ok) {
+                const float qv = qp.q, q3 = qv * qv * qv, q4 = q3 * qv;
+                acc += (double)(0.5f * P.C_s * ni * ni / q3);
+                const float cn = 1.5f * P.C_s * ni * ni / q4;
+                ax = make_float4(ni * qp.dq_dn, ni * qp.dq_dg, P.C_s * ni / q3 - cn * qp.dq_dn, -cn * qp.dq_dg);
+            }
+            aux[i] = ax;
+            nn[s] = ok ? ni : 0.f;
+            kk[s] = ok ? qp.k : 0;
+            A[s] = 1.f - qp.t;
+            B[s] = qp.t;
+            cA[s] = A[s] * A[s] * A[s] - A[s];
+            cB[s] = B[s] * B[s] * B[s] - B[s];
+            h26[s] = sp.h26[kk[s]];
+        }
+        float2* dst = spec + ((long long)y * g.ncols + (2 * j * g.Nh + x));
+        const float2* m0 = mp + kk[0];
+        const float2* m1 = mp + kk[1];
 #pragma unroll
-            for (int a = 0; a < NQ; ++a) dst[a * fstride] = 0.f;
+        for (int a = 0; a < NQ; ++a) {
+            // p_a = (A at a = k, B at a = k + 1) + (cA M_ak + cB M_a,k+1) h^2/6
+            const float2 u = m0[a * MP_LD], w = m1[a * MP_LD];
+            const float y0 = a == kk[0] ? A[0] : (a == kk[0] + 1 ? B[0] : 0.f);
+            const float y1 = a == kk[1] ? A[1] : (a == kk[1] + 1 ? B[1] : 0.f);
+            const float p0 = fmaf(fmaf(cA[0], u.x, cB[0] * u.y), h26[0], y0);
+            const float p1 = fmaf(fmaf(cA[1], w.x, cB[1] * w.y), h26[1], y1);
+            dst[a * fstride] = make_float2(nn[0] * p0, nn[1] * p1);
         }
     }
     const double s = block_sum(acc, red);
@@ -148,12 +170,13 @@ constexpr int USUM_THREADS = 256;
 // One thread takes the two points z = 2 j, 2 j + 1 of a packed row, so that a
 // field's two values come by one 8-byte load.
 template <int NQ>
-__global__ void __launch_bounds__(USUM_THREADS) k_u_sum(const float2* __restrict__ uf, const float* __restrict__ grad,
+__global__ void __launch_bounds__(USUM_THREADS, 4) k_u_sum(const float2* __restrict__ uf, const float* __restrict__ grad,
                                                         const float* __restrict__ tk, const uint8_t* __restrict__ kk,
                                                         const float4* __restrict__ aux, GridArgs g, PointParams P,
                                                         float* __restrict__ v, float* __restrict__ w_out,
                                                         float* __restrict__ g_out, int mode) {
-    __shared__ SplineSmem sp;
+    __shared__ SplineMesh sp;
+    __shared__ float2 mp[NQ * MP_LD];
     {
         // density blockIdx.y of a batch
         const long long b = blockIdx.y;
@@ -166,7 +189,8 @@ __global__ void __launch_bounds__(USUM_THREADS) k_u_sum(const float2* __restrict
         if (w_out) w_out += 3 * b * g.N;
         if (g_out) g_out += b * g.N;
     }
-    load_spline_smem(&sp, P);
+    load_spline_mesh(&sp, P);
+    load_spline_pairs<NQ>(mp, P);
     __syncthreads();
     const long long N = g.N;
     const long long fstride = (long long)g.N2 * g.ncols;  // values between the planes of two fields
@@ -182,11 +206,11 @@ __global__ void __launch_bounds__(USUM_THREADS) k_u_sum(const float2* __restrict
 #pragma unroll
         for (int a = 0; a < NQ; ++a) {
             const float2 u = up[a * fstride];
-            const float* Ma = sp.Mq + a * MAX_NQ;
-            m0.x = fmaf(u.x, Ma[c0], m0.x);
-            m1.x = fmaf(u.x, Ma[c0 + 1], m1.x);
-            m0.y = fmaf(u.y, Ma[c1], m0.y);
-            m1.y = fmaf(u.y, Ma[c1 + 1], m1.y);
+            const float2 M0 = mp[a * MP_LD + c0], M1 = mp[a * MP_LD + c1];
+            m0.x = fmaf(u.x, M0.x, m0.x);
+            m1.x = fmaf(u.x, M0.y, m1.x);
+            m0.y = fmaf(u.y, M1.x, m0.y);
+            m1.y = fmaf(u.y, M1.y, m1.y);
             uk.x = (a == c0) ? u.x : uk.x;
             uk1.x = (a == c0 + 1) ? u.x : uk1.x;
             uk.y = (a == c1) ? u.y : uk.y;
@@ -745,7 +769,6 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
         cudaEventRecord(c->ev[0], s);
     }
     VDW_CUDA(cudaMemsetAsync(c->d_invalid, 0, sizeof(unsigned long long), s));
-    float* specf = reinterpret_cast<float*>(c->d_spec);
     // one launch over all slabs, or (host entry point) one per slab as its inputs arrive
     const int nlaunch = slab_ready ? c->p0_chunks : 1;
     for (int sl = 0; sl < nlaunch; ++sl) {
@@ -754,7 +777,7 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
         const int nblk = slab_ready ? c->nb_p0 : c->nb_point;
 #define VDW_POINTWISE(NQ)                                                                                  \
     k_pointwise<NQ><<<dim3(nblk, B), 256, 0, s>>>(n, grad, g, P, slab, c->p0_nj, c->p0_mnj, c->nb_p0, c->d_t, c->d_k, \
-                                         c->d_aux, specf, c->d_epart, c->d_invalid)
+                                         c->d_aux, c->d_spec, c->d_epart, c->d_invalid)
         switch (P.Nq) {
             case 20: VDW_POINTWISE(20); break;
             case 8: VDW_POINTWISE(8); break;

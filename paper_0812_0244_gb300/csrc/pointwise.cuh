@@ -107,15 +107,17 @@ __device__ __forceinline__ QPoint q_point(float n, float gx, float gy, float gz,
 // Shared-memory copy of the spline tables: qm[MAX_NQ], Mq[a][k] as
 // Mq[a * MAX_NQ + k].  Indexing them by the per-point interval k from the
 // constant bank would serialise the warp.
-struct SplineSmem {
+struct SplineMesh {
     float qm[MAX_NQ];
-    float Mq[MAX_NQ * MAX_NQ];
     float ih[MAX_NQ];   // 1 / h_k, h_k = q_{k+1} - q_k
     float h26[MAX_NQ];  // h_k^2 / 6
     float h6[MAX_NQ];   // h_k / 6
 };
+struct SplineSmem : SplineMesh {
+    float Mq[MAX_NQ * MAX_NQ];
+};
 
-__device__ __forceinline__ void load_spline_smem(SplineSmem* sp, const PointParams& P) {
+__device__ __forceinline__ void load_spline_mesh(SplineMesh* sp, const PointParams& P) {
     for (int i = threadIdx.x; i < MAX_NQ; i += blockDim.x) {
         sp->qm[i] = P.qm[i];
         const float h = (i + 1 < P.Nq) ? P.qm[i + 1] - P.qm[i] : 1.f;
@@ -123,7 +125,23 @@ __device__ __forceinline__ void load_spline_smem(SplineSmem* sp, const PointPara
         sp->h26[i] = h * h * (1.f / 6.f);
         sp->h6[i] = h * (1.f / 6.f);
     }
-    for (int i = threadIdx.x; i < MAX_NQ * MAX_NQ; i += blockDim.x) sp->Mq[i] = P.Mq[i / MAX_NQ][i % MAX_NQ];
+}
+__device__ __forceinline__ void load_spline_smem(SplineSmem* sp, const PointParams& P) {
+    load_spline_mesh(sp, P);
+    for (int i = threadIdx.x; i < MAX_NQ * MAX_NQ; i += blockDim.x) sp->Mq[i] = P.Mq[i];
+}
+
+// The second derivatives at both ends of interval k as one 8-byte entry,
+// mp[a MP_LD + k] = {M_ak, M_a,k+1} (odd row length: the lanes' intervals
+// spread over the banks)
+constexpr int MP_LD = MAX_NQ - 1;
+template <int NQ>
+__device__ __forceinline__ void load_spline_pairs(float2* mp, const PointParams& P) {
+    for (int i = threadIdx.x; i < NQ * MP_LD; i += blockDim.x) {
+        const int a = i / MP_LD, k = i - a * MP_LD;
+        const float* m = P.Mq + a * MAX_NQ + k;
+        mp[i] = make_float2(m[0], m[1]);
+    }
 }
 
 // p_a and dp_a/dq on interval k at local position t.

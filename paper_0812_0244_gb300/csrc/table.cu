@@ -512,10 +512,14 @@ int table_upload(vdw_ctx* c, const double* h_phik, double C_s) {
     P.q_c = (float)p->q_c;
     P.n_min = (float)p->n_min;
     P.C_s = (float)C_s;
+    std::vector<float> Mf((size_t)MAX_NQ * MAX_NQ);
     for (int i = 0; i < MAX_NQ; ++i) {
         P.qm[i] = i < Nq ? (float)qm[i] : 0.f;
-        for (int k = 0; k < MAX_NQ; ++k) P.Mq[i][k] = (i < Nq && k < Nq) ? (float)M[(size_t)i * Nq + k] : 0.f;
+        for (int k = 0; k < MAX_NQ; ++k) Mf[i * MAX_NQ + k] = (i < Nq && k < Nq) ? (float)M[(size_t)i * Nq + k] : 0.f;
     }
+    if (!c->d_Mq) VDW_CUDA(cudaMalloc(&c->d_Mq, sizeof(float) * Mf.size()));
+    VDW_CUDA(cudaMemcpy(c->d_Mq, Mf.data(), sizeof(float) * Mf.size(), cudaMemcpyHostToDevice));
+    P.Mq = c->d_Mq;
     c->C_s = C_s;
     return VDW_OK;
 }
