@@ -4,7 +4,6 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 #include <stddef.h>
-#include <initializer_list>
 #include <string>
 
 #include "../../include/vdwnl.h"
@@ -260,9 +259,10 @@ int pipeline_xc_final(vdw_ctx* c, double* E, cudaStream_t s);
 // central-difference gradient of a field (into grad [3][N])
 int pipeline_stencil_gradient(vdw_ctx* c, const float* f, float* grad, cudaStream_t s);
 int pipeline_plan_check(vdw_ctx* c);
-size_t smem_plane(const GridArgs& g);
-int plane_block(const vdw_ctx* c, long long nblocks);
-int best_threads(std::initializer_list<int> items, int lo, int hi);
+// shared memory and block size of a plane kernel on nblocks planes, forward or
+// inverse, with hi/lo (exact) or FP32 twiddles
+size_t smem_plane(const GridArgs& g, bool inverse, bool exact);
+int plane_block(const vdw_ctx* c, long long nblocks, bool inverse, bool exact);
 int pipeline_make_twiddles(vdw_ctx* c);
 int pipeline_configure(vdw_ctx* c);
 // the divergence term of a potential (w(G) in d_wspec) and the energy reduction

@@ -365,6 +365,8 @@ struct Grp {
     // output digit q' of register i (the radices run in place: register
     // (ka B + kb) C + kc ends with output ka + A kb + A B kc)
     static constexpr int digit(int i) { return i / (B * C) + A * ((i / C) % B) + A * B * (i % C); }
+    // register of output digit d
+    static constexpr int reg(int d) { return ((d % A) * B + (d / A) % B) * C + d / (A * B); }
 };
 
 // The group's transform of v (input q in register q).  FIRST: Ns = 1,

@@ -1514,8 +1514,8 @@ int configure(vdw_ctx* c) {
     const GridArgs& g = c->g;
     int rc = set_smem(k_learned_net<true>, smem_net(), "k_learned_net");
     if (!rc) rc = set_smem(k_learned_net<false>, smem_net(), "k_learned_net");
-    if (!rc) rc = set_smem(k_field_plane<CN1, CN3>, smem_plane(g), "k_field_plane");
-    if (!rc) rc = set_smem(k_plane_inv3<CN1, CN3>, smem_plane(g), "k_plane_inv3");
+    if (!rc) rc = set_smem(k_field_plane<CN1, CN3>, smem_plane(g, false, true), "k_field_plane");
+    if (!rc) rc = set_smem(k_plane_inv3<CN1, CN3>, smem_plane(g, true, true), "k_plane_inv3");
     if (!rc) rc = set_smem(k_pencil_grad<CN2>, smem_pgrad_pencil(g), "k_pencil_grad");
     if (!rc) rc = set_smem(k_learned_param_grad, smem_pgrad(), "k_learned_param_grad");
     return rc;
@@ -1661,10 +1661,10 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
 template <int CN1, int CN2, int CN3>
 void spectral_gradient(vdw_ctx* c, const float* f, float* out, cudaStream_t s) {
     const GridArgs& g = c->g;
-    k_field_plane<CN1, CN3><<<g.N2, plane_block(c, g.N2), smem_plane(g), s>>>(f, g, c->d_tw, c->d_spec);
+    k_field_plane<CN1, CN3><<<g.N2, plane_block(c, g.N2, false, true), smem_plane(g, false, true), s>>>(f, g, c->d_tw, c->d_spec);
     k_pencil_grad<CN2><<<(g.ncols + GRAD_COLS - 1) / GRAD_COLS, 256, smem_pgrad_pencil(g), s>>>(
         c->d_spec, c->d_wspec, g, c->d_tw + tw_off_y(g));
-    k_plane_inv3<CN1, CN3><<<dim3(g.N2, 3), plane_block(c, 3LL * g.N2), smem_plane(g), s>>>(c->d_wspec, g, c->d_tw, out);
+    k_plane_inv3<CN1, CN3><<<dim3(g.N2, 3), plane_block(c, 3LL * g.N2, true, true), smem_plane(g, true, true), s>>>(c->d_wspec, g, c->d_tw, out);
 }
 
 bool lrn_ready(vdw_ctx* c) {
@@ -1924,8 +1924,8 @@ int vdw_spectral_gradient(vdw_handle c, const float* f, float* grad, void* strea
     cudaStream_t s = (cudaStream_t)stream;
     const int rc = on_grid(g, [&](auto d) {
         using D = decltype(d);
-        int r = set_smem(k_field_plane<D::N1, D::N3>, smem_plane(g), "k_field_plane");
-        if (!r) r = set_smem(k_plane_inv3<D::N1, D::N3>, smem_plane(g), "k_plane_inv3");
+        int r = set_smem(k_field_plane<D::N1, D::N3>, smem_plane(g, false, true), "k_field_plane");
+        if (!r) r = set_smem(k_plane_inv3<D::N1, D::N3>, smem_plane(g, true, true), "k_plane_inv3");
         if (!r) r = set_smem(k_pencil_grad<D::N2>, smem_pgrad_pencil(g), "k_pencil_grad");
         if (!r) spectral_gradient<D::N1, D::N2, D::N3>(c, f, grad, s);
         return r;

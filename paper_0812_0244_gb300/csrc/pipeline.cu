@@ -30,6 +30,7 @@
 #include <cooperative_groups.h>
 
 #include <algorithm>
+#include <initializer_list>
 #include <string>
 #include <vector>
 
@@ -642,42 +643,58 @@ int make_line_plan(int n, bool sized, LinePlan* lp) {
 }
 
 // Block size in [lo, hi] (whole warps) with the fewest thread slots over
-// passes of the given numbers of items, the largest on a tie.
-int best_threads(std::initializer_list<int> items, int lo, int hi) {
+// passes of items of a given cost each, the largest on a tie.
+struct Pass {
+    int items, cost;
+};
+static int best_threads(std::initializer_list<Pass> passes, int lo, int hi) {
     int best = hi;
-    long long cost = -1;
+    long long least = -1;
     for (int t = hi; t >= lo; t -= 32) {
         long long c = 0;
-        for (int n : items) c += (long long)((n + t - 1) / t) * t;
-        if (cost < 0 || c < cost) {
-            cost = c;
+        for (const Pass& p : passes) c += (long long)((p.items + t - 1) / t) * t * p.cost;
+        if (least < 0 || c < least) {
+            least = c;
             best = t;
         }
     }
     return best;
 }
 
-// shared memory of the plane kernels, forward or inverse
-static size_t smem_plane_of(const GridArgs& g, bool inverse, bool pad) {
+// shared memory of a plane kernel, forward or inverse, with hi/lo (exact) or
+// FP32 twiddles
+static size_t smem_plane_of(const GridArgs& g, bool inverse, bool exact, bool pad) {
     const PlaneGeo p = plane_geo(g.p1.P1, g.p1.P2, inverse, pad);
     return sizeof(float2) * tw_offset((size_t)(g.N3 / 2) * p.S) +
-           sizeof(Tw) * ((size_t)(g.N1 - g.p1.P1) + (g.N3 - g.p3.P1));
+           (exact ? sizeof(Tw) : sizeof(float2)) * ((size_t)(g.N1 - g.p1.P1) + (g.N3 - g.p3.P1));
 }
-size_t smem_plane(const GridArgs& g) {
-    return std::max(smem_plane_of(g, false, g.pad_fwd), smem_plane_of(g, true, g.pad_inv));
+size_t smem_plane(const GridArgs& g, bool inverse, bool exact) {
+    return smem_plane_of(g, inverse, exact, inverse ? g.pad_inv : g.pad_fwd);
 }
-// Block size of a plane kernel launched on nblocks planes: about 1024 threads
-// per SM over the blocks that shared memory and the grid allow there, and
-// among the sizes near that the one that wastes the fewest thread slots over
-// the five passes.
-int plane_block(const vdw_ctx* c, long long nblocks) {
+
+// Block size of a plane kernel launched on nblocks planes: as many threads
+// per SM as its registers allow, over the blocks that shared memory and the
+// grid allow there, and among the sizes near that the one that wastes the
+// fewest thread slots over the passes.
+int plane_block(const vdw_ctx* c, long long nblocks, bool inverse, bool exact) {
     const GridArgs& g = c->g;
-    const int nr = g.N3 / 2, nsm = std::max(c->nsm, 1);
-    const long long fit = std::max<long long>(1, 228 * 1024 / (long long)(smem_plane(g) + 1024));
-    const long long per_sm = std::max<long long>(1, std::min<long long>(fit, (nblocks + nsm - 1) / nsm));
-    const int hi = std::max(64, (int)std::min<long long>(PLANE_THREADS, 1024 / per_sm) / 32 * 32);
-    return best_threads({nr * g.p1.P2, nr * g.p1.P1, g.Nh * nr, g.Nh * g.p3.P2, g.Nh * g.p3.P1},
-                        std::max(64, hi * 3 / 4 / 32 * 32), hi);
+    const int nr = g.N3 / 2;
+    const long long nsm = std::max(c->nsm, 1);
+    const long long smem = (long long)smem_plane(g, inverse, exact) + 1024;
+    // three blocks may fill the SM's memory; a fourth only where it leaves
+    // some for L1, through which the planes are loaded (w planes of 180 x 180
+    // x 72: 29 us with three blocks of 288 threads, 37 with four of 256)
+    const long long fit = std::max(1LL, std::min(228 * 1024 / smem, std::max(3LL, 192 * 1024 / smem)));
+    const long long per_sm = std::max(1LL, std::min(fit, (nblocks + nsm - 1) / nsm));
+    const int most = PLANE_THREADS;
+    const bool fused = !inverse && exact && on_grid(g, [&](auto d) { return g.p1.P2 <= FUSE_P<decltype(d)::N1, Tw>; });
+    const int items = std::max({nr * g.p1.P2, nr * g.p1.P1, g.Nh * g.p3.P2, g.Nh * g.p3.P1});
+    const int hi = std::min((int)std::min<long long>(most, 2 * most / per_sm) / 32 * 32, (items + 31) / 32 * 32);
+    const int lo = std::min(hi, (int)(2 * most / (per_sm + 1)) / 32 * 32 + 32);  // no room for another block
+    const Pass second = fused ? Pass{nr * (g.p1.P1 / 2 + 1), 2 * g.p1.P2} : Pass{nr * g.p1.P1, g.p1.P2};
+    return best_threads({{nr * g.p1.P2, g.p1.P1}, second, {fused ? 0 : g.Nh * nr, 2}, {g.Nh * g.p3.P2, g.p3.P1},
+                         {g.Nh * g.p3.P1, g.p3.P2}},
+                        lo, hi);
 }
 static size_t smem_div(const GridArgs& g) {
     return sizeof(float2) * tw_offset((size_t)3 * DIV_COLS * pencil_stride(g.p2)) +
@@ -689,11 +706,11 @@ static const size_t SMEM_MAX = 227 * 1024 - 1024;
 
 int pipeline_plan_check(vdw_ctx* c) {
     GridArgs& g = c->g;
-    g.pad_fwd = smem_plane_of(g, false, true) <= SMEM_MAX;
-    g.pad_inv = smem_plane_of(g, true, true) <= SMEM_MAX;
+    g.pad_fwd = smem_plane_of(g, false, true, true) <= SMEM_MAX;
+    g.pad_inv = smem_plane_of(g, true, true, true) <= SMEM_MAX;
     // the whole-plane limit of the unpadded rows
     if (sizeof(float2) * (size_t)g.N3 * g.Nh + sizeof(Tw) * (g.N1 + g.N3) > 222 * 1024 ||
-        smem_plane(g) > SMEM_MAX || sorted_pencil_smem(g) > SMEM_MAX || smem_div(g) > SMEM_MAX)
+        smem_plane(g, false, true) > SMEM_MAX || smem_plane(g, true, true) > SMEM_MAX || sorted_pencil_smem(g) > SMEM_MAX || smem_div(g) > SMEM_MAX)
         return VDW_ERR_SIZE;
     return VDW_OK;
 }
@@ -789,7 +806,6 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
     }
     mark(ST_POINTWISE);
 
-    const size_t sp = smem_plane(g);
     int rc = planes_inplace(c, P.Nq, false, s, B);
     if (rc) return rc;
     mark(ST_PLANES_FWD);
@@ -859,12 +875,14 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
             k_stencil_div_sub<<<stencil_blocks(g), 256, 0, s>>>(c->d_gg, grad, g, stencil_ih2(c), v);
             mark(ST_DIV_FINAL);
         } else if (mode == 1) {
-            k_w_planes<CN1, CN3><<<dim3(g.N2, 3, B), plane_block(c, 3LL * g.N2 * B), sp, s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
+            k_w_planes<CN1, CN3><<<dim3(g.N2, 3, B), plane_block(c, 3LL * g.N2 * B, false, false),
+                                   smem_plane(g, false, false), s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
             mark(ST_W_PLANES);
             k_pencil_div<CN2><<<dim3((g.ncols + DIV_COLS - 1) / DIV_COLS, B), DIV_THREADS, smem_div(g), s>>>(
                 c->d_wspec, g, c->d_tw + tw_off_y(g), c->d_tw + tw_off_swap(g));
             mark(ST_PENCIL_DIV);
-            k_div_final<CN1, CN3><<<dim3(g.N2, B), plane_block(c, (long long)g.N2 * B), sp, s>>>(c->d_wspec, g, c->d_tw, v);
+            k_div_final<CN1, CN3><<<dim3(g.N2, B), plane_block(c, (long long)g.N2 * B, true, false),
+                                    smem_plane(g, true, false), s>>>(c->d_wspec, g, c->d_tw, v);
             mark(ST_DIV_FINAL);
         }
     }
@@ -876,12 +894,12 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
 template <int CN1, int CN2, int CN3>
 static int configure_sized(vdw_ctx* c) {
     const GridArgs& g = c->g;
-    const int sp = (int)smem_plane(g);
+    const int sf = (int)smem_plane(g, false, false), sp = (int)smem_plane(g, true, false);
     const int sd = (int)smem_div(g);
     int rc = planes_configure(c);
     if (!rc) rc = set_and_check(k_pencil_div<CN2>, "k_pencil_div", sd, DIV_THREADS);
     if (!rc) rc = set_and_check(k_div_final<CN1, CN3>, "k_div_final", sp, PLANE_THREADS);
-    if (!rc) rc = set_and_check(k_w_planes<CN1, CN3>, "k_w_planes", sp, PLANE_THREADS);
+    if (!rc) rc = set_and_check(k_w_planes<CN1, CN3>, "k_w_planes", sf, PLANE_THREADS);
     if (rc) return rc;
     rc = sorted_configure(c);
     if (rc) return rc;
@@ -909,13 +927,13 @@ static void launch_divergence(vdw_ctx* c, float* v, cudaStream_t s) {
     const GridArgs& g = c->g;
     k_pencil_div<CN2><<<(g.ncols + DIV_COLS - 1) / DIV_COLS, DIV_THREADS, smem_div(g), s>>>(
         c->d_wspec, g, c->d_tw + tw_off_y(g), c->d_tw + tw_off_swap(g));
-    k_div_final<CN1, CN3><<<g.N2, plane_block(c, g.N2), smem_plane(g), s>>>(c->d_wspec, g, c->d_tw, v);
+    k_div_final<CN1, CN3><<<g.N2, plane_block(c, g.N2, true, false), smem_plane(g, true, false), s>>>(c->d_wspec, g, c->d_tw, v);
 }
 
 template <int CN1, int CN3>
 static void launch_w_planes(vdw_ctx* c, const float* grad, cudaStream_t s) {
     const GridArgs& g = c->g;
-    k_w_planes<CN1, CN3><<<dim3(g.N2, 3), plane_block(c, 3LL * g.N2), smem_plane(g), s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
+    k_w_planes<CN1, CN3><<<dim3(g.N2, 3), plane_block(c, 3LL * g.N2, false, false), smem_plane(g, false, false), s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
 }
 
 int pipeline_w_planes(vdw_ctx* c, const float* grad, cudaStream_t s) {

@@ -123,26 +123,31 @@ __host__ __device__ __forceinline__ int pencil_stride(const LinePlan& p) {
 // ---------------------------------------------------------------------------
 // Shared memory of a plane transform: N3/2 rows, row j holding the complex
 // row j = (real row 2j) + i (real row 2j + 1), and later the half spectra of
-// those two rows.  Element k of a row sits at slot(k) = k + (k / P)(stride - P)
-// with a run length P and stride = P or P + 1 (padded so that steps of P
-// elements change the bank); a row takes an odd number of slots, so that
-// lanes on consecutive rows hit distinct banks.  Half spectra: real row 2j's
+// those two rows.  Element k of a row sits at slot(k) = k plus one for every
+// 2^sh runs of P elements before it, where P is the step that one pass takes
+// from lane to lane and has a factor of 4 or more in common with the 16
+// 8-byte banks (16 / that factor = 2^sh runs come back to the same bank); no
+// pads for other P.  A row takes an odd number of slots, so that lanes on
+// consecutive rows hit distinct banks.  Half spectra: real row 2j's
 // value at kx takes slot(kx) of row j, real row 2j + 1's takes slot(N1 - kx)
 // (two extra slots at the row's end for kx = 0 and N1/2), so that every pass
 // writes where the same thread read and no pass needs a second buffer.
 struct PlaneGeo {
-    int run, stride;  // slot(k) = k + (k / run)(stride - run)
+    int run, sh;
     int len;          // slots of a row before the two extra ones
     int S;            // slots of a row
+    // offset of the first element of run q, and slot of element k (dP: division by run)
+    __host__ __device__ __forceinline__ constexpr int at(int q) const { return q * run + (q >> sh); }
+    __device__ __forceinline__ int slot(int k, SmallDiv dP) const { return k + (sdiv(k, dP) >> sh); }
 };
 // forward: run P1 (the row transform's first group stores steps of P1);
 // inverse: run P2 (its second group reads steps of P2).  Without the pads
 // where they would not fit in shared memory (wide planes).
 __host__ __device__ constexpr PlaneGeo plane_geo(int P1, int P2, bool inverse, bool pad) {
-    const int run = inverse ? P2 : P1;
-    const int stride = pad ? (run | 1) : run;
-    const int len = stride * (inverse ? P1 : P2);
-    return PlaneGeo{run, stride, len, pad ? ((len + 2) | 1) : len + 2};
+    const int run = inverse ? P2 : P1, cnt = inverse ? P1 : P2;
+    const int sh = !pad ? 31 : run % 16 == 0 ? 0 : run % 8 == 0 ? 1 : run % 4 == 0 ? 2 : 31;
+    const int len = run * cnt + ((cnt - 1) >> sh);
+    return PlaneGeo{run, sh, len, pad ? ((len + 2) | 1) : len + 2};
 }
 template <int CN1, bool INVERSE>
 __device__ __forceinline__ PlaneGeo geo_of(const GridArgs& g) {
@@ -152,6 +157,28 @@ __device__ __forceinline__ PlaneGeo geo_of(const GridArgs& g) {
     } else {
         return plane_geo(g.p1.P1, g.p1.P2, INVERSE, INVERSE ? g.pad_inv : g.pad_fwd);
     }
+}
+// the slots of kx for the even and the odd real row
+__device__ __forceinline__ void half_slots(const PlaneGeo& G, SmallDiv dP, int N1, int kx, int& se, int& so) {
+    const int km = N1 - kx;
+    se = G.slot(kx, dP);
+    so = kx == 0 ? G.len : (kx == km ? G.len + 1 : G.slot(km, dP));
+}
+// A second group of at most this many points is transformed for k and N1 - k
+// in one thread and split into the two half spectra in its registers, which
+// takes a quarter off the shared-memory accesses (180 x 180 x 72: 108 -> 101
+// us, 128^3: 114 -> 100 us forward); above it the split is a pass of its own
+// (registers).  So it is for the w planes (W = float2), a single wave of
+// blocks where the longer thread is slower (35 against 29 us).
+template <int CN1, class W>
+constexpr int FUSE_P = sizeof(W) < sizeof(Tw) ? 0 : CN1 > 0 ? 12 : 9;
+// The half spectra's values from Z_k = f and Z_{-k} = s:
+// (Z_k + conj Z_{-k})/2 and -i (Z_k - conj Z_{-k})/2
+__device__ __forceinline__ float2 split_even(float2 f, float2 s) {
+    return make_float2(0.5f * (f.x + s.x), 0.5f * (f.y - s.y));
+}
+__device__ __forceinline__ float2 split_odd(float2 f, float2 s) {
+    return make_float2(0.5f * (f.y + s.y), -0.5f * (f.x - s.x));
 }
 // position of (z, kx): even and odd real rows of a complex row at slots se, so
 __device__ __forceinline__ int zpos(int z, int S, int se, int so) { return (z >> 1) * S + ((z & 1) ? so : se); }
@@ -196,7 +223,7 @@ __device__ __forceinline__ void plane_forward(float2* sm, const GridArgs& g, con
 #pragma unroll
             for (int q = 0; q < R::P; ++q) v[q] = ld(row, j + q * m);
             group_fft<R, false, true, W>(v, (const W*)nullptr, 1);
-            float2* d = sm + row * S + G.stride * j;
+            float2* d = sm + row * S + G.at(j);
 #pragma unroll
             for (int i = 0; i < R::P; ++i) d[R::digit(i)] = v[i];
         }
@@ -204,47 +231,92 @@ __device__ __forceinline__ void plane_forward(float2* sm, const GridArgs& g, con
     __syncthreads();
     constexpr int CR = CN3 > 0 ? CN3 / 2 : 0;
     const SmallDiv dr = small_div(nr);
+    const SmallDiv dP = small_div(G.run);
     on_second<CN1>(g.p1, [&](auto tag) {
         using R = decltype(tag);
-        for (int it = t0; it < P1 * nr; it += nt) {
-            const int k1 = cdiv<CR>(it, dr), row = it - k1 * nr;
-            float2* d = sm + row * S + k1;
-            float2 v[R::P];
+        constexpr int P = R::P;
+        if constexpr (P <= FUSE_P<CN1, W>) {
+            // k1 = ka and P1 - ka: digit d of one is -(digit P - 1 - d of the
+            // other); k1 = 0 and P1/2 are their own partners
+            for (int it = t0; it < (P1 / 2 + 1) * nr; it += nt) {
+                const int ka = cdiv<CR>(it, dr), row = it - ka * nr;
+                float2* d = sm + row * S;
+                float2* da = d + ka;
+                float2 a[P];
 #pragma unroll
-            for (int q = 0; q < R::P; ++q) v[q] = d[q * G.stride];
-            group_fft<R, false, false, W>(v, tw1 + k1, P1);
+                for (int q = 0; q < P; ++q) a[q] = da[G.at(q)];
+                group_fft<R, false, false, W>(a, tw1 + ka, P1);
+                if (ka == 0) {
+                    da[0] = split_even(a[0], a[0]);
+                    d[G.len] = split_odd(a[0], a[0]);
+                    static_for<P / 2>([&](auto Q) {
+                        constexpr int q = decltype(Q)::value + 1, m = P - q;
+                        const float2 f = a[R::reg(q)], s = a[R::reg(m)];
+                        da[G.at(q)] = split_even(f, s);
+                        (q == m ? d[G.len + 1] : da[G.at(m)]) = split_odd(f, s);
+                    });
+                } else if (2 * ka == P1) {
+                    static_for<(P + 1) / 2>([&](auto Q) {
+                        constexpr int q = decltype(Q)::value, m = P - 1 - q;
+                        const float2 f = a[R::reg(q)], s = a[R::reg(m)];
+                        da[G.at(q)] = split_even(f, s);
+                        (q == m ? d[G.len + 1] : da[G.at(m)]) = split_odd(f, s);
+                    });
+                } else {
+                    const int kb = P1 - ka;
+                    float2* db = d + kb;
+                    float2 b[P];
 #pragma unroll
-            for (int i = 0; i < R::P; ++i) d[R::digit(i) * G.stride] = v[i];
+                    for (int q = 0; q < P; ++q) b[q] = db[G.at(q)];
+                    group_fft<R, false, false, W>(b, tw1 + kb, P1);
+                    static_for<P>([&](auto Q) {
+                        constexpr int q = decltype(Q)::value, m = P - 1 - q;
+                        const float2 x = a[R::reg(q)], y = b[R::reg(m)];
+                        if constexpr (q <= m) {  // k = ka + P1 q below N1/2
+                            da[G.at(q)] = split_even(x, y);
+                            db[G.at(m)] = split_odd(x, y);
+                        } else {
+                            db[G.at(m)] = split_even(y, x);
+                            da[G.at(q)] = split_odd(y, x);
+                        }
+                    });
+                }
+            }
+        } else {
+            for (int it = t0; it < P1 * nr; it += nt) {
+                const int k1 = cdiv<CR>(it, dr), row = it - k1 * nr;
+                float2* d = sm + row * S + k1;
+                float2 v[P];
+#pragma unroll
+                for (int q = 0; q < P; ++q) v[q] = d[G.at(q)];
+                group_fft<R, false, false, W>(v, tw1 + k1, P1);
+#pragma unroll
+                for (int i = 0; i < P; ++i) d[G.at(R::digit(i))] = v[i];
+            }
         }
     });
     __syncthreads();
-    // the two half spectra of each complex row: A = (Z_k + conj Z_{-k})/2,
-    // B = -i (Z_k - conj Z_{-k})/2
-    const SmallDiv dP = small_div(G.run);
-    for (int it = t0; it < Nh * nr; it += nt) {
-        const int k = cdiv<CR>(it, dr), row = it - k * nr;
-        const int km = k == 0 ? 0 : N1 - k;
-        float2* d = sm + row * S;
-        const int sk = k + sdiv(k, dP) * (G.stride - G.run), sm_ = km + sdiv(km, dP) * (G.stride - G.run);
-        const float2 zk = d[sk], zm = d[sm_];
-        d[sk] = make_float2(0.5f * (zk.x + zm.x), 0.5f * (zk.y - zm.y));
-        d[k == 0 ? G.len : (k == km ? G.len + 1 : sm_)] = make_float2(0.5f * (zk.y + zm.y), -0.5f * (zk.x - zm.x));
+    if (N1 / P1 > FUSE_P<CN1, W>) {
+        for (int it = t0; it < Nh * nr; it += nt) {
+            const int k = cdiv<CR>(it, dr), row = it - k * nr;
+            float2* d = sm + row * S;
+            int se, so;
+            half_slots(G, dP, N1, k, se, so);
+            const float2 zk = d[se], zm = d[k == 0 || 2 * k == N1 ? se : so];
+            d[se] = split_even(zk, zm);
+            d[so] = split_odd(zk, zm);
+        }
+        __syncthreads();
     }
-    __syncthreads();
     constexpr int CH = CN1 > 0 ? CN1 / 2 + 1 : 0;
     const SmallDiv dh = small_div(Nh);
-    const auto slots = [&](int kx, int& se, int& so) {
-        const int km = N1 - kx;
-        se = kx + sdiv(kx, dP) * (G.stride - G.run);
-        so = kx == 0 ? G.len : (kx == km ? G.len + 1 : km + sdiv(km, dP) * (G.stride - G.run));
-    };
     on_first<CN3, false>(g.p3, [&](auto tag) {
         using R = decltype(tag);
         const int m = CN3 > 0 ? CN3 / R::P : g.p3.P2;
         for (int it = t0; it < m * Nh; it += nt) {
             const int j = cdiv<CH>(it, dh), kx = it - j * Nh;
             int se, so;
-            slots(kx, se, so);
+            half_slots(G, dP, N1, kx, se, so);
             float2* d0 = sm + zpos(j, S, se, so);
             float2* d1 = sm + zpos(j + m, S, se, so);
             float2 v[R::P];
@@ -261,7 +333,7 @@ __device__ __forceinline__ void plane_forward(float2* sm, const GridArgs& g, con
         for (int it = t0; it < Q1 * Nh; it += nt) {
             const int k1 = cdiv<CH>(it, dh), kx = it - k1 * Nh;
             int se, so;
-            slots(kx, se, so);
+            half_slots(G, dP, N1, kx, se, so);
             const float2* d0 = sm + zpos(k1 * R::P, S, se, so);
             const float2* d1 = sm + zpos(k1 * R::P + 1, S, se, so);
             float2 v[R::P];
@@ -292,11 +364,6 @@ __device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, con
     const int t0 = threadIdx.x, nt = blockDim.x;
     constexpr int CH = CN1 > 0 ? CN1 / 2 + 1 : 0;
     const SmallDiv dh = small_div(Nh), dP = small_div(G.run);
-    const auto slots = [&](int kx, int& se, int& so) {
-        const int km = N1 - kx;
-        se = kx + sdiv(kx, dP) * (G.stride - G.run);
-        so = kx == 0 ? G.len : (kx == km ? G.len + 1 : km + sdiv(km, dP) * (G.stride - G.run));
-    };
     on_first<CN3, false>(g.p3, [&](auto tag) {
         using R = decltype(tag);
         const int m = CN3 > 0 ? CN3 / R::P : g.p3.P2;
@@ -306,7 +373,7 @@ __device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, con
 #pragma unroll
             for (int q = 0; q < R::P; ++q) v[q] = ld(j + q * m, kx);
             int se, so;
-            slots(kx, se, so);
+            half_slots(G, dP, N1, kx, se, so);
             float2* d0 = sm + zpos(R::P * j, S, se, so);
             float2* d1 = sm + zpos(R::P * j + 1, S, se, so);
             group_fft<R, true, true, W>(v, (const W*)nullptr, 1);
@@ -320,7 +387,7 @@ __device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, con
         for (int it = t0; it < Q1 * Nh; it += nt) {
             const int k1 = cdiv<CH>(it, dh), kx = it - k1 * Nh;
             int se, so;
-            slots(kx, se, so);
+            half_slots(G, dP, N1, kx, se, so);
             float2* d0 = sm + zpos(k1, S, se, so);
             float2* d1 = sm + zpos(k1 + Q1, S, se, so);
             float2 v[R::P];
@@ -338,7 +405,7 @@ __device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, con
     for (int it = t0; it < Nh * nr; it += nt) {
         const int k = cdiv<CR>(it, dr), row = it - k * nr;
         int se, so;
-        slots(k, se, so);
+        half_slots(G, dP, N1, k, se, so);
         float2* d = sm + row * S;
         float2 a = d[se], b = d[so];
         const bool edge = k == 0 || 2 * k == N1;
@@ -355,10 +422,10 @@ __device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, con
             float2* d = sm + row * S + j;
             float2 v[R::P];
 #pragma unroll
-            for (int q = 0; q < R::P; ++q) v[q] = d[q * G.stride];
+            for (int q = 0; q < R::P; ++q) v[q] = d[G.at(q)];
             group_fft<R, true, true, W>(v, (const W*)nullptr, 1);
 #pragma unroll
-            for (int i = 0; i < R::P; ++i) d[R::digit(i) * G.stride] = v[i];
+            for (int i = 0; i < R::P; ++i) d[G.at(R::digit(i))] = v[i];
         }
     });
     __syncthreads();
@@ -368,7 +435,7 @@ __device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, con
         using R = decltype(tag);
         for (int it = t0; it < P1 * nr; it += nt) {
             const int row = cdiv<CK>(it, dk), k1 = it - row * P1;
-            const float2* d = sm + row * S + k1 * G.stride;
+            const float2* d = sm + row * S + G.at(k1);
             float2 v[R::P];
 #pragma unroll
             for (int q = 0; q < R::P; ++q) v[q] = d[q];

@@ -43,11 +43,11 @@ __global__ void __launch_bounds__(PLANE_THREADS, 2)
 }
 
 int planes_configure(vdw_ctx* c) {
-    const size_t sm = smem_plane(c->g);
+    const int sf = (int)smem_plane(c->g, false, true), si = (int)smem_plane(c->g, true, false);
     return on_grid(c->g, [&](auto d) {
         using D = decltype(d);
-        int rc = set_and_check(k_planes_inplace<D::N1, D::N3, true>, "k_planes_inplace", (int)sm, PLANE_THREADS);
-        if (!rc) rc = set_and_check(k_planes_inplace<D::N1, D::N3, false>, "k_planes_inplace", (int)sm, PLANE_THREADS);
+        int rc = set_and_check(k_planes_inplace<D::N1, D::N3, true>, "k_planes_inplace", si, PLANE_THREADS);
+        if (!rc) rc = set_and_check(k_planes_inplace<D::N1, D::N3, false>, "k_planes_inplace", sf, PLANE_THREADS);
         return rc;
     });
 }
@@ -55,11 +55,12 @@ int planes_configure(vdw_ctx* c) {
 int planes_inplace(vdw_ctx* c, int nfields, bool inverse, cudaStream_t s, int B) {
     const GridArgs& g = c->g;
     const dim3 grid(g.N2, nfields, B);
-    const int nt = plane_block(c, (long long)g.N2 * nfields * B);
+    const int nt = plane_block(c, (long long)g.N2 * nfields * B, inverse, !inverse);
+    const size_t sm = smem_plane(g, inverse, !inverse);
     on_grid(g, [&](auto d) {
         using D = decltype(d);
-        if (inverse) k_planes_inplace<D::N1, D::N3, true><<<grid, nt, smem_plane(g), s>>>(c->d_spec, g, c->d_tw);
-        else k_planes_inplace<D::N1, D::N3, false><<<grid, nt, smem_plane(g), s>>>(c->d_spec, g, c->d_tw);
+        if (inverse) k_planes_inplace<D::N1, D::N3, true><<<grid, nt, sm, s>>>(c->d_spec, g, c->d_tw);
+        else k_planes_inplace<D::N1, D::N3, false><<<grid, nt, sm, s>>>(c->d_spec, g, c->d_tw);
     });
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;
