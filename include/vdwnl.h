@@ -149,6 +149,16 @@ int vdw_plan_cell(vdw_handle h, int n1, int n2, int n3, const double cell[9]);
 int vdw_energy_potential(vdw_handle h, const float* n, const float* grad,
                          double* E, float* v, float* w, void* stream);
 
+/* E_c^nl and its gradients for an automatic-differentiation framework: E
+ * (device FP64 [1] or NULL) receives E_c^nl; dn [N] and dg [3][N] (device,
+ * each may be NULL) receive gE[0] dE/dn_i at fixed gradient and gE[0]
+ * dE/d(grad_c n)_i, i.e. gE[0] dOmega times v_loc and w of
+ * vdw_energy_potential, gE (device FP64 [1]) being the gradient of the
+ * caller's objective with respect to E (not read, and may be NULL, when dn
+ * and dg are NULL: energy only).  grad must be given.  Asynchronous on stream. */
+int vdw_energy_gradients(vdw_handle h, const float* n, const float* grad, const double* gE, double* E, float* dn,
+                         float* dg, void* stream);
+
 /* ---- several densities per call ------------------------------------------
  * The per-SCF-step cost of the method is its Nq forward and Nq inverse FFTs
  * (text after Eq. Eoffk); a training set or an energy-map scan evaluates many

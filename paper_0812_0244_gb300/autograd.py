@@ -7,7 +7,8 @@ backward : runs the pipeline again with the potential requested in its
              dE/dn_i         = dOmega v_loc,i
              dE/d(grad_c n)_i = dOmega w_c,i
            (Eq. Vi of the paper with the chain through grad n left to
-           autograd), both scaled by the incoming gradient.
+           autograd), both scaled by the incoming gradient inside the
+           assembly kernel (vdw_energy_gradients).
 
 So when the caller builds grad n from n with its own differentiable
 operator, autograd reproduces v_nl of Eq. (Vi) for that operator.
@@ -22,22 +23,27 @@ from .vdwnl import VdwNL
 class VdwEnergy(torch.autograd.Function):
     @staticmethod
     def forward(ctx, n, grad, handle: VdwNL):
-        E = torch.empty(3, dtype=torch.float64, device=n.device)
-        handle.energy_potential(n.contiguous(), grad.contiguous(), E, None, None)
+        E = torch.empty((), dtype=torch.float64, device=n.device)
+        handle.energy_gradients(n.contiguous(), grad.contiguous(), E=E)
         ctx.save_for_backward(n, grad)
         ctx.handle = handle
-        return E[0].clone()
+        return E
 
     @staticmethod
     def backward(ctx, gE):
         n, grad = ctx.saved_tensors
         h = ctx.handle
-        v = torch.empty_like(n, dtype=torch.float32).contiguous()
-        w = torch.empty_like(grad, dtype=torch.float32).contiguous()
-        h.energy_potential(n.contiguous(), grad.contiguous(), None, v, w)
-        scale = (gE * h.dOmega).to(torch.float32)
-        dn = v * scale if ctx.needs_input_grad[0] else None
-        dg = w * scale if ctx.needs_input_grad[1] else None
+        if torch.is_grad_enabled():  # create_graph: the scaling by gE stays a torch operation
+            v = torch.empty_like(n, dtype=torch.float32).contiguous()
+            w = torch.empty_like(grad, dtype=torch.float32).contiguous()
+            h.energy_potential(n.contiguous(), grad.contiguous(), None, v, w)
+            scale = (gE * h.dOmega).to(torch.float32)
+            return (v * scale if ctx.needs_input_grad[0] else None,
+                    w * scale if ctx.needs_input_grad[1] else None, None)
+        n, grad = n.contiguous(), grad.contiguous()
+        dn = torch.empty_like(n) if ctx.needs_input_grad[0] else None
+        dg = torch.empty_like(grad) if ctx.needs_input_grad[1] else None
+        h.energy_gradients(n, grad, gE, None, dn, dg)
         return dn, dg, None
 
 

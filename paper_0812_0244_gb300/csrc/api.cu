@@ -8,6 +8,7 @@
 #include <mutex>
 #include <new>
 #include <string>
+#include <vector>
 
 namespace vdw {
 
@@ -54,7 +55,9 @@ static void free_plan(vdw_ctx* c) {
     cudaFree(c->d_k);
     cudaFree(c->d_aux);
     cudaFree(c->d_epart);
-    cudaFree(c->d_invalid);
+    cudaFree(c->d_ecount);
+    c->d_ecount = nullptr;
+    cudaFree(c->d_bad);
     cudaFree(c->d_in);
     cudaFree(c->d_v);
     cudaFree(c->d_E);
@@ -64,7 +67,7 @@ static void free_plan(vdw_ctx* c) {
     c->d_k = nullptr;
     c->d_aux = nullptr;
     c->d_epart = nullptr;
-    c->d_invalid = nullptr;
+    c->d_bad = nullptr;
     c->d_in = c->d_v = nullptr;
     c->d_E = nullptr;
     cudaFree(c->d_gtmp);
@@ -93,6 +96,18 @@ static void free_plan(vdw_ctx* c) {
     c->planned = 0;
 }
 
+// The last call's count of negative or non-finite densities (its work is complete).
+static int invalid_count(vdw_ctx* c, unsigned long long* sum) {
+    *sum = 0;
+    if (!c->d_bad) return VDW_OK;
+    unsigned n = 0;
+    VDW_CUDA(cudaMemcpy(&n, c->d_bad, sizeof(n), cudaMemcpyDeviceToHost));
+    std::vector<unsigned> v(n);
+    if (n) VDW_CUDA(cudaMemcpy(v.data(), c->d_bad + 1, sizeof(n) * n, cudaMemcpyDeviceToHost));
+    for (unsigned x : v) *sum += x;
+    return VDW_OK;
+}
+
 // The per-density workspaces for Bmax densities at once (spectra, records,
 // w spectra, the pointwise results and the energy partial sums), with the
 // batch strides the kernels use.  Frees the previous ones.
@@ -102,6 +117,15 @@ int alloc_density_work(vdw_ctx* c, int Bmax) {
     const size_t spec_n = Nq * g.N2 * g.ncols, wspec_n = 3 * (size_t)g.N2 * g.ncols;
     const size_t q_n = Nq * (size_t)c->Npad / 2;  // float4 values (Nq/4 quads of Npad 32-byte records)
     const size_t ep_n = (size_t)c->nb_point + c->nb_sorted + 2 * EPART_SPLIT;
+    // the last call's count survives in one entry
+    unsigned long long bad = 0;
+    if (const int rc = invalid_count(c, &bad)) return rc;
+    cudaFree(c->d_bad);
+    c->d_bad = nullptr;
+    c->bad_cap = std::max(c->nb_point * Bmax, 8 * g.N2);  // (learned path: at most 8 N2 blocks)
+    VDW_CUDA(cudaMalloc(&c->d_bad, sizeof(unsigned) * (1 + (size_t)c->bad_cap)));
+    const unsigned keep[2] = {1u, (unsigned)bad};
+    VDW_CUDA(cudaMemcpy(c->d_bad, keep, sizeof(keep), cudaMemcpyHostToDevice));
     const size_t old = c->batch_max > 0
                            ? (size_t)c->batch_max * (8 * (spec_n + wspec_n) + 16 * q_n + 25 * N + 8 * ep_n)
                            : 0;
@@ -131,6 +155,10 @@ int alloc_density_work(vdw_ctx* c, int Bmax) {
     VDW_CUDA(cudaMalloc(&c->d_aux, sizeof(float4) * N * B));
     VDW_CUDA(cudaMalloc(&c->d_gg, sizeof(float) * N * B));
     VDW_CUDA(cudaMalloc(&c->d_epart, sizeof(double) * ep_n * B));
+    cudaFree(c->d_ecount);
+    c->d_ecount = nullptr;
+    VDW_CUDA(cudaMalloc(&c->d_ecount, sizeof(unsigned) * B));
+    VDW_CUDA(cudaMemset(c->d_ecount, 0, sizeof(unsigned) * B));
     g.bs_spec = (long long)spec_n;
     g.bs_wspec = (long long)wspec_n;
     g.bs_Q = (long long)q_n;
@@ -283,7 +311,6 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
     if (rc) return rc;
     rc = alloc_density_work(c, 1);
     if (rc) return rc;
-    VDW_CUDA(cudaMalloc(&c->d_invalid, sizeof(unsigned long long)));
     VDW_CUDA(cudaHostAlloc(&c->h_flags, 2 * sizeof(int), cudaHostAllocMapped));
     c->h_flags[0] = c->h_flags[1] = 0;
     VDW_CUDA(cudaHostGetDevicePointer((void**)&c->d_flags, c->h_flags, 0));
@@ -295,7 +322,6 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
     VDW_CUDA(cudaEventCreateWithFlags(&c->ev_join, cudaEventDisableTiming));
     VDW_CUDA(cudaEventCreateWithFlags(&c->ev_in, cudaEventDisableTiming));
     for (int i = 0; i < 4; ++i) VDW_CUDA(cudaEventCreateWithFlags(&c->ev_slab[i], cudaEventDisableTiming));
-    VDW_CUDA(cudaMemset(c->d_invalid, 0, sizeof(unsigned long long)));
     rc = pipeline_make_twiddles(c);
     if (rc) return rc;
     rc = pipeline_configure(c);
@@ -320,6 +346,17 @@ int vdw_energy_potential(vdw_handle c, const float* n, const float* grad, double
         grad = c->d_gtmp;
     }
     return pipeline_run(c, n, grad, E, v, w, (cudaStream_t)stream);
+}
+
+int vdw_energy_gradients(vdw_handle c, const float* n, const float* grad, const double* gE, double* E, float* dn,
+                         float* dg, void* stream) {
+    if (!c || !n || !grad || ((dn || dg) && !gE)) return VDW_ERR_ARG;
+    if (!c->planned) return VDW_ERR_STATE;
+    if (const int rw = check_wait(c)) return rw;
+    GradScale gs;
+    gs.on = true;
+    gs.gE = gE;
+    return pipeline_run(c, n, grad, E, dn, dg, (cudaStream_t)stream, 0, 0, nullptr, 1, gs);
 }
 
 int vdw_plan_cell(vdw_handle c, int n1, int n2, int n3, const double cell[9]) {
@@ -429,7 +466,7 @@ int vdw_last_invalid_points(vdw_handle c, long long* count) {
     if (!c->planned) return VDW_ERR_STATE;
     unsigned long long v = 0;
     VDW_CUDA(cudaDeviceSynchronize());
-    VDW_CUDA(cudaMemcpy(&v, c->d_invalid, sizeof(v), cudaMemcpyDeviceToHost));
+    if (const int rc = invalid_count(c, &v)) return rc;
     *count = (long long)v;
     return VDW_OK;
 }

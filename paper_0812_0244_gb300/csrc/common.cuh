@@ -143,6 +143,7 @@ struct vdw_ctx {
     uint8_t* d_k;               // [N] mesh interval of q (K_INVALID: theta = 0)
     float4* d_aux;              // [N] n dq/dn, n dq/d|grad n| / |grad n|, and the Delta E derivatives
     double* d_epart;            // per-block energy partial sums
+    unsigned* d_ecount;         // per density: blocks of the running energy reduction that are done
     int nb_point;               // their count for the pointwise kernel
     // points of the half spectrum in |G| order (contract.cu)
     long long nG, Npad;         // N2 N3 (N1/2 + 1), rounded up to whole contraction blocks
@@ -163,7 +164,10 @@ struct vdw_ctx {
     cudaEvent_t ev_slab[4];     // slab c of the inputs is on the device
     cudaStream_t s_side;        // the energy reduction beside the inverse transforms
     cudaEvent_t ev_fork, ev_join;
-    unsigned long long* d_invalid;  // count of negative / non-finite densities
+    // negative or non-finite densities of the last call: [0] the number of
+    // entries, then one count per block of its pointwise kernel
+    unsigned* d_bad;
+    int bad_cap;                // entries d_bad has room for
     float* d_gg;                // [N] g of w = g grad n (assembly -> w plane transforms)
     // give-up flags of the bounded waits, in mapped page-locked host memory so
     // that an entry point can read them without synchronising: [1] the
@@ -204,6 +208,36 @@ int cuda_fail(cudaError_t e, const char* what);
 int check_wait(vdw_ctx* c);
 // per-density workspaces for Bmax densities (api.cu)
 int alloc_density_work(vdw_ctx* c, int Bmax);
+
+// Programmatic dependent launch: a kernel started by launch() may begin while
+// the kernel before it in the stream still runs its last blocks.  Such a
+// kernel calls pdl_wait() before it touches anything that earlier work of the
+// stream reads or writes (the wait ends when all of that work is complete and
+// visible); ahead of it only tables that live as long as the plan are read
+// (twiddles, the spline mesh, |G| order).  pdl_wait() also lets the kernel
+// after it start in the same way.
+__device__ __forceinline__ void pdl_wait() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// early: small grids only (early_launch), where launch latency and the first
+// loads are a good part of a kernel; the blocks that wait take shared memory
+// and L1 from the running kernel, which costs a large grid more (24^3 74 -> 53
+// us a call, 100^3 497 -> 456; 256 x 256 x 96 2697 -> 2733, so not there).
+template <class... K, class... A>
+inline void launch(bool early, void (*kernel)(K...), dim3 grid, int block, size_t smem, cudaStream_t s, A&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = early ? 1 : 0;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<K>(args)...);
+}
 
 #define VDW_CUDA(call)                                         \
     do {                                                       \
@@ -247,13 +281,21 @@ int set_and_check(K kernel, const char* name, int smem, int threads) {
     return VDW_OK;
 }
 
+inline bool early_launch(const GridArgs& g, int B) { return g.N * B <= (1LL << 21); }
+
 // pipeline launchers (pipeline.cu)
 // slab_ready (optional): per slab of the pointwise pass, an event to wait on
 // before processing it (the host entry point's copies)
 // B > 1: a batch of B densities (n [B][N], grad [B][3][N], E [B][3], v [B][N],
 // w [B][3][N]), one launch per stage; needs the batch workspaces of vdw_plan_batch
+// gs: gradient outputs (v_loc, w) times gE[0] dOmega, and E is E_c^nl alone
+struct GradScale {
+    bool on = false;
+    const double* gE = nullptr;
+};
 int pipeline_run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, float* w,
-                 cudaStream_t s, int fd = 0, int xc = 0, const cudaEvent_t* slab_ready = nullptr, int B = 1);
+                 cudaStream_t s, int fd = 0, int xc = 0, const cudaEvent_t* slab_ready = nullptr, int B = 1,
+                 GradScale gs = {});
 // E[4] of the functional from the nonlocal energy (d_xc[0]) and the semilocal sums
 int pipeline_xc_final(vdw_ctx* c, double* E, cudaStream_t s);
 // central-difference gradient of a field (into grad [3][N])
@@ -290,10 +332,10 @@ int sorted_contract_table(vdw_ctx* c, int nq, const float4* table, float inv_dk,
                           int write_back, cudaStream_t s, int B = 1);
 constexpr int SORTED_BLOCK = 128;  // sorted points per contraction block
 // The energy's partial sums (one per block of the pointwise pass and of the
-// contraction) are reduced in two passes: EPART_SPLIT blocks each sum a fixed
-// contiguous share of both arrays, one block sums their EPART_SPLIT results in
-// index order.  The per-density partial-sum array ends with those 2
-// EPART_SPLIT values.
+// contraction) are reduced by EPART_SPLIT blocks that each sum a fixed
+// contiguous share of both arrays; the block that finishes last sums their
+// EPART_SPLIT results in index order.  The per-density partial-sum array ends
+// with those 2 EPART_SPLIT values.
 constexpr int EPART_SPLIT = 64;
 
 // learned reduced basis (learned.cu)

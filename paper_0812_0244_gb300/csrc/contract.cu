@@ -84,6 +84,7 @@ __global__ void __launch_bounds__(PEN_THREADS, 3) k_pencil_fwd(const float2* __r
     const int S = pencil_stride(L), LS = pencil_field_stride(L, false);
     Tw* tw2 = twiddles_after(sm, (size_t)4 * LS);
     load_twiddles(tw2, tw, N2 - P1);
+    pdl_wait();
     const int c0 = blockIdx.x * PEN_COLS, q = blockIdx.y;
     spec += blockIdx.z * g.bs_spec + (long long)4 * q * N2 * g.ncols;  // density blockIdx.z of a batch
     float2* Qf = reinterpret_cast<float2*>(Q + blockIdx.z * g.bs_Q + q * qstride);
@@ -146,6 +147,7 @@ __global__ void __launch_bounds__(PEN_THREADS, 3) k_pencil_inv(float2* __restric
     const int S = pencil_stride(L), LS = pencil_field_stride(L, true);
     float2* tw2 = twiddles_after<float2>(sm, (size_t)4 * LS);
     load_twiddles(tw2, tw, N2 - P1);
+    pdl_wait();
     const int c0 = blockIdx.x * PEN_COLS, q = blockIdx.y;
     spec += blockIdx.z * g.bs_spec + (long long)4 * q * N2 * g.ncols;  // density blockIdx.z of a batch
     const float2* Qf = reinterpret_cast<const float2*>(Q + blockIdx.z * g.bs_Q + q * qstride);
@@ -250,6 +252,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 4) k_contract_sorted(float4* __r
     __shared__ float4 rows[STAGED ? CONTRACT_ROWS * NP : 1];
     Q += blockIdx.y * bsQ;  // density blockIdx.y of a batch
     epart += blockIdx.y * bsE;
+    pdl_wait();
     const long long r0 = (long long)blockIdx.x * SORT_THREADS;
     const long long r = r0 + threadIdx.x;
     float2 th[NQ];
@@ -364,6 +367,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, 6) k_contract_pairs(
     __shared__ float4 rows[CONTRACT_ROWS * NP * 2];
     Q += blockIdx.y * bsQ;  // density blockIdx.y of a batch
     epart += blockIdx.y * bsE;
+    pdl_wait();
     const long long r0 = (long long)blockIdx.x * SORT_THREADS;
     const long long r = r0 + threadIdx.x, r1 = r + PAIR_THREADS;
     float2 thx[NQ], thy[NQ], ux[NQ], uy[NQ];
@@ -504,8 +508,7 @@ int sorted_forward(vdw_ctx* c, int nfields, cudaStream_t s, int B) {
     const GridArgs& g = c->g;
     const dim3 grid((g.ncols + PEN_COLS - 1) / PEN_COLS, nfields / 4, B);
     on_grid(g, [&](auto d) {
-        k_pencil_fwd<decltype(d)::N2><<<grid, PEN_THREADS, sorted_pencil_smem(g), s>>>(
-            c->d_spec, g, c->d_tw + tw_off_y(g), c->d_pos, c->d_Q, 2 * c->Npad);
+        launch(early_launch(g, B), k_pencil_fwd<decltype(d)::N2>, grid, PEN_THREADS, sorted_pencil_smem(g), s, c->d_spec, g, c->d_tw + tw_off_y(g), c->d_pos, c->d_Q, 2 * c->Npad);
     });
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;
@@ -515,8 +518,7 @@ int sorted_inverse(vdw_ctx* c, int nfields, cudaStream_t s, int B) {
     const GridArgs& g = c->g;
     const dim3 grid((g.ncols + PEN_COLS - 1) / PEN_COLS, nfields / 4, B);
     on_grid(g, [&](auto d) {
-        k_pencil_inv<decltype(d)::N2><<<grid, PEN_THREADS, sorted_pencil_smem(g), s>>>(
-            c->d_spec, g, c->d_tw + tw_off_y(g), c->d_pos, c->d_Q, 2 * c->Npad);
+        launch(early_launch(g, B), k_pencil_inv<decltype(d)::N2>, grid, PEN_THREADS, sorted_pencil_smem(g), s, c->d_spec, g, c->d_tw + tw_off_y(g), c->d_pos, c->d_Q, 2 * c->Npad);
     });
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;
@@ -536,8 +538,8 @@ int sorted_contract_table(vdw_ctx* c, int nq, const float4* table, float inv_dk,
                                          std::pow(g.N3 / c->L[2], 2));
     const bool staged = c->nb_sorted >= 2.0 * gmax * inv_dk;
 #define VDW_CONTRACT_K(KERNEL, THREADS)                                                                  \
-    KERNEL<<<dim3(c->nb_sorted, B), THREADS, 0, s>>>(c->d_Q, qs, c->d_gs, table, inv_dk, nk, g.invN, epart, \
-                                                     write_back, g.bs_Q, g.bs_epart)
+    launch(early_launch(g, B), KERNEL, dim3(c->nb_sorted, B), THREADS, 0, s, c->d_Q, qs, c->d_gs, table, inv_dk, nk, g.invN, epart, \
+           write_back, g.bs_Q, g.bs_epart)
 #define VDW_CONTRACT(NQ)                                                                                 \
     if (staged) VDW_CONTRACT_K((k_contract_sorted<NQ, true>), SORT_THREADS);                             \
     else VDW_CONTRACT_K((k_contract_sorted<NQ, false>), SORT_THREADS)

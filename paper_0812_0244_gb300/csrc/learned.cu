@@ -480,7 +480,7 @@ template <bool JAC>
 __global__ void __launch_bounds__(L_NET_THREADS, 1)
     k_learned_net(const float* __restrict__ n, const float* __restrict__ grad, GridArgs g, PointParams P,
                   LearnedArgs la, float* __restrict__ specf, double* __restrict__ epart,
-                  unsigned long long* __restrict__ invalid, float* __restrict__ lw) {
+                  unsigned* __restrict__ badp, float* __restrict__ lw) {
     extern __shared__ __align__(128) unsigned char smraw[];
     __shared__ MlpCtl ctl;
     __shared__ double red[32];
@@ -567,7 +567,10 @@ __global__ void __launch_bounds__(L_NET_THREADS, 1)
     if (threadIdx.x == 0) epart[blockIdx.x] = es;
     __syncthreads();
     const double b = block_sum((double)bad, red);
-    if (threadIdx.x == 0 && b > 0.0) atomicAdd(invalid, (unsigned long long)b);
+    if (threadIdx.x == 0) {
+        badp[1 + blockIdx.x] = (unsigned)b;
+        if (blockIdx.x == 0) badp[0] = gridDim.x;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -641,13 +644,14 @@ __global__ void __launch_bounds__(LOOKUP_THREADS, 3) k_learned_lookup(const floa
                                                                      PointParams P, LearnedArgs la,
                                                                      float* __restrict__ specf,
                                                                      double* __restrict__ epart,
-                                                                     unsigned long long* __restrict__ invalid,
+                                                                     unsigned* __restrict__ badp,
                                                                      float* __restrict__ lw) {
     __shared__ double red[32];
     __shared__ float qm[MAX_NQ];
     __shared__ float bMq_s[LRN_M * LRN_M];
     for (int i = threadIdx.x; i < MAX_NQ; i += blockDim.x) qm[i] = P.qm[i];
     for (int i = threadIdx.x; i < LRN_M * LRN_M; i += blockDim.x) bMq_s[i] = la.bMq[i];
+    pdl_wait();
     __syncthreads();
     const long long N = g.N;
     const long long fstride = 2LL * g.N2 * g.ncols;  // floats between the planes of two channels
@@ -745,7 +749,10 @@ __global__ void __launch_bounds__(LOOKUP_THREADS, 3) k_learned_lookup(const floa
     if (threadIdx.x == 0) epart[blockIdx.x] = es;
     __syncthreads();
     const double bsum = block_sum((double)bad, red);
-    if (threadIdx.x == 0 && bsum > 0.0) atomicAdd(invalid, (unsigned long long)bsum);
+    if (threadIdx.x == 0) {
+        badp[1 + blockIdx.x] = (unsigned)bsum;
+        if (blockIdx.x == 0) badp[0] = gridDim.x;
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -888,6 +895,7 @@ __global__ void __launch_bounds__(SORTED_BLOCK, 6) k_learned_contract_gradk(
 __global__ void __launch_bounds__(256, 6) k_learned_usum(const float* __restrict__ uf, const float* __restrict__ grad,
                                                       GridArgs g, const float* __restrict__ lw, float* __restrict__ v,
                                                       float* __restrict__ w_out, float* __restrict__ g_out, int mode) {
+    pdl_wait();
     const long long N = g.N;
     const long long fstride = 2LL * g.N2 * g.ncols;
     for (long long q = blockIdx.x * (long long)blockDim.x + threadIdx.x; q < N; q += (long long)gridDim.x * blockDim.x) {
@@ -1354,6 +1362,7 @@ __global__ void __launch_bounds__(256, 2) k_pencil_grad(const float2* __restrict
     const int S = pencil_stride(L);
     Tw* tw2 = twiddles_after(sm, (size_t)4 * C * S);  // lines [4][C][S]: the field, then its three derivatives
     load_twiddles(tw2, tw, N2 - P1);
+    pdl_wait();
     const int c0 = blockIdx.x * C;
     const SmallDiv dP = small_div(P1);
     on_first<CN2, true>(L, [&](auto tag) {
@@ -1559,16 +1568,15 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
         for (int i = 0; i < VDW_NSTAGES; ++i) c->ev_done[i] = 0;
         cudaEventRecord(c->ev[0], s);
     }
-    VDW_CUDA(cudaMemsetAsync(c->d_invalid, 0, sizeof(unsigned long long), s));
     const bool want_pot = (v != nullptr) || (w != nullptr);
     if (lookup)
-        k_learned_lookup<<<nb0, LOOKUP_THREADS, 0, s>>>(n, grad, g, P, la, specf, ep, c->d_invalid,
-                                                       want_pot ? c->d_lw : nullptr);
+        launch(early_launch(g, 1), k_learned_lookup, nb0, LOOKUP_THREADS, 0, s, n, grad, g, P, la, specf, ep, c->d_bad,
+               want_pot ? c->d_lw : nullptr);
     else
     {
         const bool lw = want_pot && kind != RUN_GRAD;
-        if (lw) k_learned_net<true><<<nb0, L_NET_THREADS, smem_net(), s>>>(n, grad, g, P, la, specf, ep, c->d_invalid, c->d_lw);
-        else k_learned_net<false><<<nb0, L_NET_THREADS, smem_net(), s>>>(n, grad, g, P, la, specf, ep, c->d_invalid, nullptr);
+        if (lw) k_learned_net<true><<<nb0, L_NET_THREADS, smem_net(), s>>>(n, grad, g, P, la, specf, ep, c->d_bad, c->d_lw);
+        else k_learned_net<false><<<nb0, L_NET_THREADS, smem_net(), s>>>(n, grad, g, P, la, specf, ep, c->d_bad, nullptr);
     }
     mark(ST_POINTWISE);
     int rc = planes_inplace(c, LRN_M, false, s);
@@ -1639,7 +1647,7 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
         rc = planes_inplace(c, LRN_M, true, s);
         if (!rc) {
             mark(ST_PLANES_INV);
-            k_learned_usum<<<nb_pt, 256, 0, s>>>(specf, grad, g, c->d_lw, v, w, c->d_gg, mode);
+            launch(early_launch(g, 1), k_learned_usum, nb_pt, 256, 0, s, specf, grad, g, c->d_lw, v, w, c->d_gg, mode);
             mark(ST_USUM);
         }
         if (!rc && mode == 1) {
@@ -1661,10 +1669,12 @@ int run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, floa
 template <int CN1, int CN2, int CN3>
 void spectral_gradient(vdw_ctx* c, const float* f, float* out, cudaStream_t s) {
     const GridArgs& g = c->g;
-    k_field_plane<CN1, CN3><<<g.N2, plane_block(c, g.N2, false, true), smem_plane(g, false, true), s>>>(f, g, c->d_tw, c->d_spec);
-    k_pencil_grad<CN2><<<(g.ncols + GRAD_COLS - 1) / GRAD_COLS, 256, smem_pgrad_pencil(g), s>>>(
-        c->d_spec, c->d_wspec, g, c->d_tw + tw_off_y(g));
-    k_plane_inv3<CN1, CN3><<<dim3(g.N2, 3), plane_block(c, 3LL * g.N2, true, true), smem_plane(g, true, true), s>>>(c->d_wspec, g, c->d_tw, out);
+    launch(early_launch(g, 1), k_field_plane<CN1, CN3>, g.N2, plane_block(c, g.N2, false, true), smem_plane(g, false, true), s, f, g, c->d_tw,
+           c->d_spec);
+    launch(early_launch(g, 1), k_pencil_grad<CN2>, (g.ncols + GRAD_COLS - 1) / GRAD_COLS, 256, smem_pgrad_pencil(g), s, c->d_spec, c->d_wspec, g,
+           c->d_tw + tw_off_y(g));
+    launch(early_launch(g, 1), k_plane_inv3<CN1, CN3>, dim3(g.N2, 3), plane_block(c, 3LL * g.N2, true, true), smem_plane(g, true, true), s,
+           c->d_wspec, g, c->d_tw, out);
 }
 
 bool lrn_ready(vdw_ctx* c) {

@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(256, POINT_BLOCKS) k_pointwise(const float* __
                                                    int nbs, float* __restrict__ t_out, uint8_t* __restrict__ k_out,
                                                    float4* __restrict__ aux, float2* __restrict__ spec,
                                                    double* __restrict__ epart,
-                                                   unsigned long long* __restrict__ invalid) {
+                                                   unsigned* __restrict__ badp) {
     __shared__ double red[32];
     __shared__ SplineMesh sp;
     __shared__ float2 mp[NQ * MP_LD];
@@ -78,6 +78,7 @@ __global__ void __launch_bounds__(256, POINT_BLOCKS) k_pointwise(const float* __
     }
     load_spline_mesh(&sp, P);
     load_spline_pairs<NQ>(mp, P);
+    pdl_wait();
     __syncthreads();
     const int sl = slab >= 0 ? slab : (int)blockIdx.x / nbs;
     const int lb = slab >= 0 ? (int)blockIdx.x : (int)blockIdx.x - sl * nbs;
@@ -148,7 +149,11 @@ __global__ void __launch_bounds__(256, POINT_BLOCKS) k_pointwise(const float* __
     if (threadIdx.x == 0) epart[sl * nbs + lb] = s;
     __syncthreads();
     const double b = block_sum((double)bad, red);
-    if (threadIdx.x == 0 && b > 0.0) atomicAdd(invalid, (unsigned long long)b);
+    if (threadIdx.x == 0) {
+        const int nb = (int)(slab >= 0 ? gridDim.x * (g.N3 / 2 / nj) : gridDim.x);  // blocks of a density
+        badp[1 + blockIdx.y * nb + sl * nbs + lb] = (unsigned)b;
+        if (blockIdx.x == 0 && blockIdx.y == 0) badp[0] = nb * gridDim.y;
+    }
 }
 
 // P1 (the forward plane transforms of theta_a) is in planes.cu; P2 (y
@@ -164,7 +169,8 @@ __global__ void __launch_bounds__(256, POINT_BLOCKS) k_pointwise(const float* __
 // only u_k, u_k+1 and the two dot products m0 = sum_a u_a M_ak, m1 = sum_a
 // u_a M_a,k+1.  Then, with aux from the pointwise pass,
 //   v_loc = S0 + S1 n dq/dn + d(Delta eps)/dn,   g = S1 n dq/d|grad n| / |grad n| + ...
-// mode 0: v_loc to v (if v), w = g grad n to w_out; mode 1: v_loc to v, g to
+// mode 0: v_loc to v (if v), w = g grad n to w_out (if w_out), both times
+// gE[0] dOmega if gE; mode 1: v_loc to v, g to
 // g_out (the plane transforms of w follow in k_w_planes).
 constexpr int USUM_THREADS = 256;
 
@@ -175,7 +181,8 @@ __global__ void __launch_bounds__(USUM_THREADS, 4) k_u_sum(const float2* __restr
                                                         const float* __restrict__ tk, const uint8_t* __restrict__ kk,
                                                         const float4* __restrict__ aux, GridArgs g, PointParams P,
                                                         float* __restrict__ v, float* __restrict__ w_out,
-                                                        float* __restrict__ g_out, int mode) {
+                                                        float* __restrict__ g_out, int mode,
+                                                        const double* __restrict__ gE, double dOmega) {
     __shared__ SplineMesh sp;
     __shared__ float2 mp[NQ * MP_LD];
     {
@@ -192,7 +199,9 @@ __global__ void __launch_bounds__(USUM_THREADS, 4) k_u_sum(const float2* __restr
     }
     load_spline_mesh(&sp, P);
     load_spline_pairs<NQ>(mp, P);
+    pdl_wait();
     __syncthreads();
+    const float scale = gE ? (float)(gE[0] * dOmega) : 1.f;
     const long long N = g.N;
     const long long fstride = (long long)g.N2 * g.ncols;  // values between the planes of two fields
     const long long zs = (long long)g.N1 * g.N2;
@@ -229,11 +238,11 @@ __global__ void __launch_bounds__(USUM_THREADS, 4) k_u_sum(const float2* __restr
             const float s1 = (a1 - a0) * sp.ih[k] + ((3.f * B * B - 1.f) * b1 - (3.f * A * A - 1.f) * b0) * sp.h6[k];
             const bool ok = (s ? k1 : k0) != K_INVALID;
             const float vl = ok ? s0 + ax.x * s1 + ax.z : 0.f, gg = ok ? ax.y * s1 + ax.w : 0.f;
-            if (v) v[ii] = vl;
+            if (v) v[ii] = vl * scale;
             if (mode == 0 && w_out) {
-                w_out[ii] = gg * grad[ii];
-                w_out[N + ii] = gg * grad[N + ii];
-                w_out[2 * N + ii] = gg * grad[2 * N + ii];
+                w_out[ii] = gg * grad[ii] * scale;
+                w_out[N + ii] = gg * grad[N + ii] * scale;
+                w_out[2 * N + ii] = gg * grad[2 * N + ii] * scale;
             }
             if (mode == 1) g_out[ii] = gg;
         }
@@ -287,6 +296,7 @@ __global__ void __launch_bounds__(DIV_THREADS) k_pencil_div(float2* __restrict__
     float2* tw2s = tw2 + (N2 - P1);
     load_twiddles(tw2, tw, N2 - P1);
     load_twiddles(tw2s, tw_swap, N2 - P2);
+    pdl_wait();
     wspec += blockIdx.y * g.bs_wspec;  // density blockIdx.y of a batch
     const int c0 = blockIdx.x * C;
     on_first<CN2, true>(L, [&](auto tag) {
@@ -503,18 +513,25 @@ __global__ void k_xc_final(const double* __restrict__ Enl, const double* __restr
 }
 
 // ---------------------------------------------------------------------------
-// energy: fixed-order FP64 reduction of the block partials, in two passes
-// (the GPU's FP64 rate is low: one block summing all partials took 17 us)
+// energy: fixed-order FP64 reduction of the block partials (the GPU's FP64
+// rate is low: one block summing all partials took 17 us)
 // ---------------------------------------------------------------------------
 constexpr int ESPLIT_THREADS = 256;
 
-// First pass: block b of density blockIdx.y sums the share
-// [b n / EPART_SPLIT, (b + 1) n / EPART_SPLIT) of each partial-sum array.
-__global__ void __launch_bounds__(ESPLIT_THREADS) k_energy_split(const double* __restrict__ epart, int nb0, int nb2,
-                                                                 double* __restrict__ escr, int bs_epart) {
+// Block b of density blockIdx.y sums the share [b n / EPART_SPLIT, (b + 1) n /
+// EPART_SPLIT) of each partial-sum array; the last block to finish adds the
+// shares in index order, scaled into {E, E_soft, Delta E} (E alone if !all).
+// One launch: a second one for the 64 shares cost 4 us of a small call.
+__global__ void __launch_bounds__(ESPLIT_THREADS) k_energy(const double* __restrict__ epart, int nb0, int nb2,
+                                                           double* escr, unsigned* __restrict__ count, double s0,
+                                                           double s2, double* __restrict__ E, int all, int bs_epart) {
     __shared__ double red[32];
+    __shared__ bool last;
+    pdl_wait();
     epart += (long long)blockIdx.y * bs_epart;  // density blockIdx.y of a batch
     escr += (long long)blockIdx.y * bs_epart;
+    E += (all ? 3 : 1) * blockIdx.y;
+    count += blockIdx.y;
     const long long b = blockIdx.x;
     const int lo0 = (int)(b * nb0 / EPART_SPLIT), hi0 = (int)((b + 1) * nb0 / EPART_SPLIT);
     const int lo2 = (int)(b * nb2 / EPART_SPLIT), hi2 = (int)((b + 1) * nb2 / EPART_SPLIT);
@@ -525,26 +542,26 @@ __global__ void __launch_bounds__(ESPLIT_THREADS) k_energy_split(const double* _
     __syncthreads();
     const double t2 = block_sum(a2, red);
     if (threadIdx.x == 0) {
-        escr[b] = t0;
-        escr[EPART_SPLIT + b] = t2;
+        __stcg(escr + b, t0);
+        __stcg(escr + EPART_SPLIT + b, t2);
+        __threadfence();
+        last = atomicAdd(count, 1u) == EPART_SPLIT - 1;
     }
-}
-
-// Second pass (EPART_SPLIT threads per density): the shares in index order,
-// scaled into {E, E_soft, Delta E}.
-__global__ void __launch_bounds__(EPART_SPLIT) k_energy_final(const double* __restrict__ escr, double s0, double s2,
-                                                              double* __restrict__ E, int bs_epart) {
-    __shared__ double red[32];
-    escr += (long long)blockIdx.x * bs_epart;  // density blockIdx.x of a batch
-    E += 3 * blockIdx.x;
-    const double t0 = block_sum(escr[threadIdx.x], red);
     __syncthreads();
-    const double t2 = block_sum(escr[EPART_SPLIT + threadIdx.x], red);
+    if (!last) return;
+    __threadfence();
+    const int i = threadIdx.x;
+    const double u0 = block_sum(i < EPART_SPLIT ? __ldcg(escr + i) : 0.0, red);
+    __syncthreads();
+    const double u2 = block_sum(i < EPART_SPLIT ? __ldcg(escr + EPART_SPLIT + i) : 0.0, red);
     if (threadIdx.x == 0) {
-        const double dE = s0 * t0, Es = s2 * t2;
+        const double dE = s0 * u0, Es = s2 * u2;
         E[0] = Es + dE;
-        E[1] = Es;
-        E[2] = dE;
+        if (all) {
+            E[1] = Es;
+            E[2] = dE;
+        }
+        *count = 0;
     }
 }
 
@@ -751,12 +768,14 @@ static int u_sum_blocks(const vdw_ctx* c) {
                                     (long long)std::max(c->usum_per_sm, 1) * std::max(c->nsm, 1));
 }
 
-static int launch_u_sum(vdw_ctx* c, const float* n, const float* grad, float* v, float* w, int mode, cudaStream_t s,
-                        int B) {
+static int launch_u_sum(vdw_ctx* c, const float* grad, float* v, float* w, int mode, cudaStream_t s, int B,
+                        GradScale gs) {
     const GridArgs& g = c->g;
     const int nb = u_sum_blocks(c);
+    const double dOmega = c->L[0] * c->L[1] * c->L[2] / (double)g.N;
 #define VDW_U_SUM(NQ) \
-    k_u_sum<NQ><<<dim3(nb, B), USUM_THREADS, 0, s>>>(c->d_spec, grad, c->d_t, c->d_k, c->d_aux, g, c->pp, v, w, c->d_gg, mode)
+    launch(early_launch(g, B), k_u_sum<NQ>, dim3(nb, B), USUM_THREADS, 0, s, c->d_spec, grad, c->d_t, c->d_k, c->d_aux, g, c->pp, v, w, \
+           c->d_gg, mode, gs.on ? gs.gE : nullptr, dOmega)
     switch (c->pp.Nq) {
         case 20: VDW_U_SUM(20); break;
         case 8: VDW_U_SUM(8); break;
@@ -770,7 +789,7 @@ static int launch_u_sum(vdw_ctx* c, const float* n, const float* grad, float* v,
 
 template <int CN1, int CN2, int CN3>
 static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, float* w, cudaStream_t s,
-                     int fd, int xc, const cudaEvent_t* slab_ready, int B) {
+                     int fd, int xc, const cudaEvent_t* slab_ready, int B, GradScale gs) {
     const GridArgs& g = c->g;
     const PointParams& P = c->pp;
     const bool want_pot = (v != nullptr) || (w != nullptr);
@@ -785,7 +804,6 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
         for (int i = 0; i < VDW_NSTAGES; ++i) c->ev_done[i] = 0;
         cudaEventRecord(c->ev[0], s);
     }
-    VDW_CUDA(cudaMemsetAsync(c->d_invalid, 0, sizeof(unsigned long long), s));
     // one launch over all slabs, or (host entry point) one per slab as its inputs arrive
     const int nlaunch = slab_ready ? c->p0_chunks : 1;
     for (int sl = 0; sl < nlaunch; ++sl) {
@@ -793,8 +811,8 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
         const int slab = slab_ready ? sl : -1;
         const int nblk = slab_ready ? c->nb_p0 : c->nb_point;
 #define VDW_POINTWISE(NQ)                                                                                  \
-    k_pointwise<NQ><<<dim3(nblk, B), 256, 0, s>>>(n, grad, g, P, slab, c->p0_nj, c->p0_mnj, c->nb_p0, c->d_t, c->d_k, \
-                                         c->d_aux, c->d_spec, c->d_epart, c->d_invalid)
+    launch(early_launch(g, B), k_pointwise<NQ>, dim3(nblk, B), 256, 0, s, n, grad, g, P, slab, c->p0_nj, c->p0_mnj, c->nb_p0, c->d_t, \
+           c->d_k, c->d_aux, c->d_spec, c->d_epart, c->d_bad)
         switch (P.Nq) {
             case 20: VDW_POINTWISE(20); break;
             case 8: VDW_POINTWISE(8); break;
@@ -836,9 +854,9 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
             VDW_CUDA(cudaStreamWaitEvent(c->s_side, c->ev_fork, 0));
             se = c->s_side;
         }
-        k_energy_split<<<dim3(EPART_SPLIT, B), ESPLIT_THREADS, 0, se>>>(c->d_epart, c->nb_point, c->nb_sorted, escr,
-                                                                        g.bs_epart);
-        k_energy_final<<<B, EPART_SPLIT, 0, se>>>(escr, Omega / Nd, 0.5 * Omega / (Nd * Nd), E, g.bs_epart);
+        launch(se == s && early_launch(g, B), k_energy, dim3(EPART_SPLIT, B), ESPLIT_THREADS, 0, se, c->d_epart,
+               c->nb_point, c->nb_sorted, escr, c->d_ecount, Omega / Nd, 0.5 * Omega / (Nd * Nd), E, gs.on ? 0 : 1,
+               g.bs_epart);
         if (se != s) {
             VDW_CUDA(cudaEventRecord(c->ev_join, se));
             forked = true;
@@ -854,14 +872,14 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
             return rc;
         }
         mark(ST_PENCILS_INV);
-        const int mode = (w != nullptr) ? 0 : 1;
+        const int mode = (w != nullptr || gs.on) ? 0 : 1;
         rc = planes_inplace(c, P.Nq, true, s, B);
         if (rc) {
             join();
             return rc;
         }
         mark(ST_PLANES_INV);
-        const int rcs = launch_u_sum(c, n, grad, v, w, mode, s, B);
+        const int rcs = launch_u_sum(c, grad, v, w, mode, s, B, gs);
         if (rcs) {
             join();
             return rcs;
@@ -875,14 +893,14 @@ static int run_sized(vdw_ctx* c, const float* n, const float* grad, double* E, f
             k_stencil_div_sub<<<stencil_blocks(g), 256, 0, s>>>(c->d_gg, grad, g, stencil_ih2(c), v);
             mark(ST_DIV_FINAL);
         } else if (mode == 1) {
-            k_w_planes<CN1, CN3><<<dim3(g.N2, 3, B), plane_block(c, 3LL * g.N2 * B, false, false),
-                                   smem_plane(g, false, false), s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
+            launch(early_launch(g, B), k_w_planes<CN1, CN3>, dim3(g.N2, 3, B), plane_block(c, 3LL * g.N2 * B, false, false),
+                   smem_plane(g, false, false), s, c->d_gg, grad, g, c->d_tw, c->d_wspec);
             mark(ST_W_PLANES);
-            k_pencil_div<CN2><<<dim3((g.ncols + DIV_COLS - 1) / DIV_COLS, B), DIV_THREADS, smem_div(g), s>>>(
-                c->d_wspec, g, c->d_tw + tw_off_y(g), c->d_tw + tw_off_swap(g));
+            launch(early_launch(g, B), k_pencil_div<CN2>, dim3((g.ncols + DIV_COLS - 1) / DIV_COLS, B), DIV_THREADS, smem_div(g), s,
+                   c->d_wspec, g, c->d_tw + tw_off_y(g), c->d_tw + tw_off_swap(g));
             mark(ST_PENCIL_DIV);
-            k_div_final<CN1, CN3><<<dim3(g.N2, B), plane_block(c, (long long)g.N2 * B, true, false),
-                                    smem_plane(g, true, false), s>>>(c->d_wspec, g, c->d_tw, v);
+            launch(early_launch(g, B), k_div_final<CN1, CN3>, dim3(g.N2, B), plane_block(c, (long long)g.N2 * B, true, false),
+                   smem_plane(g, true, false), s, c->d_wspec, g, c->d_tw, v);
             mark(ST_DIV_FINAL);
         }
     }
@@ -925,15 +943,17 @@ int pipeline_configure(vdw_ctx* c) {
 template <int CN1, int CN2, int CN3>
 static void launch_divergence(vdw_ctx* c, float* v, cudaStream_t s) {
     const GridArgs& g = c->g;
-    k_pencil_div<CN2><<<(g.ncols + DIV_COLS - 1) / DIV_COLS, DIV_THREADS, smem_div(g), s>>>(
-        c->d_wspec, g, c->d_tw + tw_off_y(g), c->d_tw + tw_off_swap(g));
-    k_div_final<CN1, CN3><<<g.N2, plane_block(c, g.N2, true, false), smem_plane(g, true, false), s>>>(c->d_wspec, g, c->d_tw, v);
+    launch(early_launch(g, 1), k_pencil_div<CN2>, (g.ncols + DIV_COLS - 1) / DIV_COLS, DIV_THREADS, smem_div(g), s,
+                   c->d_wspec, g, c->d_tw + tw_off_y(g), c->d_tw + tw_off_swap(g));
+    launch(early_launch(g, 1), k_div_final<CN1, CN3>, g.N2, plane_block(c, g.N2, true, false),
+                   smem_plane(g, true, false), s, c->d_wspec, g, c->d_tw, v);
 }
 
 template <int CN1, int CN3>
 static void launch_w_planes(vdw_ctx* c, const float* grad, cudaStream_t s) {
     const GridArgs& g = c->g;
-    k_w_planes<CN1, CN3><<<dim3(g.N2, 3), plane_block(c, 3LL * g.N2, false, false), smem_plane(g, false, false), s>>>(c->d_gg, grad, g, c->d_tw, c->d_wspec);
+    launch(early_launch(g, 1), k_w_planes<CN1, CN3>, dim3(g.N2, 3), plane_block(c, 3LL * g.N2, false, false),
+                   smem_plane(g, false, false), s, c->d_gg, grad, g, c->d_tw, c->d_wspec);
 }
 
 int pipeline_w_planes(vdw_ctx* c, const float* grad, cudaStream_t s) {
@@ -959,17 +979,17 @@ int pipeline_energy_final(vdw_ctx* c, const double* epart, int nb0, int nb2, dou
     const double Nd = (double)c->g.N;
     // the shares go to the context's own scratch (after density 0's partial sums)
     double* escr = c->d_epart + c->nb_point + c->nb_sorted;
-    k_energy_split<<<dim3(EPART_SPLIT, 1), ESPLIT_THREADS, 0, s>>>(epart, nb0, nb2, escr, 0);
-    k_energy_final<<<1, EPART_SPLIT, 0, s>>>(escr, Omega / Nd, 0.5 * Omega / (Nd * Nd), E, 0);
+    launch(early_launch(c->g, 1), k_energy, dim3(EPART_SPLIT, 1), ESPLIT_THREADS, 0, s, epart, nb0, nb2, escr, c->d_ecount,
+           Omega / Nd, 0.5 * Omega / (Nd * Nd), E, 1, 0);
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;
 }
 
 int pipeline_run(vdw_ctx* c, const float* n, const float* grad, double* E, float* v, float* w, cudaStream_t s,
-                 int fd, int xc, const cudaEvent_t* slab_ready, int B) {
+                 int fd, int xc, const cudaEvent_t* slab_ready, int B, GradScale gs) {
     return on_grid(c->g, [&](auto d) {
         using D = decltype(d);
-        return run_sized<D::N1, D::N2, D::N3>(c, n, grad, E, v, w, s, fd, xc, slab_ready, B);
+        return run_sized<D::N1, D::N2, D::N3>(c, n, grad, E, v, w, s, fd, xc, slab_ready, B, gs);
     });
 }
 

@@ -211,6 +211,7 @@ __device__ __forceinline__ void plane_forward(float2* sm, const GridArgs& g, con
     W* tw3 = tw1 + (N1 - P1);
     load_twiddles(tw1, tw, N1 - P1);
     load_twiddles(tw3, tw + g.N1 + g.N2, N3 - Q1);
+    pdl_wait();
     const int t0 = threadIdx.x, nt = blockDim.x;
     on_first<CN1, false>(g.p1, [&](auto tag) {
         using R = decltype(tag);
@@ -361,6 +362,7 @@ __device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, con
     W* tw3 = tw1 + (N1 - P1);
     load_twiddles(tw1, tw, N1 - P1);
     load_twiddles(tw3, tw + g.N1 + g.N2, N3 - Q1);
+    pdl_wait();
     const int t0 = threadIdx.x, nt = blockDim.x;
     constexpr int CH = CN1 > 0 ? CN1 / 2 + 1 : 0;
     const SmallDiv dh = small_div(Nh), dP = small_div(G.run);

@@ -59,8 +59,8 @@ int planes_inplace(vdw_ctx* c, int nfields, bool inverse, cudaStream_t s, int B)
     const size_t sm = smem_plane(g, inverse, !inverse);
     on_grid(g, [&](auto d) {
         using D = decltype(d);
-        if (inverse) k_planes_inplace<D::N1, D::N3, true><<<grid, nt, sm, s>>>(c->d_spec, g, c->d_tw);
-        else k_planes_inplace<D::N1, D::N3, false><<<grid, nt, sm, s>>>(c->d_spec, g, c->d_tw);
+        if (inverse) launch(early_launch(g, B), k_planes_inplace<D::N1, D::N3, true>, grid, nt, sm, s, c->d_spec, g, c->d_tw);
+        else launch(early_launch(g, B), k_planes_inplace<D::N1, D::N3, false>, grid, nt, sm, s, c->d_spec, g, c->d_tw);
     });
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;

@@ -71,6 +71,7 @@ class Params:
 
 
 EXPORTS = ["vdw_params_default", "vdw_kernel_table", "vdw_create", "vdw_plan", "vdw_energy_potential",
+           "vdw_energy_gradients",
            "vdw_plan_batch", "vdw_plan_cell", "vdw_energy_potential_batched",
            "vdw_energy_potential_fd", "vdw_xc_energy_potential",
            "vdw_energy_potential_host", "vdw_last_invalid_points", "vdw_profile_enable", "vdw_profile_read",
@@ -100,6 +101,7 @@ def lib():
     L.vdw_create.argtypes = [P(vp), P(_Params), dp, ctypes.c_double]
     L.vdw_plan.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, dp]
     L.vdw_energy_potential.argtypes = [vp, vp, vp, vp, vp, vp, vp]
+    L.vdw_energy_gradients.argtypes = [vp, vp, vp, vp, vp, vp, vp, vp]
     L.vdw_energy_potential_host.argtypes = [vp, fp, fp, dp, fp, vp]
     L.vdw_plan_batch.argtypes = [vp, ctypes.c_int]
     L.vdw_plan_cell.argtypes = [vp, ctypes.c_int, ctypes.c_int, ctypes.c_int, dp]
@@ -244,6 +246,21 @@ class VdwNL:
         _check(lib().vdw_energy_potential(self._h, ptr(n), ptr(grad), ptr(E), ptr(v), ptr(w),
                                           _stream_handle(stream)), "vdw_energy_potential")
         return E, v, w
+
+    def energy_gradients(self, n, grad, gE=None, E=None, dn=None, dg=None):
+        """vdw_energy_gradients on torch's current stream (contiguous FP32 device
+        tensors; gE, E FP64 device scalars)."""
+        import torch
+        _cuda_f32(n, self.shape)
+        _cuda_f32(grad, (3,) + self.shape)
+        for t, s in ((dn, self.shape), (dg, (3,) + self.shape)):
+            if t is not None:
+                _cuda_f32(t, s)
+        for t in (gE, E):
+            assert t is None or (t.is_cuda and t.dtype == torch.float64 and t.numel() == 1)
+        p = [None if t is None else t.data_ptr() for t in (n, grad, gE, E, dn, dg)]
+        _check(lib().vdw_energy_gradients(self._h, *p, torch.cuda.current_stream().cuda_stream),
+               "vdw_energy_gradients")
 
     def plan_batch(self, Bmax):
         """vdw_plan_batch: workspaces for Bmax densities per call (after plan())."""
