@@ -220,6 +220,12 @@ __device__ __forceinline__ void pdl_wait() {
     asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
+// Asks for bytes of global memory (16-byte aligned, a multiple of 16 bytes) to
+// be brought into L2: one thread of a block does it for the block that will
+// take its place on the SM, whose first loads then miss L1 only.
+__device__ __forceinline__ void prefetch_l2(const void* p, unsigned bytes) {
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(__cvta_generic_to_global(p)), "r"(bytes) : "memory");
+}
 // early: small grids only (early_launch), where launch latency and the first
 // loads are a good part of a kernel; the blocks that wait take shared memory
 // and L1 from the running kernel, which costs a large grid more (24^3 74 -> 53

@@ -221,6 +221,23 @@ __global__ void __launch_bounds__(PEN_THREADS, 3) k_pencil_inv(float2* __restric
 // 24^3, 25 -> 14 us at 48^3).
 constexpr int CONTRACT_ROWS = 4;  // table rows staged per block at most
 
+// One record (four fields of a point): 32 bytes by one access.  As two 16-byte
+// accesses every lane's half sector went through L1 twice (contraction of 8 x
+// 144 x 144 x 72 518 us against 498, 256 x 256 x 96 274 against 268).
+__device__ __forceinline__ void load_record(const float4* p, float2* v) {
+    asm volatile("ld.global.v8.f32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+                 : "=f"(v[0].x), "=f"(v[0].y), "=f"(v[1].x), "=f"(v[1].y), "=f"(v[2].x), "=f"(v[2].y), "=f"(v[3].x),
+                   "=f"(v[3].y)
+                 : "l"(__cvta_generic_to_global(p))
+                 : "memory");
+}
+__device__ __forceinline__ void store_record(float4* p, const float2* v, float s) {
+    asm volatile("st.global.v8.f32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(__cvta_generic_to_global(p)),
+                 "f"(v[0].x * s), "f"(v[0].y * s), "f"(v[1].x * s), "f"(v[1].y * s), "f"(v[2].x * s), "f"(v[2].y * s),
+                 "f"(v[3].x * s), "f"(v[3].y * s)
+                 : "memory");
+}
+
 // u += Phi(t) theta with the row's pair coefficients cf
 template <int NQ>
 __device__ __forceinline__ void pair_loop(const float4* cf, float t, const float2 (&th)[NQ], float2 (&u)[NQ]) {
@@ -257,13 +274,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 4) k_contract_sorted(float4* __r
     const long long r = r0 + threadIdx.x;
     float2 th[NQ];
 #pragma unroll
-    for (int q = 0; q < NQ / 4; ++q) {
-        const float4 a = Q[q * qstride + 2 * r], b = Q[q * qstride + 2 * r + 1];
-        th[4 * q] = make_float2(a.x, a.y);
-        th[4 * q + 1] = make_float2(a.z, a.w);
-        th[4 * q + 2] = make_float2(b.x, b.y);
-        th[4 * q + 3] = make_float2(b.z, b.w);
-    }
+    for (int q = 0; q < NQ / 4; ++q) load_record(Q + q * qstride + 2 * r, th + 4 * q);
     const float gm = gs[r];
     const float wgt = signbit(gm) ? 1.f : 2.f;
     const float s = fabsf(gm) * inv_dk;
@@ -293,12 +304,7 @@ __global__ void __launch_bounds__(SORT_THREADS, 4) k_contract_sorted(float4* __r
     if (threadIdx.x == 0) epart[blockIdx.x] = es;
     if (!write_back) return;
 #pragma unroll
-    for (int q = 0; q < NQ / 4; ++q) {
-        Q[q * qstride + 2 * r] =
-            make_float4(u[4 * q].x * invN, u[4 * q].y * invN, u[4 * q + 1].x * invN, u[4 * q + 1].y * invN);
-        Q[q * qstride + 2 * r + 1] =
-            make_float4(u[4 * q + 2].x * invN, u[4 * q + 2].y * invN, u[4 * q + 3].x * invN, u[4 * q + 3].y * invN);
-    }
+    for (int q = 0; q < NQ / 4; ++q) store_record(Q + q * qstride + 2 * r, u + 4 * q, invN);
 }
 
 // The same with two points per thread, r and r + 64 of the block's 128, in

@@ -2,6 +2,9 @@
 // u_a, in place.
 #include "plane.cuh"
 
+#include <algorithm>
+#include <climits>
+
 namespace vdw {
 
 // One block per (y plane, field).  Both sides of the transform keep the
@@ -24,11 +27,15 @@ namespace vdw {
 // 266 -> 116 / 113, 100^3 174 / 171 -> 64 / 65.
 template <int CN1, int CN3, bool INV>
 __global__ void __launch_bounds__(PLANE_THREADS, 2)
-    k_planes_inplace(float2* __restrict__ spec, GridArgs g, const Tw* __restrict__ tw) {
+    k_planes_inplace(float2* __restrict__ spec, GridArgs g, const Tw* __restrict__ tw, int ahead) {
     extern __shared__ float2 sm[];
     const int Nh = CN1 > 0 ? CN1 / 2 + 1 : g.Nh;
     const int y = blockIdx.x, a = blockIdx.y;
     float2* p = spec + blockIdx.z * g.bs_spec + ((long long)a * g.N2 + y) * g.ncols;
+    // the planes of a launch are contiguous in block order
+    const long long left = (long long)gridDim.x * gridDim.y * gridDim.z - 1 -
+                           (y + (long long)gridDim.x * (a + (long long)gridDim.y * blockIdx.z));
+    if (threadIdx.x == 0 && ahead <= left) prefetch_l2(p + (long long)ahead * g.ncols, (unsigned)sizeof(float2) * g.ncols);
     const auto row_at = [&](int row, int x) { return p + (row * 2 * Nh + x); };
     const auto pt_at = [&](int kz, int kx) { return p + (kz * Nh + kx); };
     // the forward transforms of theta feed the energy: hi/lo twiddles there
@@ -57,10 +64,16 @@ int planes_inplace(vdw_ctx* c, int nfields, bool inverse, cudaStream_t s, int B)
     const dim3 grid(g.N2, nfields, B);
     const int nt = plane_block(c, (long long)g.N2 * nfields * B, inverse, !inverse);
     const size_t sm = smem_plane(g, inverse, !inverse);
+    // Where an SM holds two planes at most, a block asks L2 for the plane of the
+    // block that follows it (256 x 256 x 96: 285 -> 274 us; with three blocks
+    // per SM the others hide that latency, and 128^3 takes 104 us against 101);
+    // with fewer fields than planned the densities are not contiguous.
+    const int per_sm = std::max(1, std::min((int)(228 * 1024 / (sm + 1024)), 2 * PLANE_THREADS / nt));
+    const int ahead = per_sm > 2 || (B > 1 && nfields != c->p.Nq) ? INT_MAX : std::max(1, c->nsm) * per_sm;
     on_grid(g, [&](auto d) {
         using D = decltype(d);
-        if (inverse) launch(early_launch(g, B), k_planes_inplace<D::N1, D::N3, true>, grid, nt, sm, s, c->d_spec, g, c->d_tw);
-        else launch(early_launch(g, B), k_planes_inplace<D::N1, D::N3, false>, grid, nt, sm, s, c->d_spec, g, c->d_tw);
+        if (inverse) launch(early_launch(g, B), k_planes_inplace<D::N1, D::N3, true>, grid, nt, sm, s, c->d_spec, g, c->d_tw, ahead);
+        else launch(early_launch(g, B), k_planes_inplace<D::N1, D::N3, false>, grid, nt, sm, s, c->d_spec, g, c->d_tw, ahead);
     });
     VDW_CUDA(cudaGetLastError());
     return VDW_OK;
