@@ -65,6 +65,7 @@ struct GridArgs {
     int Nk;                // points of the radial table
     float invN;            // 1 / N
     LinePlan p1, p2, p3;   // line transforms along x, y, z
+    LinePlan p1i;          // inverse along x of u and D.w (its groups may be in the other order)
     int pad_fwd, pad_inv;  // plane transforms with padded rows (plane_geo)
     // Flat-index divisions by N1, N2 and N3/2 as multiply-high by
     // m = ceil(2^32 / d), exact for i d < 2^32; fast = 0 (plain division)
@@ -362,5 +363,6 @@ inline bool sized_grid(int n1, int n2, int n3) {
 // offsets of the twiddle tables in d_tw (entries)
 inline int tw_off_y(const GridArgs& g) { return g.N1; }
 inline int tw_off_swap(const GridArgs& g) { return g.N1 + g.N2 + g.N3; }
+__host__ __device__ inline int tw_off_xi(const GridArgs& g) { return g.N1 + 2 * g.N2 + g.N3; }
 
 }  // namespace vdw

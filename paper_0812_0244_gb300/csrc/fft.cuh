@@ -430,11 +430,14 @@ __device__ __forceinline__ void group_fft(float2 (&v)[G::P], const W* tw, int Ns
 // Compile-time lengths (the grids 180 x 180 x 72 and 256 x 256 x 96): two
 // in-register radices each.  Any other length takes its groups at run time
 // from the list 4, .., 4, 2, 3, .., 3, 5, .., 5 (make_line_plan).
-template <int CN> struct CtLine { using G1 = Grp<1>; using G2 = Grp<1>; };
-template <> struct CtLine<180> { using G1 = Grp<15>; using G2 = Grp<12>; };
-template <> struct CtLine<72> { using G1 = Grp<9>; using G2 = Grp<8>; };
-template <> struct CtLine<256> { using G1 = Grp<16>; using G2 = Grp<16>; };
-template <> struct CtLine<96> { using G1 = Grp<12>; using G2 = Grp<8>; };
+// CtLine<N, true>: the order of the inverse x transforms of u and D.w
+// (LinePlan p1i).
+template <int CN, bool XI = false> struct CtLine { using G1 = Grp<1>; using G2 = Grp<1>; };
+template <> struct CtLine<180, false> { using G1 = Grp<15>; using G2 = Grp<12>; };
+template <> struct CtLine<180, true> { using G1 = Grp<12>; using G2 = Grp<15>; };
+template <> struct CtLine<72, false> { using G1 = Grp<9>; using G2 = Grp<8>; };
+template <bool XI> struct CtLine<256, XI> { using G1 = Grp<16>; using G2 = Grp<16>; };
+template <> struct CtLine<96, false> { using G1 = Grp<12>; using G2 = Grp<8>; };
 
 // Run-time lengths: any, or (ANY16) with no group above 16.  The second kind
 // leaves the larger groups' registers out of a kernel.
@@ -480,7 +483,8 @@ __device__ __forceinline__ void first_group(int P, F&& f) {
             }
     }
 }
-template <bool BIG, class F>
+// WIDE: also the groups that are second only in an inverse x transform
+template <bool BIG, bool WIDE, class F>
 __device__ __forceinline__ void second_group(int P, F&& f) {
     switch (P) {
         case 1: f(Grp<1>{}); break;
@@ -499,17 +503,22 @@ __device__ __forceinline__ void second_group(int P, F&& f) {
             if constexpr (BIG) {
                 if (P == 25) f(Grp<5, 5>{});
             }
+            if constexpr (BIG && WIDE) {
+                if (P == 18) f(Grp<2, 3, 3>{});
+                if (P == 20) f(Grp<4, 5>{});
+                if (P == 24) f(Grp<4, 2, 3>{});
+            }
     }
 }
-template <int CN, bool ODD, class F>
+template <int CN, bool ODD, bool XI = false, class F>
 __device__ __forceinline__ void on_first(const LinePlan& lp, F&& f) {
-    if constexpr (CN > 0) f(typename CtLine<CN>::G1{});
-    else first_group<ODD, CN == ANY>(lp.P1, f);
+    if constexpr (CN > 0) f(typename CtLine<CN, XI>::G1{});
+    else first_group<ODD || XI, CN == ANY>(lp.P1, f);
 }
-template <int CN, class F>
+template <int CN, bool XI = false, class F>
 __device__ __forceinline__ void on_second(const LinePlan& lp, F&& f) {
-    if constexpr (CN > 0) f(typename CtLine<CN>::G2{});
-    else second_group<CN == ANY>(lp.P2, f);
+    if constexpr (CN > 0) f(typename CtLine<CN, XI>::G2{});
+    else second_group<CN == ANY, XI>(lp.P2, f);
 }
 
 }  // namespace vdw

@@ -681,9 +681,10 @@ static int best_threads(std::initializer_list<Pass> passes, int lo, int hi) {
 // shared memory of a plane kernel, forward or inverse, with hi/lo (exact) or
 // FP32 twiddles
 static size_t smem_plane_of(const GridArgs& g, bool inverse, bool exact, bool pad) {
-    const PlaneGeo p = plane_geo(g.p1.P1, g.p1.P2, inverse, pad);
+    const LinePlan& l = inverse && !exact ? g.p1i : g.p1;
+    const PlaneGeo p = plane_geo(l.P1, l.P2, inverse, pad);
     return sizeof(float2) * tw_offset((size_t)(g.N3 / 2) * p.S) +
-           (exact ? sizeof(Tw) : sizeof(float2)) * ((size_t)(g.N1 - g.p1.P1) + (g.N3 - g.p3.P1));
+           (exact ? sizeof(Tw) : sizeof(float2)) * ((size_t)(g.N1 - l.P1) + (g.N3 - g.p3.P1));
 }
 size_t smem_plane(const GridArgs& g, bool inverse, bool exact) {
     return smem_plane_of(g, inverse, exact, inverse ? g.pad_inv : g.pad_fwd);
@@ -708,8 +709,11 @@ int plane_block(const vdw_ctx* c, long long nblocks, bool inverse, bool exact) {
     const int items = std::max({nr * g.p1.P2, nr * g.p1.P1, g.Nh * g.p3.P2, g.Nh * g.p3.P1});
     const int hi = std::min((int)std::min<long long>(most, 2 * most / per_sm) / 32 * 32, (items + 31) / 32 * 32);
     const int lo = std::min(hi, (int)(2 * most / (per_sm + 1)) / 32 * 32 + 32);  // no room for another block
-    const Pass second = fused ? Pass{nr * (g.p1.P1 / 2 + 1), 2 * g.p1.P2} : Pass{nr * g.p1.P1, g.p1.P2};
-    return best_threads({{nr * g.p1.P2, g.p1.P1}, second, {fused ? 0 : g.Nh * nr, 2}, {g.Nh * g.p3.P2, g.p3.P1},
+    const bool merged = inverse && !exact && on_grid(g, [&](auto d) { return g.p1i.P1 <= MERGE_P<decltype(d)::N1>; });
+    const LinePlan& l = inverse && !exact ? g.p1i : g.p1;
+    const Pass first = merged ? Pass{nr * (l.P2 / 2 + 1), 2 * l.P1} : Pass{nr * l.P2, l.P1};
+    const Pass second = fused ? Pass{nr * (l.P1 / 2 + 1), 2 * l.P2} : Pass{nr * l.P1, l.P2};
+    return best_threads({first, second, {fused || merged ? 0 : g.Nh * nr, 2}, {g.Nh * g.p3.P2, g.p3.P1},
                          {g.Nh * g.p3.P1, g.p3.P2}},
                         lo, hi);
 }
@@ -724,10 +728,11 @@ static const size_t SMEM_MAX = 227 * 1024 - 1024;
 int pipeline_plan_check(vdw_ctx* c) {
     GridArgs& g = c->g;
     g.pad_fwd = smem_plane_of(g, false, true, true) <= SMEM_MAX;
-    g.pad_inv = smem_plane_of(g, true, true, true) <= SMEM_MAX;
+    g.pad_inv = smem_plane_of(g, true, true, true) <= SMEM_MAX && smem_plane_of(g, true, false, true) <= SMEM_MAX;
     // the whole-plane limit of the unpadded rows
     if (sizeof(float2) * (size_t)g.N3 * g.Nh + sizeof(Tw) * (g.N1 + g.N3) > 222 * 1024 ||
-        smem_plane(g, false, true) > SMEM_MAX || smem_plane(g, true, true) > SMEM_MAX || sorted_pencil_smem(g) > SMEM_MAX || smem_div(g) > SMEM_MAX)
+        smem_plane(g, false, true) > SMEM_MAX || smem_plane(g, true, true) > SMEM_MAX ||
+        smem_plane(g, true, false) > SMEM_MAX || sorted_pencil_smem(g) > SMEM_MAX || smem_div(g) > SMEM_MAX)
         return VDW_ERR_SIZE;
     return VDW_OK;
 }
@@ -743,6 +748,7 @@ int pipeline_make_twiddles(vdw_ctx* c) {
     make(tw_off_y(g), g.N2, g.p2.P1, g.p2.P2);
     make(g.N1 + g.N2, g.N3, g.p3.P1, g.p3.P2);
     make(tw_off_swap(g), g.N2, g.p2.P2, g.p2.P1);
+    make(tw_off_xi(g), g.N1, g.p1i.P1, g.p1i.P2);
     VDW_CUDA(cudaGetLastError());
     VDW_CUDA(cudaDeviceSynchronize());
     return VDW_OK;

@@ -149,13 +149,14 @@ __host__ __device__ constexpr PlaneGeo plane_geo(int P1, int P2, bool inverse, b
     const int len = run * cnt + ((cnt - 1) >> sh);
     return PlaneGeo{run, sh, len, pad ? ((len + 2) | 1) : len + 2};
 }
-template <int CN1, bool INVERSE>
+template <int CN1, bool INVERSE, bool XI = false>
 __device__ __forceinline__ PlaneGeo geo_of(const GridArgs& g) {
     if constexpr (CN1 > 0) {
-        constexpr PlaneGeo p = plane_geo(CtLine<CN1>::G1::P, CtLine<CN1>::G2::P, INVERSE, true);
+        constexpr PlaneGeo p = plane_geo(CtLine<CN1, XI>::G1::P, CtLine<CN1, XI>::G2::P, INVERSE, true);
         return p;
     } else {
-        return plane_geo(g.p1.P1, g.p1.P2, INVERSE, INVERSE ? g.pad_inv : g.pad_fwd);
+        const LinePlan& l = XI ? g.p1i : g.p1;
+        return plane_geo(l.P1, l.P2, INVERSE, INVERSE ? g.pad_inv : g.pad_fwd);
     }
 }
 // the slots of kx for the even and the odd real row
@@ -180,6 +181,13 @@ __device__ __forceinline__ float2 split_even(float2 f, float2 s) {
 __device__ __forceinline__ float2 split_odd(float2 f, float2 s) {
     return make_float2(0.5f * (f.y + s.y), -0.5f * (f.x - s.x));
 }
+// The inverse: Z_k and Z_{-k} of Z = A + i B from A_k = a and B_k = b.  A first
+// group of at most MERGE_P points does it in registers, for k and N1 - k in
+// one thread; otherwise it is a pass of its own.
+template <int CN1>
+constexpr int MERGE_P = CN1 == 180 ? 12 : CN1 > 0 ? 0 : 9;
+__device__ __forceinline__ float2 merge_pos(float2 a, float2 b) { return make_float2(a.x - b.y, a.y + b.x); }
+__device__ __forceinline__ float2 merge_neg(float2 a, float2 b) { return make_float2(a.x + b.y, b.x - a.y); }
 // position of (z, kx): even and odd real rows of a complex row at slots se, so
 __device__ __forceinline__ int zpos(int z, int S, int se, int so) { return (z >> 1) * S + ((z & 1) ? so : se); }
 
@@ -355,12 +363,14 @@ template <int CN1, int CN3, class W, class LD, class ST>
 __device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, const Tw* __restrict__ tw, LD ld, ST st) {
     const int N1 = CN1 > 0 ? CN1 : g.N1, N3 = CN3 > 0 ? CN3 : g.N3;
     const int Nh = N1 / 2 + 1, nr = N3 / 2;
-    const PlaneGeo G = geo_of<CN1, true>(g);
+    constexpr bool XI = sizeof(W) < sizeof(Tw);  // (the gradient keeps the forward order)
+    const LinePlan& lx = XI ? g.p1i : g.p1;
+    const PlaneGeo G = geo_of<CN1, true, XI>(g);
     const int S = G.S;
-    const int P1 = CN1 > 0 ? CtLine<CN1>::G1::P : g.p1.P1, Q1 = CN3 > 0 ? CtLine<CN3>::G1::P : g.p3.P1;
+    const int P1 = CN1 > 0 ? CtLine<CN1, XI>::G1::P : lx.P1, Q1 = CN3 > 0 ? CtLine<CN3>::G1::P : g.p3.P1;
     W* tw1 = twiddles_after<W>(sm, (size_t)nr * S);
     W* tw3 = tw1 + (N1 - P1);
-    load_twiddles(tw1, tw, N1 - P1);
+    load_twiddles(tw1, tw + (XI ? tw_off_xi(g) : 0), N1 - P1);
     load_twiddles(tw3, tw + g.N1 + g.N2, N3 - Q1);
     pdl_wait();
     const int t0 = threadIdx.x, nt = blockDim.x;
@@ -401,39 +411,103 @@ __device__ __forceinline__ void plane_inverse(float2* sm, const GridArgs& g, con
         }
     });
     __syncthreads();
-    // Z = A + i B on the full circle from the two half spectra
     constexpr int CR = CN3 > 0 ? CN3 / 2 : 0;
     const SmallDiv dr = small_div(nr);
-    for (int it = t0; it < Nh * nr; it += nt) {
-        const int k = cdiv<CR>(it, dr), row = it - k * nr;
-        int se, so;
-        half_slots(G, dP, N1, k, se, so);
-        float2* d = sm + row * S;
-        float2 a = d[se], b = d[so];
-        const bool edge = k == 0 || 2 * k == N1;
-        if (edge) a.y = b.y = 0.f;
-        d[se] = make_float2(a.x - b.y, a.y + b.x);
-        if (!edge) d[so] = make_float2(a.x + b.y, b.x - a.y);
+    const bool merged = XI && P1 <= MERGE_P<CN1>;
+    if (!merged) {
+        // Z = A + i B on the full circle from the two half spectra
+        for (int it = t0; it < Nh * nr; it += nt) {
+            const int k = cdiv<CR>(it, dr), row = it - k * nr;
+            int se, so;
+            half_slots(G, dP, N1, k, se, so);
+            float2* d = sm + row * S;
+            float2 a = d[se], b = d[so];
+            const bool edge = k == 0 || 2 * k == N1;
+            if (edge) a.y = b.y = 0.f;
+            d[se] = merge_pos(a, b);
+            if (!edge) d[so] = merge_neg(a, b);
+        }
+        __syncthreads();
     }
-    __syncthreads();
-    on_first<CN1, false>(g.p1, [&](auto tag) {
+    on_first<CN1, false, XI>(lx, [&](auto tag) {
         using R = decltype(tag);
-        const int m = CN1 > 0 ? CN1 / R::P : g.p1.P2;
-        for (int it = t0; it < m * nr; it += nt) {
-            const int j = cdiv<CR>(it, dr), row = it - j * nr;
-            float2* d = sm + row * S + j;
-            float2 v[R::P];
-#pragma unroll
-            for (int q = 0; q < R::P; ++q) v[q] = d[G.at(q)];
+        constexpr int P = R::P;
+        const int m = CN1 > 0 ? CN1 / P : lx.P2;
+        const auto run = [&](float2* d, float2 (&v)[P]) {
             group_fft<R, true, true, W>(v, (const W*)nullptr, 1);
 #pragma unroll
-            for (int i = 0; i < R::P; ++i) d[G.at(R::digit(i))] = v[i];
+            for (int i = 0; i < P; ++i) d[G.at(R::digit(i))] = v[i];
+        };
+        if constexpr (XI && P <= MERGE_P<CN1>) {
+            // j and m - j: element r of one is -(element P - 1 - r of the
+            // other); j = 0 and m/2 are their own partners
+            for (int it = t0; it < (m / 2 + 1) * nr; it += nt) {
+                const int j = cdiv<CR>(it, dr), row = it - j * nr;
+                float2* d = sm + row * S;
+                float2* da = d + j;
+                float2 a[P];
+#pragma unroll
+                for (int r = 0; r < P; ++r) a[r] = da[G.at(r)];
+                if (j == 0) {
+                    a[0].y = d[G.len].x;
+                    static_for<P / 2>([&](auto Q) {
+                        constexpr int r = decltype(Q)::value + 1, s = P - r;
+                        if constexpr (r == s) {
+                            a[r].y = d[G.len + 1].x;
+                        } else {
+                            const float2 x = a[r], y = a[s];
+                            a[r] = merge_pos(x, y);
+                            a[s] = merge_neg(x, y);
+                        }
+                    });
+                    run(da, a);
+                } else if (2 * j == m) {
+                    static_for<(P + 1) / 2>([&](auto Q) {
+                        constexpr int r = decltype(Q)::value, s = P - 1 - r;
+                        if constexpr (r == s) {
+                            a[r].y = d[G.len + 1].x;
+                        } else {
+                            const float2 x = a[r], y = a[s];
+                            a[r] = merge_pos(x, y);
+                            a[s] = merge_neg(x, y);
+                        }
+                    });
+                    run(da, a);
+                } else {
+                    float2* db = d + (m - j);
+                    float2 b[P];
+#pragma unroll
+                    for (int r = 0; r < P; ++r) b[r] = db[G.at(r)];
+                    static_for<P>([&](auto Q) {
+                        constexpr int r = decltype(Q)::value, s = P - 1 - r;
+                        const float2 x = a[r], y = b[s];
+                        if constexpr (r <= s) {  // k = j + r m below N1/2
+                            a[r] = merge_pos(x, y);
+                            b[s] = merge_neg(x, y);
+                        } else {
+                            b[s] = merge_pos(y, x);
+                            a[r] = merge_neg(y, x);
+                        }
+                    });
+                    run(da, a);
+                    run(db, b);
+                }
+            }
+        } else {
+            for (int it = t0; it < m * nr; it += nt) {
+                const int j = cdiv<CR>(it, dr), row = it - j * nr;
+                float2* d = sm + row * S + j;
+                float2 v[P];
+#pragma unroll
+                for (int r = 0; r < P; ++r) v[r] = d[G.at(r)];
+                run(d, v);
+            }
         }
     });
     __syncthreads();
     const SmallDiv dk = small_div(P1);
-    constexpr int CK = CN1 > 0 ? CtLine<CN1>::G1::P : 0;
-    on_second<CN1>(g.p1, [&](auto tag) {
+    constexpr int CK = CN1 > 0 ? CtLine<CN1, XI>::G1::P : 0;
+    on_second<CN1, XI>(lx, [&](auto tag) {
         using R = decltype(tag);
         for (int it = t0; it < P1 * nr; it += nt) {
             const int row = cdiv<CK>(it, dk), k1 = it - row * P1;
