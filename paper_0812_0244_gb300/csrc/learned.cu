@@ -1001,7 +1001,8 @@ __global__ void __launch_bounds__(L_THREADS, 1) k_learned_channels(const float* 
 // against the columns dz2, h2 and dz1 (tensor memory: 256 columns per team,
 // scratch and one block of 64 per factor).  Each row of H is wanted with one
 // of the three factors only, so a thread adds 32 columns of its row to FP32
-// registers after every tile: the tensor cores' accumulation does not round
+// registers after every tile (dz1's columns hold silu'(z1) until its sum is
+// due): the tensor cores' accumulation does not round
 // to nearest, and summed over all tiles there it left 1e-5 of relative error
 // against 64 bits (the smallest terms go first for the same reason).
 // Bound by the CUDA-core work per point (about 5 k instructions: SiLU and its
@@ -1026,24 +1027,32 @@ struct __align__(128) PgShared {
     uint16_t w2f[LRN_H * LRN_H];  // [out][in]
     uint16_t w2t[LRN_H * LRN_H];  // [in][out]
     float w3[LRN_M * LRN_H];
-    float w1[2 * LRN_H], b1[LRN_H], b2[LRN_H], b3[LRN_M];
+    float4 l1[LRN_H];             // {W1[j][0], W1[j][1], b1[j], b2[j]}
+    float b3[LRN_M];
 };
 
-// v as three bf16 terms: a + b + c = v
+// v as three bf16 terms, a + b + c = v: the leading 8 significant bits, the
+// leading 8 of what is left (both differences are exact), and the rest, at
+// most 8 bits
 __device__ __forceinline__ void split3(float v, float& a, float& b, float& c) {
-    a = bf16r(v);
+    a = __uint_as_float(__float_as_uint(v) & 0xffff0000u);
     const float r = v - a;
-    b = bf16r(r);
+    b = __uint_as_float(__float_as_uint(r) & 0xffff0000u);
     c = r - b;
+}
+// 8 bf16 values held as FP32 to one 16-byte core-matrix row
+__device__ __forceinline__ void store8_exact(uint16_t* dst, const float* v) {
+    const auto pack = [&](int i) { return __byte_perm(__float_as_uint(v[i]), __float_as_uint(v[i + 1]), 0x7632); };
+    *reinterpret_cast<uint4*>(dst) = make_uint4(pack(0), pack(2), pack(4), pack(6));
 }
 // 8 values in three terms to one 16-byte chunk of each of three tiles
 __device__ __forceinline__ void store8_split(uint16_t* d0, uint16_t* d1, uint16_t* d2, const float* v) {
     float a[8], b[8], c[8];
 #pragma unroll
     for (int i = 0; i < 8; ++i) split3(v[i], a[i], b[i], c[i]);
-    store8_bf16(d0, a);
-    store8_bf16(d1, b);
-    store8_bf16(d2, c);
+    store8_exact(d0, a);
+    store8_exact(d1, b);
+    store8_exact(d2, c);
 }
 
 __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
@@ -1061,11 +1070,8 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
         S->w2t[tc::kmaj(k, o, LRN_H)] = w;
     }
     for (int i = threadIdx.x; i < LRN_M * LRN_H; i += PG_THREADS) S->w3[i] = la.w3r[i];
-    for (int i = threadIdx.x; i < 2 * LRN_H; i += PG_THREADS) S->w1[i] = la.w1[i];
-    for (int i = threadIdx.x; i < LRN_H; i += PG_THREADS) {
-        S->b1[i] = la.b1[i];
-        S->b2[i] = la.b2[i];
-    }
+    for (int i = threadIdx.x; i < LRN_H; i += PG_THREADS)
+        S->l1[i] = make_float4(la.w1[2 * i], la.w1[2 * i + 1], la.b1[i], la.b2[i]);
     if (threadIdx.x < LRN_M) S->b3[threadIdx.x] = la.b3[threadIdx.x];
     // the unused columns of H stay zero
     for (int i = t; i < PG_TILE * 4; i += PG_TEAM)
@@ -1165,21 +1171,23 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
         }
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            float h[8];
+            float h[8], s1[8];
 #pragma unroll
             for (int q = 0; q < 8; ++q) {
-                const int j = 32 * hf + 8 * c + q;
-                h[q] = silu(fmaf(S->w1[2 * j], x1, fmaf(S->w1[2 * j + 1], x2, S->b1[j])));
+                const float4 w = S->l1[32 * hf + 8 * c + q];
+                silu_both(fmaf(w.x, x1, fmaf(w.y, x2, w.z)), h[q], s1[q]);
             }
             store8_bf16(T->H + tc::kmaj(p, 32 * hf + 8 * c, PG_HK), h);
+            tc::tmem_st8(lane + 192 + 32 * hf + 8 * c, s1);
         }
+        tc::tmem_st_wait();
         if (hf == 0) {
             float x[8];
             split3(x1, x[0], x[1], x[2]);
             split3(x2, x[3], x[4], x[5]);
             x[6] = 1.f;
             x[7] = 1.f;
-            store8_bf16(T->H + tc::kmaj(p, PG_X, PG_HK), x);
+            store8_exact(T->H + tc::kmaj(p, PG_X, PG_HK), x);
         }
         issue([&]() {
             for (int k = 0; k < LRN_H / 16; ++k)
@@ -1197,7 +1205,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
             float v[16];
             tc::tmem_ld16(lane + 32 * hf + 16 * c, v);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) silu_both(v[q] + S->b2[32 * hf + 16 * c + q], v[q], sp[16 * c + q]);
+            for (int q = 0; q < 16; ++q) silu_both(v[q] + S->l1[32 * hf + 16 * c + q].w, v[q], sp[16 * c + q]);
             store8_bf16(T->H2 + tc::kmaj(p, 32 * hf + 16 * c, LRN_H), v);
             store8_bf16(T->H2 + tc::kmaj(p, 32 * hf + 16 * c + 8, LRN_H), v + 8);
             if (mode == 1) {
@@ -1270,13 +1278,11 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
         // dz1 = dh1 silu'(z1)
 #pragma unroll
         for (int c = 0; c < 2; ++c) {
-            float v[16];
+            float v[16], s1[16];
             tc::tmem_ld16(lane + 32 * hf + 16 * c, v);
+            tc::tmem_ld16(lane + 192 + 32 * hf + 16 * c, s1);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) {
-                const int j = 32 * hf + 16 * c + q;
-                v[q] *= silu_prime(fmaf(S->w1[2 * j], x1, fmaf(S->w1[2 * j + 1], x2, S->b1[j])));
-            }
+            for (int q = 0; q < 16; ++q) v[q] *= s1[q];
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int at = tc::kmaj(p, 32 * hf + 16 * c + 8 * h, LRN_H);

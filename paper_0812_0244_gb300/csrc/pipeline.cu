@@ -111,7 +111,7 @@ __global__ void __launch_bounds__(256, POINT_BLOCKS) k_pointwise(const float* __
             const long long i = i0 + s * zs;
             const float ni = n[i];
             bad += (!(ni >= 0.f) || !isfinite(ni)) ? 1u : 0u;
-            const QPoint qp = q_point(ni, grad[i], grad[N + i], grad[2 * N + i], P, sp.qm);
+            const QPoint qp = q_point<NQ>(ni, grad[i], grad[N + i], grad[2 * N + i], P, sp.qm);
             t_out[i] = qp.t;
             k_out[i] = (uint8_t)qp.k;
             const bool ok = qp.k != K_INVALID;

@@ -40,7 +40,10 @@ __device__ __forceinline__ void saturation_sum_n(float y, int mc, const float* i
 }
 
 // qm: the q mesh (Nq values), normally a shared-memory copy of P.qm so that
-// the divergent interval search does not serialise on the constant bank.
+// the lanes' own intervals do not serialise on the constant bank.  NQ > 0: the
+// mesh size at compile time; the interval is then the number of inner knots
+// at or below q, counted against the constant bank without a branch.
+template <int NQ = 0>
 __device__ __forceinline__ QPoint q_point(float n, float gx, float gy, float gz, const PointParams& P,
                                           const float* qm) {
     QPoint r;
@@ -91,10 +94,16 @@ __device__ __forceinline__ QPoint q_point(float n, float gx, float gy, float gz,
     if (h < qm[0]) hp = 0.f;
     float q = fminf(fmaxf(h, qm[0]), qm[P.Nq - 1]);
     // interval: number of knots <= q, minus one, in [0, Nq-2]
-    int lo = 0, hi = P.Nq - 1;  // invariant: qm[lo] <= q (or lo = 0), answer in [lo, hi)
-    while (hi - lo > 1) {
-        const int mid = (lo + hi) >> 1;
-        if (qm[mid] <= q) lo = mid; else hi = mid;
+    int lo = 0;
+    if constexpr (NQ > 0) {
+#pragma unroll
+        for (int i = 1; i < NQ - 1; ++i) lo += P.qm[i] <= q ? 1 : 0;
+    } else {
+        int hi = P.Nq - 1;  // invariant: qm[lo] <= q (or lo = 0), answer in [lo, hi)
+        while (hi - lo > 1) {
+            const int mid = (lo + hi) >> 1;
+            if (qm[mid] <= q) lo = mid; else hi = mid;
+        }
     }
     r.k = lo;
     r.t = (q - qm[lo]) / (qm[lo + 1] - qm[lo]);
