@@ -367,13 +367,12 @@ int vdw_basis_weights(vdw_handle h, const float* n, const float* grad, float* p_
 int vdw_adam_step(float* p, const double* g, float* m, float* v, long long count, double lr, double beta1,
                   double beta2, double eps, int step, void* stream);
 
-/* *gave_up = 1 if, since vdw_plan, a bounded wait inside a kernel (an
- * asynchronous copy or a tensor-core completion) ran out, else 0.  Every such
+/* *gave_up = 1 if, since vdw_plan, a bounded wait inside a kernel (for a
+ * tensor-core completion in the learned path) ran out, else 0.  Every such
  * wait polls a bounded number of times instead of spinning forever; a kernel
  * whose wait gives up waits once more (bounded) for the operation in flight,
- * then stops without using its data (a plane transform leaves its plane
- * as it was, a network warpgroup skips its remaining tiles), so that call's
- * results are wrong.  The flag lives in page-locked host memory: the next call
+ * then stops without using its data (a network warpgroup skips its
+ * remaining tiles), so that call's results are wrong.  The flag lives in page-locked host memory: the next call
  * of vdw_energy_potential, vdw_energy_potential_fd, vdw_xc_energy_potential,
  * vdw_energy_potential_host, vdw_learned_energy_potential or
  * vdw_learned_param_grad on the context returns VDW_ERR_TIMEOUT without

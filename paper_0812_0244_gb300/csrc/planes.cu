@@ -21,10 +21,10 @@ namespace vdw {
 // real/half-spectrum step touch shared memory (the form before staged the
 // plane by a bulk copy and made every radix pass, 3 or 4 per line at a
 // run-time length, a load and a store).  us per launch, 20 fields, before and
-// after, forward / inverse: 180 x 180 x 72 156 / 154 -> 108 / 117; 256 x 256 x
-// 96 358 / 323 -> 285 / 281; run-time lengths, 144 x 144 x 72 (per density)
-// 304 / 288 -> 72 / 62, 200 x 200 x 72 545 / 506 -> 158 / 159, 128^3 303 /
-// 266 -> 116 / 113, 100^3 174 / 171 -> 64 / 65.
+// after, forward / inverse: 180 x 180 x 72 156 / 154 -> 96 / 94; 256 x 256 x
+// 96 358 / 323 -> 274 / 274; run-time lengths, 144 x 144 x 72 (per density)
+// 304 / 288 -> 70 / 64, 200 x 200 x 72 545 / 506 -> 164 / 142, 128^3 303 /
+// 266 -> 102 / 98, 100^3 174 / 171 -> 56 / 55.
 template <int CN1, int CN3, bool INV>
 __global__ void __launch_bounds__(PLANE_THREADS, 2)
     k_planes_inplace(float2* __restrict__ spec, GridArgs g, const Tw* __restrict__ tw, int ahead) {
