@@ -238,7 +238,10 @@ __device__ __forceinline__ void store_record(float4* p, const float2* v, float s
                  : "memory");
 }
 
-// u += Phi(t) theta with the row's pair coefficients cf
+// u += Phi(t) theta with the row's pair coefficients cf; the real and the
+// imaginary part by one packed instruction (the loop is bound by issue: 112 ->
+// 104 us at 180 x 180 x 72, 268 -> 250 at 256 x 256 x 96, the same bits; phi of
+// two pairs at a time packed as well took 136)
 template <int NQ>
 __device__ __forceinline__ void pair_loop(const float4* cf, float t, const float2 (&th)[NQ], float2 (&u)[NQ]) {
     int p = 0;
@@ -248,12 +251,9 @@ __device__ __forceinline__ void pair_loop(const float4* cf, float t, const float
         for (int b = a; b < NQ; ++b, ++p) {
             const float4 c = cf[p];
             const float phi = fmaf(t, fmaf(t, fmaf(t, c.w, c.z), c.y), c.x);
-            u[a].x = fmaf(phi, th[b].x, u[a].x);
-            u[a].y = fmaf(phi, th[b].y, u[a].y);
-            if (b != a) {
-                u[b].x = fmaf(phi, th[a].x, u[b].x);
-                u[b].y = fmaf(phi, th[a].y, u[b].y);
-            }
+            const float2 pp = make_float2(phi, phi);
+            u[a] = __ffma2_rn(pp, th[b], u[a]);
+            if (b != a) u[b] = __ffma2_rn(pp, th[a], u[b]);
         }
     }
 }
