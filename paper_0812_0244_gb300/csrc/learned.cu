@@ -1011,9 +1011,10 @@ __global__ void __launch_bounds__(L_THREADS, 1) k_learned_channels(const float* 
 // to nearest, and summed over all tiles there it left 1e-5 of relative error
 // against 64 bits (the smallest terms go first for the same reason).
 // Bound by the CUDA-core work per point (about 5 k instructions: SiLU and its
-// derivative for 64 + 64 units, the splits, dh2 = W3^T dout).
+// derivative for 64 + 64 units, the splits, dh2 = W3^T dout; two units per
+// packed instruction where there is one: 735 -> 686 us).
 // 180 x 180 x 72: 6828 us with one thread per point on the CUDA cores (each
-// product a shared-memory read and an FMA) -> 812 us; error against 64 bits,
+// product a shared-memory read and an FMA) -> 686 us; error against 64 bits,
 // norms of the blocks: 2e-7 to 2e-5 before, 6e-8 to 2e-5 now (the larger ones
 // are activations that round to bf16 the other way).
 constexpr int PG_TILE = 128;
@@ -1032,7 +1033,7 @@ struct __align__(128) PgShared {
     uint16_t w2f[LRN_H * LRN_H];  // [out][in]
     uint16_t w2t[LRN_H * LRN_H];  // [in][out]
     float w3[LRN_M * LRN_H];
-    float4 l1[LRN_H];             // {W1[j][0], W1[j][1], b1[j], b2[j]}
+    float4 l1[LRN_H];             // per two units j, j': {W1[j][0], W1[j'][0], W1[j][1], W1[j'][1]}, {b1, b1', b2, b2'}
     float b3[LRN_M];
 };
 
@@ -1045,6 +1046,18 @@ __device__ __forceinline__ void split3(float v, float& a, float& b, float& c) {
     b = __uint_as_float(__float_as_uint(r) & 0xffff0000u);
     c = r - b;
 }
+__device__ __forceinline__ float2 twice(float x) { return make_float2(x, x); }
+__device__ __forceinline__ float2 head(float2 v) {
+    return make_float2(__uint_as_float(__float_as_uint(v.x) & 0xffff0000u),
+                       __uint_as_float(__float_as_uint(v.y) & 0xffff0000u));
+}
+// silu_both of two units, their products by packed instructions
+__device__ __forceinline__ void silu_both2(float2 z, float2& f, float2& fp) {
+    const float2 d = __fadd2_rn(make_float2(__expf(fminf(-z.x, 80.f)), __expf(fminf(-z.y, 80.f))), twice(1.f));
+    const float2 s = make_float2(__fdividef(1.f, d.x), __fdividef(1.f, d.y));
+    f = __fmul2_rn(z, s);
+    fp = __fmul2_rn(s, __ffma2_rn(z, __ffma2_rn(s, twice(-1.f), twice(1.f)), twice(1.f)));
+}
 // 8 bf16 values held as FP32 to one 16-byte core-matrix row
 __device__ __forceinline__ void store8_exact(uint16_t* dst, const float* v) {
     const auto pack = [&](int i) { return __byte_perm(__float_as_uint(v[i]), __float_as_uint(v[i + 1]), 0x7632); };
@@ -1054,7 +1067,16 @@ __device__ __forceinline__ void store8_exact(uint16_t* dst, const float* v) {
 __device__ __forceinline__ void store8_split(uint16_t* d0, uint16_t* d1, uint16_t* d2, const float* v) {
     float a[8], b[8], c[8];
 #pragma unroll
-    for (int i = 0; i < 8; ++i) split3(v[i], a[i], b[i], c[i]);
+    for (int i = 0; i < 8; i += 2) {
+        const float2 w = make_float2(v[i], v[i + 1]), h = head(w);
+        const float2 r = __ffma2_rn(h, twice(-1.f), w), m = head(r), e = __ffma2_rn(m, twice(-1.f), r);
+        a[i] = h.x;
+        a[i + 1] = h.y;
+        b[i] = m.x;
+        b[i + 1] = m.y;
+        c[i] = e.x;
+        c[i + 1] = e.y;
+    }
     store8_exact(d0, a);
     store8_exact(d1, b);
     store8_exact(d2, c);
@@ -1075,8 +1097,10 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
         S->w2t[tc::kmaj(k, o, LRN_H)] = w;
     }
     for (int i = threadIdx.x; i < LRN_M * LRN_H; i += PG_THREADS) S->w3[i] = la.w3r[i];
-    for (int i = threadIdx.x; i < LRN_H; i += PG_THREADS)
-        S->l1[i] = make_float4(la.w1[2 * i], la.w1[2 * i + 1], la.b1[i], la.b2[i]);
+    for (int i = 2 * threadIdx.x; i < LRN_H; i += 2 * PG_THREADS) {
+        S->l1[i] = make_float4(la.w1[2 * i], la.w1[2 * i + 2], la.w1[2 * i + 1], la.w1[2 * i + 3]);
+        S->l1[i + 1] = make_float4(la.b1[i], la.b1[i + 1], la.b2[i], la.b2[i + 1]);
+    }
     if (threadIdx.x < LRN_M) S->b3[threadIdx.x] = la.b3[threadIdx.x];
     // the unused columns of H stay zero
     for (int i = t; i < PG_TILE * 4; i += PG_TEAM)
@@ -1178,9 +1202,16 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
         for (int c = 0; c < 4; ++c) {
             float h[8], s1[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const float4 w = S->l1[32 * hf + 8 * c + q];
-                silu_both(fmaf(w.x, x1, fmaf(w.y, x2, w.z)), h[q], s1[q]);
+            for (int q = 0; q < 8; q += 2) {
+                const float4 w = S->l1[32 * hf + 8 * c + q], b = S->l1[32 * hf + 8 * c + q + 1];
+                const float2 z = __ffma2_rn(make_float2(w.x, w.y), twice(x1),
+                                            __ffma2_rn(make_float2(w.z, w.w), twice(x2), make_float2(b.x, b.y)));
+                float2 f2, fp;
+                silu_both2(z, f2, fp);
+                h[q] = f2.x;
+                h[q + 1] = f2.y;
+                s1[q] = fp.x;
+                s1[q + 1] = fp.y;
             }
             store8_bf16(T->H + tc::kmaj(p, 32 * hf + 8 * c, PG_HK), h);
             tc::tmem_st8(lane + 192 + 32 * hf + 8 * c, s1);
@@ -1210,7 +1241,15 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
             float v[16];
             tc::tmem_ld16(lane + 32 * hf + 16 * c, v);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) silu_both(v[q] + S->l1[32 * hf + 16 * c + q].w, v[q], sp[16 * c + q]);
+            for (int q = 0; q < 16; q += 2) {
+                const float4 b = S->l1[32 * hf + 16 * c + q + 1];
+                float2 f2, fp;
+                silu_both2(__fadd2_rn(make_float2(v[q], v[q + 1]), make_float2(b.z, b.w)), f2, fp);
+                v[q] = f2.x;
+                v[q + 1] = f2.y;
+                sp[16 * c + q] = fp.x;
+                sp[16 * c + q + 1] = fp.y;
+            }
             store8_bf16(T->H2 + tc::kmaj(p, 32 * hf + 16 * c, LRN_H), v);
             store8_bf16(T->H2 + tc::kmaj(p, 32 * hf + 16 * c + 8, LRN_H), v + 8);
             if (mode == 1) {
@@ -1249,24 +1288,25 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
         // dz2 = (W3^T dout) silu'(z2)
 #pragma unroll
         for (int c = 0; c < 4; ++c) {
-            float d[8];
+            float2 e[4];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) d[q] = 0.f;
+            for (int q = 0; q < 4; ++q) e[q] = twice(0.f);
 #pragma unroll
             for (int m = 0; m < LRN_M; ++m) {
                 const float4* w = reinterpret_cast<const float4*>(S->w3 + m * LRN_H + 32 * hf + 8 * c);
                 const float4 w0 = w[0], w1 = w[1];
-                d[0] = fmaf(w0.x, dout[m], d[0]);
-                d[1] = fmaf(w0.y, dout[m], d[1]);
-                d[2] = fmaf(w0.z, dout[m], d[2]);
-                d[3] = fmaf(w0.w, dout[m], d[3]);
-                d[4] = fmaf(w1.x, dout[m], d[4]);
-                d[5] = fmaf(w1.y, dout[m], d[5]);
-                d[6] = fmaf(w1.z, dout[m], d[6]);
-                d[7] = fmaf(w1.w, dout[m], d[7]);
+                e[0] = __ffma2_rn(make_float2(w0.x, w0.y), twice(dout[m]), e[0]);
+                e[1] = __ffma2_rn(make_float2(w0.z, w0.w), twice(dout[m]), e[1]);
+                e[2] = __ffma2_rn(make_float2(w1.x, w1.y), twice(dout[m]), e[2]);
+                e[3] = __ffma2_rn(make_float2(w1.z, w1.w), twice(dout[m]), e[3]);
             }
+            float d[8];
 #pragma unroll
-            for (int q = 0; q < 8; ++q) d[q] *= sp[8 * c + q];
+            for (int q = 0; q < 4; ++q) {
+                const float2 x = __fmul2_rn(e[q], make_float2(sp[8 * c + 2 * q], sp[8 * c + 2 * q + 1]));
+                d[2 * q] = x.x;
+                d[2 * q + 1] = x.y;
+            }
             const int at = tc::kmaj(p, 32 * hf + 8 * c, LRN_H);
             store8_split(T->D[0] + at, T->D[1] + at, T->D[2] + at, d);
         }
@@ -1287,7 +1327,11 @@ __global__ void __launch_bounds__(PG_THREADS, 1) k_learned_param_grad(
             tc::tmem_ld16(lane + 32 * hf + 16 * c, v);
             tc::tmem_ld16(lane + 192 + 32 * hf + 16 * c, s1);
 #pragma unroll
-            for (int q = 0; q < 16; ++q) v[q] *= s1[q];
+            for (int q = 0; q < 16; q += 2) {
+                const float2 x = __fmul2_rn(make_float2(v[q], v[q + 1]), make_float2(s1[q], s1[q + 1]));
+                v[q] = x.x;
+                v[q + 1] = x.y;
+            }
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
                 const int at = tc::kmaj(p, 32 * hf + 16 * c + 8 * h, LRN_H);
