@@ -20,6 +20,13 @@ import torch
 from .vdwnl import VdwNL
 
 
+def _has_memory(t):
+    try:
+        return t.data_ptr() != 0
+    except RuntimeError:
+        return False
+
+
 class VdwEnergy(torch.autograd.Function):
     @staticmethod
     def forward(ctx, n, grad, handle: VdwNL):
@@ -33,7 +40,9 @@ class VdwEnergy(torch.autograd.Function):
     def backward(ctx, gE):
         n, grad = ctx.saved_tensors
         h = ctx.handle
-        if torch.is_grad_enabled():  # create_graph: the scaling by gE stays a torch operation
+        # create_graph, or a gE without memory of its own (under vmap, as with
+        # is_grads_batched): the scaling by gE stays a torch operation
+        if torch.is_grad_enabled() or not _has_memory(gE):
             v = torch.empty_like(n, dtype=torch.float32).contiguous()
             w = torch.empty_like(grad, dtype=torch.float32).contiguous()
             h.energy_potential(n.contiguous(), grad.contiguous(), None, v, w)
