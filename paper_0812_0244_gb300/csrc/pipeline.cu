@@ -705,8 +705,10 @@ int plane_block(const vdw_ctx* c, long long nblocks, bool inverse, bool exact) {
     // some for L1, through which the planes are loaded (w planes of 180 x 180
     // x 72: 29 us with three blocks of 288 threads, 37 with four of 256)
     const long long fit = std::max(1LL, std::min(228 * 1024 / smem, std::max(3LL, 192 * 1024 / smem)));
-    const long long per_sm = std::max(1LL, std::min(fit, (nblocks + nsm - 1) / nsm));
     const int most = PLANE_THREADS;
+    // small planes, many of them: a block keeps at least one warp (32 densities
+    // of 24^3 213 us; two warps 229, four 240)
+    const long long per_sm = std::clamp<long long>(std::min(fit, (nblocks + nsm - 1) / nsm), 1, 2 * most / 32);
     const bool fused = !inverse && exact && on_grid(g, [&](auto d) { return g.p1.P2 <= FUSE_P<decltype(d)::N1, Tw>; });
     const int items = std::max({nr * g.p1.P2, nr * g.p1.P1, g.Nh * g.p3.P2, g.Nh * g.p3.P1});
     const int hi = std::min((int)std::min<long long>(most, 2 * most / per_sm) / 32 * 32, (items + 31) / 32 * 32);
