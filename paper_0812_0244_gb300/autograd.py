@@ -16,15 +16,21 @@ operator, autograd reproduces v_nl of Eq. (Vi) for that operator.
 from __future__ import annotations
 
 import torch
+from torch.autograd import forward_ad
 
 from .vdwnl import VdwNL
 
 
-def _has_memory(t):
+def _memory_is_value(t):
+    """Whether the bytes at t's address are all there is to t: not so for a
+    batched tensor (vmap) and a zero tensor, which have no memory, for a lazily
+    negated one and for a dual one, whose tangent is held elsewhere."""
     try:
-        return t.data_ptr() != 0
+        if t.data_ptr() == 0:
+            return False
     except RuntimeError:
         return False
+    return not t.is_neg() and forward_ad.unpack_dual(t).tangent is None
 
 
 class VdwEnergy(torch.autograd.Function):
@@ -40,9 +46,10 @@ class VdwEnergy(torch.autograd.Function):
     def backward(ctx, gE):
         n, grad = ctx.saved_tensors
         h = ctx.handle
-        # create_graph, or a gE without memory of its own (under vmap, as with
-        # is_grads_batched): the scaling by gE stays a torch operation
-        if torch.is_grad_enabled() or not _has_memory(gE):
+        # create_graph, or a gE that the library cannot read by its address
+        # (is_grads_batched, a negative bit, a tangent): the scaling by gE stays
+        # a torch operation
+        if torch.is_grad_enabled() or not _memory_is_value(gE):
             v = torch.empty_like(n, dtype=torch.float32).contiguous()
             w = torch.empty_like(grad, dtype=torch.float32).contiguous()
             h.energy_potential(n.contiguous(), grad.contiguous(), None, v, w)
