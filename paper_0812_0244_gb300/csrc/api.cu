@@ -159,6 +159,8 @@ int alloc_density_work(vdw_ctx* c, int Bmax) {
     c->d_ecount = nullptr;
     VDW_CUDA(cudaMalloc(&c->d_ecount, sizeof(unsigned) * B));
     VDW_CUDA(cudaMemset(c->d_ecount, 0, sizeof(unsigned) * B));
+    // the first call may come on a stream that does not wait for the default one
+    VDW_CUDA(cudaStreamSynchronize(nullptr));
     g.bs_spec = (long long)spec_n;
     g.bs_wspec = (long long)wspec_n;
     g.bs_Q = (long long)q_n;

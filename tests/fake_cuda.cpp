@@ -4,6 +4,7 @@
 //
 //   fake_cuda planes NQ   every call of planes that are small enough for many
 //                         to share an SM, up to 32 densities per call
+//   fake_cuda batch       a call on the caller's stream right after vdw_plan_batch
 //
 // Exits 1 with a line per fault.
 #include <cuda_runtime_api.h>
@@ -20,12 +21,14 @@
 static std::map<const void*, std::string> g_names;
 static std::string g_case;
 static int g_faults = 0, g_launches = 0;
+static bool g_pending = false;  // a memset was queued on the default stream and nothing waited for it
 
 static void fault(const std::string& what) {
     if (++g_faults <= 20) std::printf("%s: %s\n", g_case.c_str(), what.c_str());
 }
-static cudaError_t launched(const void* f, dim3 grid, dim3 block, size_t smem, cudaStream_t) {
+static cudaError_t launched(const void* f, dim3 grid, dim3 block, size_t smem, cudaStream_t s) {
     ++g_launches;
+    if (g_pending && s) fault(g_names[f] + " does not wait for a memset on the default stream");
     const unsigned t = block.x * block.y * block.z;
     if (t < 1 || t > 1024 || grid.x < 1 || grid.y < 1 || grid.z < 1 || grid.y > 65535 || grid.z > 65535 ||
         smem > 227 * 1024)
@@ -93,10 +96,22 @@ cudaError_t cudaMemcpy(void* d, const void* s, size_t n, cudaMemcpyKind) {
     return cudaSuccess;
 }
 cudaError_t cudaMemcpyAsync(void*, const void*, size_t, cudaMemcpyKind, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaMemset(void*, int, size_t) { return cudaSuccess; }
-cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t) { return cudaSuccess; }
-cudaError_t cudaDeviceSynchronize() { return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t) { return cudaSuccess; }
+cudaError_t cudaMemset(void*, int, size_t) {
+    g_pending = true;
+    return cudaSuccess;
+}
+cudaError_t cudaMemsetAsync(void*, int, size_t, cudaStream_t s) {
+    g_pending = g_pending || !s;
+    return cudaSuccess;
+}
+cudaError_t cudaDeviceSynchronize() {
+    g_pending = false;
+    return cudaSuccess;
+}
+cudaError_t cudaStreamSynchronize(cudaStream_t s) {
+    g_pending = g_pending && s;
+    return cudaSuccess;
+}
 cudaError_t cudaGetDevice(int* d) {
     *d = 0;
     return cudaSuccess;
@@ -188,9 +203,23 @@ static void planes(int Nq) {
     vdw_destroy(h);
 }
 
+static void batch() {
+    vdw_handle h = context(8);
+    const double L[3] = {6.0, 6.0, 6.0};
+    double E[1];
+    ok(vdw_plan(h, 12, 12, 12, L), "vdw_plan");
+    g_case = "after vdw_plan";
+    ok(vdw_energy_potential(h, g_buf, g_buf, E, g_buf, nullptr, STREAM), "vdw_energy_potential");
+    ok(vdw_plan_batch(h, 3), "vdw_plan_batch");
+    g_case = "after vdw_plan_batch";
+    ok(vdw_energy_potential_batched(h, 3, g_buf, g_buf, E, g_buf, STREAM), "batched");
+    vdw_destroy(h);
+}
+
 int main(int argc, char** argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "planes") planes(std::atoi(argv[2]));
+    else if (what == "batch") batch();
     else return 2;
     std::printf("%d launches, %d faults\n", g_launches, g_faults);
     return g_faults ? 1 : 0;

@@ -32,3 +32,8 @@ def run(exe, *args):
 def test_block_sizes_of_many_small_planes(fake, Nq):
     """More than 32 planes per SM still leave each block at least one warp."""
     run(fake, "planes", Nq)
+
+
+def test_batch_workspaces_are_cleared_before_vdw_plan_batch_returns(fake):
+    """The caller's stream need not wait for the default stream."""
+    run(fake, "batch")
