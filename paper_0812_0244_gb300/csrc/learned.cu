@@ -1828,7 +1828,7 @@ int vdw_learned_load(vdw_handle c, int J, double k_max, const double feat[5], do
         c->d_lrn = nullptr;
         const LrnLayout L = lrn_layout(g, J, c->nb_sorted);
         VDW_CUDA(cudaMalloc(&c->d_lrn, L.total));
-        VDW_CUDA(cudaMemset(c->d_lrn, 0, L.total));
+        VDW_CUDA(cudaMemsetAsync(c->d_lrn, 0, L.total, s));  // ahead of k_learned_prepare
         unsigned char* b = static_cast<unsigned char*>(c->d_lrn);
         LearnedArgs& la = c->la;
         la.w1 = reinterpret_cast<float*>(b + L.w1);

@@ -5,6 +5,7 @@
 //   fake_cuda planes NQ   every call of planes that are small enough for many
 //                         to share an SM, up to 32 densities per call
 //   fake_cuda batch       a call on the caller's stream right after vdw_plan_batch
+//   fake_cuda learned     the learned path's calls right after vdw_learned_load
 //
 // Exits 1 with a line per fault.
 #include <cuda_runtime_api.h>
@@ -216,10 +217,28 @@ static void batch() {
     vdw_destroy(h);
 }
 
+static void learned() {
+    vdw_handle h = context(8);
+    const double L[3] = {6.0, 6.0, 6.0}, feat[5] = {0.0, 1.0, 0.0, 1.0, 1e-3};
+    double E[1];
+    ok(vdw_plan(h, 12, 12, 12, L), "vdw_plan");
+    for (int J : {16, 16, 32}) {
+        g_case = "J " + std::to_string(J);
+        ok(vdw_learned_load(h, J, 40.0, feat, 0.1, 1.4, g_buf, STREAM), "vdw_learned_load");
+        ok(vdw_learned_param_grad(h, g_buf, g_buf, 1.0, E, E, STREAM), "vdw_learned_param_grad");
+        ok(vdw_learned_fit_grad(h, g_buf, g_buf, g_buf, g_buf, 1.0, E, STREAM), "vdw_learned_fit_grad");
+        ok(vdw_learned_energy_potential(h, g_buf, g_buf, E, g_buf, nullptr, STREAM), "vdw_learned_energy_potential");
+        ok(vdw_learned_tabulate(h, 16, 4.0, STREAM), "vdw_learned_tabulate");
+        ok(vdw_learned_energy_potential(h, g_buf, g_buf, E, g_buf, nullptr, STREAM), "vdw_learned_energy_potential");
+    }
+    vdw_destroy(h);
+}
+
 int main(int argc, char** argv) {
     const std::string what = argc > 1 ? argv[1] : "";
     if (what == "planes") planes(std::atoi(argv[2]));
     else if (what == "batch") batch();
+    else if (what == "learned") learned();
     else return 2;
     std::printf("%d launches, %d faults\n", g_launches, g_faults);
     return g_faults ? 1 : 0;

@@ -37,3 +37,7 @@ def test_block_sizes_of_many_small_planes(fake, Nq):
 def test_batch_workspaces_are_cleared_before_vdw_plan_batch_returns(fake):
     """The caller's stream need not wait for the default stream."""
     run(fake, "batch")
+
+
+def test_learned_parameters_are_laid_out_after_their_memory_is_cleared(fake):
+    run(fake, "learned")
