@@ -786,7 +786,7 @@ __global__ void __launch_bounds__(SORTED_BLOCK, 6) k_learned_contract_gradk(
     __shared__ float rv_s[SORTED_BLOCK * GK_LD];
     __shared__ float4 w_s[SORTED_BLOCK];
     __shared__ int j_s[SORTED_BLOCK];
-    __shared__ float part[GK_PARTS][LRN_P][4];
+    __shared__ float4 part[GK_PARTS][LRN_P];
     const int J = la.J, tid = threadIdx.x;
     const long long r = (long long)blockIdx.x * SORTED_BLOCK + tid;
     float2 th[NQ];
@@ -863,14 +863,14 @@ __global__ void __launch_bounds__(SORTED_BLOCK, 6) k_learned_contract_gradk(
                 s.z = fmaf(rv, w.z, s.z);
                 s.w = fmaf(rv, w.w, s.w);
             }
-            *reinterpret_cast<float4*>(part[pt][pair]) = s;
+            part[pt][pair] = s;
         }
         __syncthreads();
         for (int o = tid; o < 4 * LRN_P; o += SORTED_BLOCK) {
             const int pp = o >> 2, c = o & 3;
             double s = 0.0;
 #pragma unroll
-            for (int k = 0; k < GK_PARTS; ++k) s += (double)part[k][pp][c];
+            for (int k = 0; k < GK_PARTS; ++k) s += (double)(&part[k][pp].x)[c];
             // knots of the four weights: the knot before k = 0 mirrors knot 1;
             // past the last knot the linear extrapolation 2 K_{J-1} - K_{J-2}
             double* g = gK + pp * J;
