@@ -286,14 +286,9 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
     if (!rc) rc = make_line_plan(n2, sized, &g.p2);
     if (!rc) rc = make_line_plan(n3, sized, &g.p3);
     if (rc) return rc;
-    // The inverse x transforms merge the two half spectra in their first group
-    // when that has few points, so the smaller group goes first (us inverse
-    // planes: 180 106 -> 94, 128^3 104 -> 98, 100^3 65 -> 55); not where the
-    // rows then need a pad after every run (16 points) that they do not need now
-    // (144: 514 against 520).  The spectral gradient keeps the forward order.
+    // (the spectral gradient keeps the forward order)
     g.p1i = g.p1;
-    const bool few = g.p1.P2 > 1 && g.p1.P2 <= 9 && !(g.p1.P1 % 16 == 0 && g.p1.P2 % 2 == 1);
-    if (sized ? n1 == 180 : (g.p1.P1 > g.p1.P2 && few)) std::swap(g.p1i.P1, g.p1i.P2);
+    if (merge_swaps(g.p1.P1, g.p1.P2, sized ? MERGE_CT : MERGE_RT)) std::swap(g.p1i.P1, g.p1i.P2);
     rc = pipeline_plan_check(c);
     if (rc) {
         set_error("grid too large for on-chip staging");

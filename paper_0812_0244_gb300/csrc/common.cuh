@@ -353,6 +353,16 @@ void learned_free(vdw_ctx* c);
 int table_build(const vdw_params* p, double* h_qmesh, double* h_phik, double* phi0, double* C_s);
 int table_upload(vdw_ctx* c, const double* h_phik, double C_s);
 
+// The inverse x transforms merge the two half spectra of a row in their first
+// group's registers when it has at most this many points, with compile-time
+// and with run-time groups (above 9 points the run-time kernels spill), so the
+// smaller group goes first (us inverse planes: 180 x 180 x 72 106 -> 94, 128^3
+// 104 -> 98, 100^3 65 -> 55); not where the rows then need a pad after every
+// run (16 points) that they do not need otherwise (144: 514 against 520).
+constexpr int MERGE_CT = 12, MERGE_RT = 9;
+__host__ __device__ constexpr bool merge_swaps(int P1, int P2, int most) {
+    return P1 > P2 && P2 > 1 && P2 <= most && !(P1 % 16 == 0 && P2 % 2 == 1);
+}
 // Groups of a line length ({2,3,5}-smooth, 4 <= n <= 256); sized: the
 // compile-time schedule of the grids that have one.
 int make_line_plan(int n, bool sized, LinePlan* lp);

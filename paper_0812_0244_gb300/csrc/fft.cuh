@@ -32,6 +32,7 @@
 
 #include "common.cuh"
 
+#include <type_traits>
 #include <utility>
 
 namespace vdw {
@@ -431,13 +432,20 @@ __device__ __forceinline__ void group_fft(float2 (&v)[G::P], const W* tw, int Ns
 // in-register radices each.  Any other length takes its groups at run time
 // from the list 4, .., 4, 2, 3, .., 3, 5, .., 5 (make_line_plan).
 // CtLine<N, true>: the order of the inverse x transforms of u and D.w
-// (LinePlan p1i).
-template <int CN, bool XI = false> struct CtLine { using G1 = Grp<1>; using G2 = Grp<1>; };
-template <> struct CtLine<180, false> { using G1 = Grp<15>; using G2 = Grp<12>; };
-template <> struct CtLine<180, true> { using G1 = Grp<12>; using G2 = Grp<15>; };
-template <> struct CtLine<72, false> { using G1 = Grp<9>; using G2 = Grp<8>; };
-template <bool XI> struct CtLine<256, XI> { using G1 = Grp<16>; using G2 = Grp<16>; };
-template <> struct CtLine<96, false> { using G1 = Grp<12>; using G2 = Grp<8>; };
+// (LinePlan p1i, merge_swaps).
+template <int CN> struct CtGroups { using G1 = Grp<1>; using G2 = Grp<1>; };
+template <> struct CtGroups<180> { using G1 = Grp<15>; using G2 = Grp<12>; };
+template <> struct CtGroups<72> { using G1 = Grp<9>; using G2 = Grp<8>; };
+template <> struct CtGroups<256> { using G1 = Grp<16>; using G2 = Grp<16>; };
+template <> struct CtGroups<96> { using G1 = Grp<12>; using G2 = Grp<8>; };
+template <int CN, bool XI = false>
+struct CtLine {
+    using A = typename CtGroups<CN>::G1;
+    using B = typename CtGroups<CN>::G2;
+    static constexpr bool SWAP = XI && merge_swaps(A::P, B::P, MERGE_CT);
+    using G1 = std::conditional_t<SWAP, B, A>;
+    using G2 = std::conditional_t<SWAP, A, B>;
+};
 
 // Run-time lengths: any, or (ANY16) with no group above 16.  The second kind
 // leaves the larger groups' registers out of a kernel.

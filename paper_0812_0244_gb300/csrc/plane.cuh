@@ -185,7 +185,7 @@ __device__ __forceinline__ float2 split_odd(float2 f, float2 s) {
 // group of at most MERGE_P points does it in registers, for k and N1 - k in
 // one thread; otherwise it is a pass of its own.
 template <int CN1>
-constexpr int MERGE_P = CN1 == 180 ? 12 : CN1 > 0 ? 0 : 9;
+constexpr int MERGE_P = CN1 > 0 ? MERGE_CT : MERGE_RT;
 __device__ __forceinline__ float2 merge_pos(float2 a, float2 b) { return make_float2(a.x - b.y, a.y + b.x); }
 __device__ __forceinline__ float2 merge_neg(float2 a, float2 b) { return make_float2(a.x + b.y, b.x - a.y); }
 // position of (z, kx): even and odd real rows of a complex row at slots se, so
