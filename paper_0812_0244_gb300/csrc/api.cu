@@ -275,9 +275,6 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
     g.gx = (float)(2.0 * PI_D / L[0]);
     g.gy = (float)(2.0 * PI_D / L[1]);
     g.gz = (float)(2.0 * PI_D / L[2]);
-    g.gx2 = g.gx * g.gx;
-    g.gy2 = g.gy * g.gy;
-    g.gz2 = g.gz * g.gz;
     g.Nk = c->p.Nk;
     g.inv_dk = (float)((c->p.Nk - 1) / c->p.k_max);
     g.invN = (float)(1.0 / (double)g.N);
@@ -295,7 +292,6 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
         return rc;
     }
     const int Nq = c->p.Nq;
-    const size_t spec_n = (size_t)Nq * n2 * g.ncols;
     {
         // pointwise slabs: 4, 3, 2 or 1 equal slabs of the N3/2 complex rows
         const int nh3 = n3 / 2;
@@ -332,7 +328,6 @@ int vdw_plan(vdw_handle c, int n1, int n2, int n3, const double L[3]) {
     rc = pipeline_configure(c);
     if (rc) return rc;
     const int npairs = Nq * (Nq + 1) / 2;
-    (void)spec_n;
     c->bytes += sizeof(float4) * (size_t)(c->p.Nk - 1) * npairs + sizeof(float4) * (2 * n1 + 2 * n2 + n3);
     c->planned = 1;
     return VDW_OK;

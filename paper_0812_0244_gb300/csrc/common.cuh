@@ -59,19 +59,18 @@ struct GridArgs {
     int N1, N2, N3, Nh;    // Nh = N1/2 + 1
     long long N;           // N1 N2 N3
     int ncols;             // N3 * Nh: columns of the half spectrum per y
-    float gx2, gy2, gz2;   // (2 pi / L_d)^2
     float gx, gy, gz;      // 2 pi / L_d
+    // Flat-index divisions by N1, N2 and N3/2 as multiply-high by
+    // m = ceil(2^32 / d), exact for i d < 2^32; fast = 0 (plain division)
+    // when N max(N1, N2, N3) reaches 2^32 or a divisor is 1.
+    unsigned m1, m2, mh3;
     float inv_dk;          // 1 / Delta k of the radial table
     int Nk;                // points of the radial table
     float invN;            // 1 / N
     LinePlan p1, p2, p3;   // line transforms along x, y, z
     LinePlan p1i;          // inverse along x of u and D.w (its groups may be in the other order)
     int pad_fwd, pad_inv;  // plane transforms with padded rows (plane_geo)
-    // Flat-index divisions by N1, N2 and N3/2 as multiply-high by
-    // m = ceil(2^32 / d), exact for i d < 2^32; fast = 0 (plain division)
-    // when N max(N1, N2, N3) reaches 2^32 or a divisor is 1.
-    unsigned m1, m2, mh3;
-    int fast;
+    int fast;              // flat-index divisions by m1, m2, mh3
     // batches (vdw_energy_potential_batched): density b of a batch uses the
     // workspaces at these element offsets times b; the kernels take b from
     // their last grid dimension (0 for a single density)

@@ -41,7 +41,6 @@ namespace vdw {
 // by issue slots and shared memory; 1-5 % of the plane kernels' time)
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return __fadd2_rn(a, b); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return __fadd2_rn(a, make_float2(-b.x, -b.y)); }
-__device__ __forceinline__ float2 cscale(float2 a, float s) { return make_float2(a.x * s, a.y * s); }
 __device__ __forceinline__ float2 cmul(float2 a, float2 b) {
     return make_float2(fmaf(a.x, b.x, -a.y * b.y), fmaf(a.x, b.y, a.y * b.x));
 }
@@ -289,12 +288,8 @@ __device__ __forceinline__ void dft_pfa(float2* v) {
     }
 }
 
-template <> __device__ __forceinline__ void dft<6, false>(float2* v) { dft_pfa<2, 3, false>(v); }
-template <> __device__ __forceinline__ void dft<6, true>(float2* v) { dft_pfa<2, 3, true>(v); }
 template <> __device__ __forceinline__ void dft<9, false>(float2* v) { dft_ct<3, 3, false>(v); }
 template <> __device__ __forceinline__ void dft<9, true>(float2* v) { dft_ct<3, 3, true>(v); }
-template <> __device__ __forceinline__ void dft<10, false>(float2* v) { dft_pfa<2, 5, false>(v); }
-template <> __device__ __forceinline__ void dft<10, true>(float2* v) { dft_pfa<2, 5, true>(v); }
 template <> __device__ __forceinline__ void dft<12, false>(float2* v) { dft_pfa<4, 3, false>(v); }
 template <> __device__ __forceinline__ void dft<12, true>(float2* v) { dft_pfa<4, 3, true>(v); }
 template <> __device__ __forceinline__ void dft<15, false>(float2* v) { dft_pfa<5, 3, false>(v); }
@@ -371,7 +366,7 @@ struct Grp {
 };
 
 // The group's transform of v (input q in register q).  FIRST: Ns = 1,
-// constant twiddles.  Otherwise tw points at the group's table (tw_entries)
+// constant twiddles.  Otherwise tw points at the group's table (k_twiddles)
 // plus k: the twiddle of entry i is tw[i Ns].
 template <class G, bool INV, bool FIRST, class W>
 __device__ __forceinline__ void group_fft(float2 (&v)[G::P], const W* tw, int Ns) {

@@ -29,7 +29,6 @@
 #include "pointwise.cuh"
 #include "tc.cuh"
 
-#include <cooperative_groups.h>
 #include <cuda_bf16.h>
 
 #include <algorithm>
@@ -38,8 +37,6 @@
 
 namespace vdw {
 namespace {
-
-namespace cg = cooperative_groups;
 
 constexpr int L_SLOTS = 8;        // network partial-sum slots per y plane (epart scratch)
 constexpr int L_THREADS = 256;    // two warpgroups (channel kernel)

@@ -27,8 +27,6 @@
 #include "plane.cuh"
 #include "pointwise.cuh"
 
-#include <cooperative_groups.h>
-
 #include <algorithm>
 #include <initializer_list>
 #include <string>

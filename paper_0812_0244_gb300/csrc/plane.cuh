@@ -2,8 +2,6 @@
 // the forward / inverse transform of one y plane (N3 rows of N1 reals <->
 // N3 x Nh half spectrum) through shared memory.
 #pragma once
-#include <type_traits>
-
 #include "fft.cuh"
 
 namespace vdw {
@@ -197,9 +195,6 @@ template <class W = Tw>
 __device__ __forceinline__ W* twiddles_after(float2* base, size_t n) {
     return reinterpret_cast<W*>(base + tw_offset(n));
 }
-// The twiddle kind of a transform: hi/lo pairs (EXACT) or FP32 values.
-template <bool EXACT>
-using TwOf = typename std::conditional<EXACT, Tw, float2>::type;
 
 // Forward transform of one plane: complex rows from ld(row, x) (R2C along x
 // of the two real rows in each, C2C along z), results to st(kz, kx, value).

@@ -153,15 +153,7 @@ __device__ __forceinline__ void load_spline_pairs(float2* mp, const PointParams&
     }
 }
 
-// p_a and dp_a/dq on interval k at local position t.
-__device__ __forceinline__ void cardinal(const SplineSmem* sp, int a, int k, float t, float& pa, float& dpa) {
-    const float A = 1.f - t, B = t;
-    const float M0 = sp->Mq[a * MAX_NQ + k], M1 = sp->Mq[a * MAX_NQ + k + 1];
-    const float y0 = (a == k) ? 1.f : 0.f, y1 = (a == k + 1) ? 1.f : 0.f;
-    pa = A * y0 + B * y1 + ((A * A * A - A) * M0 + (B * B * B - B) * M1) * sp->h26[k];
-    dpa = (y1 - y0) * sp->ih[k] + ((3.f * B * B - 1.f) * M1 - (3.f * A * A - 1.f) * M0) * sp->h6[k];
-}
-
+// p_a on interval k at local position t.
 __device__ __forceinline__ float cardinal_value(const SplineSmem* sp, int a, int k, float t) {
     const float A = 1.f - t, B = t;
     const float M0 = sp->Mq[a * MAX_NQ + k], M1 = sp->Mq[a * MAX_NQ + k + 1];
