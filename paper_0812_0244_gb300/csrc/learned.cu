@@ -1011,9 +1011,19 @@ __global__ void __launch_bounds__(L_THREADS, 1) k_learned_channels(const float* 
 // derivative for 64 + 64 units, the splits, dh2 = W3^T dout; two units per
 // packed instruction where there is one: 735 -> 686 us).
 // 180 x 180 x 72: 6828 us with one thread per point on the CUDA cores (each
-// product a shared-memory read and an FMA) -> 686 us; error against 64 bits,
-// norms of the blocks: 2e-7 to 2e-5 before, 6e-8 to 2e-5 now (the larger ones
-// are activations that round to bf16 the other way).
+// product a shared-memory read and an FMA) -> 686 us.
+// Error against 64 bits, norm of each block W1 b1 W2 b2 W3 b3 over its norm,
+// trained model, the largest of three tube densities at 180 x 180 x 72, in
+// units of 1e-7, before and now:
+//   energy          30 33 33 32 38 38         3.2 3.2 2.9 2.1 3.7 0.2
+//   fit, smooth     121 99 135 193 215 253    2.0 2.3 1.8 2.2 3.9 0.3
+//   fit, noise      37 37 70 40 216 10        39 39 73 46 218 0.6
+// (with a target of noise most of a sum cancels, and activations that round to
+// bf16 the other way are what is left, in both forms).  The CUDA cores' error
+// grew with the points per thread; the truncation within a tile does not, and
+// on smaller grids than the models are trained on it is the larger of the two
+// (100^3, energy: 1.4 1.6 1.8 1.5 2.9 0.9 before, 2.6 1.6 2.1 1.2 3.0 0.6 now;
+// with perturbed weights 1.8 1.6 1.9 1.7 2.5 2.4 and 3.9 2.8 3.2 2.0 4.1 1.5).
 constexpr int PG_TILE = 128;
 constexpr int PG_TEAM = 256;
 constexpr int PG_THREADS = 2 * PG_TEAM;

@@ -51,10 +51,11 @@ constexpr int XC_BLOCKS = 1024;  // blocks (and partial-sum slots) of the semilo
 // that slab alone (grid nbs); with slab < 0 the grid holds nbs blocks for
 // every slab, block b doing block b mod nbs of slab b / nbs, so that both
 // forms give the same partial sums.  mnj = ceil(2^32 / nj) when g.fast.
-// Bound by issue slots (61 % of the cycles), not by HBM (a third of its
-// bandwidth).  40 registers, six blocks of 256 threads per SM: 100 us at 180 x
-// 180 x 72 against 112 at 64 registers and four blocks; with the two z of a
-// packed row to a thread (8-byte stores) and the interval counted, 82.
+// Bound by issue slots (64 % of the cycles), not by HBM (a third of its
+// bandwidth).  Four blocks of 256 threads per SM at 62 registers, the two z of
+// a packed row to a thread (8-byte stores), the interval counted: 80 us at 180
+// x 180 x 72.  One point per thread took 100 us at 40 registers and six blocks,
+// 112 at 64 registers and four.
 template <int NQ>
 __global__ void __launch_bounds__(256, POINT_BLOCKS) k_pointwise(const float* __restrict__ n, const float* __restrict__ grad,
                                                    GridArgs g, PointParams P, int slab, int nj, unsigned mnj,
